@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "dd_coef.cuh"
+#include "dd_dose_rows.cuh"
 #include "dd_e1.cuh"
 #include "dd_field_impl.cuh"
 #include "dd_internal.h"
@@ -523,6 +524,80 @@ dd_status run_dose(const dd_scan *scan, int64_t j0, int64_t j1, double *out, cud
     return DD_OK;
 }
 
+// Whether the targets [j0, j1) take the row-invariant path (dd_dose_rows.cuh): a raster or
+// serpentine scan of every grid position with a uniform dwell, when the path's pair terms
+// (2 nx per row up to the last target's on a raster, nx^2 on a serpentine) are no more than
+// the direct sum's (j per target).  64 x 64 and up: fewer by nx / 4 and more for a whole
+// scan; more than the direct sum's only for a few targets late in a scan.
+bool dose_rows_apply(const dd_scan *scan, int64_t j0, int64_t j1) {
+    if (!scan->uniform || (scan->order != DD_RASTER && scan->order != DD_SERPENTINE)) return false;
+    if (scan->n != (int64_t)scan->nx * scan->ny || j1 < 2) return false;
+    const double nx = (double)scan->nx, rows = (double)((j1 - 1) / scan->nx + 1);
+    const double terms = scan->order == DD_RASTER ? 2.0 * nx * rows : nx * nx * (rows - 0.5);
+    return terms <= 0.5 * ((double)j1 * (double)j1 - (double)j0 * (double)j0);
+}
+
+// Source visits per work item of the row-invariant path: whole rows when those already give
+// every SM four CTAs, else halved down to 8 (one pair term per warp of the CTA: an FP64 term's
+// chain is microseconds long) while the pieces' sums stay within 1 GiB.
+int64_t dose_rows_piece(int64_t nx, int64_t n_rows, size_t part_size) {
+    int64_t qc = nx;
+    auto pieces = [&](int64_t q) { return (nx + q - 1) / q; };
+    while (qc > ddk::kDoseRowsWarps && n_rows * ((nx + 31) / 32) * pieces(qc) < 4 * (int64_t)device_sms() &&
+           (size_t)(pieces((qc + 1) / 2) * n_rows * nx) * part_size <= (size_t(1) << 30))
+        qc = (qc + 1) / 2;
+    return qc;
+}
+
+template <typename Cfg>
+dd_status run_dose_rows(const dd_scan *scan, int64_t j0, int64_t j1, double *out, cudaStream_t stream) {
+    using Rec = typename Cfg::Rec;
+    using Part = typename Cfg::Real;
+    const bool raster = scan->order == DD_RASTER;
+    const int64_t nx = scan->nx, n_rows = (j1 - 1) / nx + 1, m = j1 - j0;
+    const int64_t n_mt = (nx + 31) / 32;
+    const int64_t qc = raster ? nx : dose_rows_piece(nx, n_rows, sizeof(Part));
+    const int64_t n_q = raster ? 2 : (nx + qc - 1) / qc;
+    const int64_t n_lag = raster ? 0 : n_rows * nx;
+    const dd::MemKind out_kind = dd::memory_kind(out);
+    const bool out_host = out_kind != dd::MemKind::Device;
+    const size_t b_rec = ((size_t)n_lag * sizeof(Rec) + 255) & ~size_t(255);
+    const size_t b_part = ((size_t)(n_rows * n_q * nx) * sizeof(Part) + 255) & ~size_t(255);
+    void *ws = nullptr;
+    cudaError_t err = dd::workspace_alloc(&ws, b_rec + b_part + (out_host ? (size_t)m * sizeof(double) : 0), stream);
+    if (err != cudaSuccess) {
+        cudaGetLastError();
+        return dd::fail(err == cudaErrorMemoryAllocation ? DD_ENOMEM : DD_ECUDA,
+                        std::string("dose workspace allocation: ") + cudaGetErrorString(err));
+    }
+    Rec *d_rec = static_cast<Rec *>(ws);
+    Part *d_part = reinterpret_cast<Part *>(static_cast<char *>(ws) + b_rec);
+    double *out_dev = out_host ? reinterpret_cast<double *>(static_cast<char *>(ws) + b_rec + b_part) : out;
+    if (raster) {
+        const int half = (int)std::min<int64_t>(ddk::kDoseRasterHalf, n_mt * 32);
+        DD_PROFILED(Cfg::kDoseName, stream,
+                    (ddk::dose_raster_kernel<Cfg><<<(unsigned)n_rows, 2 * half, 0, stream>>>((int)nx, scan->s, scan->kappa, d_part)));
+    } else {
+        DD_PROFILED(Cfg::kLagCoefName, stream,
+                    (ddk::lag_coef_kernel<Rec><<<(unsigned)((n_lag + 31) / 32), 32, 0, stream>>>(n_lag, scan->s, scan->kappa, d_rec)));
+        DD_CUDA_TRY(cudaGetLastError());
+        DD_PROFILED(Cfg::kDoseName, stream,
+                    (ddk::dose_rows_kernel<Cfg><<<(unsigned)(n_rows * n_q * n_mt), 32 * ddk::kDoseRowsWarps, 0, stream>>>(
+                        nx, n_mt, n_q, qc, d_rec, d_part)));
+    }
+    DD_CUDA_TRY(cudaGetLastError());
+    DD_PROFILED("dose_reduce", stream,
+                (ddk::dose_rows_scan_kernel<Part><<<(unsigned)((nx + ddk::kDoseScanCols - 1) / ddk::kDoseScanCols),
+                                                  ddk::kDoseScanCols * ddk::kDoseScanGroups, 0, stream>>>(
+                    d_part, nx, n_rows, n_q, j0, j1, scan->pref, out_dev)));
+    DD_CUDA_TRY(cudaGetLastError());
+    if (out_host)
+        DD_CUDA_TRY(cudaMemcpyAsync(out, out_dev, (size_t)m * sizeof(double), cudaMemcpyDeviceToHost, stream));
+    DD_CUDA_TRY(dd::workspace_release(ws, stream));
+    if (dd::host_sync_needed(stream, {out_kind})) DD_CUDA_TRY(cudaStreamSynchronize(stream));
+    return DD_OK;
+}
+
 template <typename Cfg>
 dd_status run_dose_general(const dd_scan *scan, int64_t j0, int64_t j1, double *out, cudaStream_t stream) {
     const int64_t n = scan->n;
@@ -568,6 +643,10 @@ dd_status dose_range(const dd_scan *scan, dd_precision prec, int64_t j0, int64_t
         // per-visit dwells, flyback or blanker travel: no lag table, coefficients per pair
         if (prec == DD_MIXED) return run_dose_general<ddk::CfgMixed>(scan, j0, j1, out, stream);
         return run_dose_general<ddk::CfgF64>(scan, j0, j1, out, stream);
+    }
+    if (dose_rows_apply(scan, j0, j1)) {
+        if (prec == DD_MIXED) return run_dose_rows<ddk::CfgMixed>(scan, j0, j1, out, stream);
+        return run_dose_rows<ddk::CfgF64>(scan, j0, j1, out, stream);
     }
     if (prec == DD_MIXED) return run_dose<ddk::CfgMixed>(scan, j0, j1, out, stream);
     return run_dose<ddk::CfgF64>(scan, j0, j1, out, stream);

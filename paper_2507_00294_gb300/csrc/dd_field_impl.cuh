@@ -747,6 +747,13 @@ struct BlockSum<float> {
         c += (s - (t - b)) + (x - b);
         s = t;
     }
+    __device__ __forceinline__ void add(const BlockSum &o) { add(o.s); c += o.c; }
+    __device__ __forceinline__ BlockSum shfl_up(int d) const {
+        BlockSum o;
+        o.s = __shfl_up_sync(0xffffffffu, s, d);
+        o.c = __shfl_up_sync(0xffffffffu, c, d);
+        return o;
+    }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
     // s + c rounded to FP32 (one rounding; no FP64 arithmetic)
     __device__ __forceinline__ float result() const { return s + c; }
@@ -755,6 +762,12 @@ template <>
 struct BlockSum<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void add(const BlockSum &o) { s += o.s; }
+    __device__ __forceinline__ BlockSum shfl_up(int d) const {
+        BlockSum o;
+        o.s = __shfl_up_sync(0xffffffffu, s, d);
+        return o;
+    }
     __device__ __forceinline__ double value() const { return s; }
     __device__ __forceinline__ double result() const { return s; }
 };

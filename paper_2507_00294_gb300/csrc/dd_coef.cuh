@@ -9,7 +9,7 @@ namespace ddk {
 // --------------------------------------------------------------- coefficients
 
 // c_m = (-1)^m J_m(r) / m!,  J_m(r) = int_0^1 r s^m / (1 + r s) ds,  m = 0..M, c_0 = ln(1+r).
-// J_m = 1/m - J_{m-1}/r (forward) is stable for r >= 1.  For r < 1 the same recurrence
+// J_m = 1/m - J_{m-1}/r (forward) is stable for r >= 1.  For smaller r the same recurrence
 // is run downward from J_M, which comes from the positive series
 //   J_M = rho sum_k rho^k B(M+1, k+1),  rho = r/(1+r)  (expand 1/(1+rs) about s = 1).
 // 1/n for n = 0..95 (entry 0 unused), exact to FP64 rounding.
@@ -33,10 +33,23 @@ struct RecipTableF {
 static __device__ __constant__ RecipTableF kRecipFTable = RecipTableF();
 #define kRecipF kRecipFTable.v
 
+// k / (M + 1 + k), the ratio of the FP64 series' beta-function factors (M = 15).
+struct BetaRatioTable {
+    double v[64];
+    constexpr BetaRatioTable() : v() {
+        for (int k = 0; k < 64; ++k) v[k] = (double)k / (16.0 + k);
+    }
+};
+static __device__ __constant__ BetaRatioTable kBetaRatioTable = BetaRatioTable();
+
+// The forward recurrence multiplies an error of J_0 by (1/r)^m, but J_m enters as J_m h^m / m!
+// with h <= 1/2: from r = 0.4 on, the sum over m of (1 / (2 r))^m / m! keeps that below
+// e^1.25 roundings, and the series (28 terms at r = 0.4, 57 at r = 1) is not needed there.
 template <int M>
 __device__ void moment_coefficients(double r, double ell, double *c) {
+    static_assert(M == 15, "kBetaRatioTable");
     double J[M + 1];
-    if (r >= 1.0) {
+    if (r >= 0.4) {
         const double ir = 1.0 / r;
         J[0] = ell;
 #pragma unroll
@@ -44,10 +57,10 @@ __device__ void moment_coefficients(double r, double ell, double *c) {
     } else {
         const double rho = r / (1.0 + r);
         double term = rho * kRecip[M + 1], sum = 0.0;
-        // rho < 1/2 here, so the terms shrink at least geometrically: 64 suffice
+        // rho < 0.29 here: the terms shrink geometrically, 64 suffice
         for (int k = 1; k < 64; ++k) {
             sum += term;
-            term *= rho * k * kRecip[M + 1 + k];
+            term *= rho * kBetaRatioTable.v[k];
             if (term <= 1e-18 * sum) break;
         }
         J[M] = sum;

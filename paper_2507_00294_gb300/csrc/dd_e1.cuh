@@ -11,8 +11,7 @@
 // regime", used while h <= 1/2).  Larger h is rare (recent, nearby visits); there
 // E_1(a) and E_1(b) are formed separately (the difference is then well conditioned,
 // E_1(b) <= e^-h E_1(a)):  Ein series (A&S 5.1.11) below x = 1 (FP32) / 2 (FP64), a
-// rational fit of x e^x E_1(x) (FP32, generated by gen_e1_constants.py) or the
-// continued fraction of A&S 5.1.22 by modified Lentz (FP64) above.
+// rational fit of x e^x E_1(x) (generated by gen_e1_constants.py) above.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -147,33 +146,37 @@ __device__ __forceinline__ double ein_f64(double x) {
     return p * x;
 }
 
-// E_1(x) for x > 2: e^-x / f with f = (x+1) - 1/((x+3) - 4/((x+5) - ...)) (A&S 5.1.22,
-// even form), modified Lentz; converges in < 60 steps for x > 2.
-static __device__ __noinline__ double e1_large_f64(double x) {
-    const double tiny = 1e-300;
-    double f = x + 1.0, C = f, Dn = 0.0;
-    for (int k = 1; k < 200; ++k) {
-        const double ak = -(double)k * (double)k;
-        const double bk = x + 2.0 * k + 1.0;
-        Dn = fma(ak, Dn, bk);
-        if (fabs(Dn) < tiny) Dn = tiny;
-        C = bk + ak / C;
-        if (fabs(C) < tiny) C = tiny;
-        Dn = 1.0 / Dn;
-        const double delta = C * Dn;
-        f *= delta;
-        if (fabs(delta - 1.0) < 2e-16) break;
+// x E_1(x) e^x for x > 2 as P*(x) / Q*(x): a rational of degree 9 in 1/x, within 3.8e-18
+// relative on [2, inf) (gen_e1_constants.py); every coefficient is positive, so Horner's
+// rounding stays at a few ulp.  e1_ratio_f64 returns E_1(x) e^x = P* / (x Q*): 19 FMAs and a
+// division, where the continued fraction of A&S 5.1.22 took up to 60 steps of two divisions
+// (one such term alone kept a warp busy for about 70 us).
+static __device__ __constant__ double kE1P64[10] = {
+    0.99999999999999999637, 41.073876422688601655, 645.56102424747329172, 4990.1513622650472973,
+    20326.288895540010955,  43481.796815695771445, 45998.061135410915445, 20938.950545390477397,
+    2973.7124827043992538,  32.248772351909912869};
+static __device__ __constant__ double kE1Q64[10] = {
+    1.0,                    42.073876422688585967, 685.63490067017287432, 5597.6385100868289719,
+    24781.100863259999818,  60291.656989110476737, 78186.977491438231373, 49908.775676338818251,
+    13308.241550527079719,  1001.6481696827983802};
+__device__ __forceinline__ double e1_ratio_f64(double x) {
+    double p = kE1P64[0], q = kE1Q64[0];
+#pragma unroll
+    for (int k = 1; k < 10; ++k) {
+        p = fma(p, x, kE1P64[k]);
+        q = fma(q, x, kE1Q64[k]);
     }
-    return exp(-x) / f;
+    return p / (x * q);
 }
 
 // E_1(a) - E_1(a + h) for h > 1/2 in FP64; ell = ln((a + h)/a).
 static __device__ __noinline__ double e1diff_general_f64(double a, double h, double ell) {
     const double b = a + h;
     if (b <= 2.0) return ell - (ein_f64(b) - ein_f64(a));
-    const double e1b = b >= 745.0 ? 0.0 : e1_large_f64(b);
-    const double e1a = a <= 2.0 ? (-kEulerD - log(a) + ein_f64(a)) : e1_large_f64(a);
-    return e1a - e1b;
+    // E_1(b) <= e^-h E_1(a): below 5e-18 of the difference from h = 40 on
+    if (a > 2.0) return exp(-a) * (h > 40.0 ? e1_ratio_f64(a) : e1_ratio_f64(a) - exp(-h) * e1_ratio_f64(b));
+    const double e1b = b >= 745.0 ? 0.0 : exp(-b) * e1_ratio_f64(b);
+    return (-kEulerD - log(a) + ein_f64(a)) - e1b;
 }
 
 }  // namespace ddk

@@ -7,6 +7,7 @@
    reweighting) on Chebyshev nodes, followed by Lawson reweighting toward minimax.
    Values of F come from mpmath at 30 digits.  The device evaluates
    E1(x) = e^-x P*(x) / (x Q*(x)) with P*(x) = x^4 P(1/x), Q*(x) = x^4 Q(1/x).
+3. The same for FP64: a (9,9) fit on z in (0, 1/2] (x >= 2), solved at 60 digits.
 """
 import math
 from fractions import Fraction
@@ -51,6 +52,41 @@ def fit_rational(p=4, q=4, n=3000):
     return best
 
 
+def fit_rational_f64(d=9, x_min=2, n=160, iters=16):
+    mp.mp.dps = 60
+    zs = [(1 + mp.cos(mp.pi * (2 * i + 1) / (2 * n))) / (2 * x_min) for i in range(n)]
+
+    def F(z):
+        x = 1 / z
+        if x < 3000:
+            return x * mp.e ** x * mp.e1(x)
+        return mp.nsum(lambda k: (-z) ** int(k) * mp.factorial(int(k)), [0, 16])   # to 1e-42
+    f = [F(z) for z in zs]
+    w, lawson, best = [mp.mpf(1)] * n, [mp.mpf(1)] * n, None
+    for it in range(iters):
+        A, rhs = mp.matrix(n, 2 * d + 1), mp.matrix(n, 1)
+        for i, z in enumerate(zs):
+            s = w[i] * lawson[i] / f[i]
+            for k in range(d + 1):
+                A[i, k] = s * z ** k
+            for k in range(1, d + 1):
+                A[i, d + k] = -s * f[i] * z ** k
+            rhs[i] = s * f[i]
+        c = mp.lu_solve(A, rhs)                              # least squares
+        P, Q = [c[k] for k in range(d + 1)], [mp.mpf(1)] + [c[d + k] for k in range(1, d + 1)]
+        Qv = [mp.polyval(Q[::-1], z) for z in zs]
+        err = [abs(mp.polyval(P[::-1], z) / q - v) / v for z, q, v in zip(zs, Qv, f)]
+        m = max(err)
+        if best is None or m < best[0]:
+            best = (m, P, Q)
+        w = [1 / abs(q) for q in Qv]
+        if it >= 4:
+            lawson = [v * (e / m + mp.mpf("1e-3")) for v, e in zip(lawson, err)]
+            t = sum(lawson) / n
+            lawson = [v / t for v in lawson]
+    return best
+
+
 if __name__ == "__main__":
     for k, c in enumerate(ein_coefficients(12), 1):
         print("ein c%-2d = % .17e" % (k, float(c)))
@@ -59,3 +95,7 @@ if __name__ == "__main__":
     # reversed (x-form) coefficients, highest power first for Horner in x
     print("P* (x^4..x^0):", ", ".join("%.9ef" % v for v in P))
     print("Q* (x^4..x^0):", ", ".join("%.9ef" % v for v in Q))
+    m, P, Q = fit_rational_f64()
+    print("max rel err of the (9,9) fit: %s" % mp.nstr(m, 3))
+    print("P* (x^9..x^0):", ", ".join(mp.nstr(v, 20) for v in P))
+    print("Q* (x^9..x^0):", ", ".join(mp.nstr(v, 20) for v in Q))

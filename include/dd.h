@@ -143,12 +143,12 @@ dd_status dd_field_at_times(const dd_scan *scan, const double *pts_xy_m, int64_t
    rounded once in FP64, no fused multiply-add), and
      out[it * n_cols * n_rows + r * n_cols + c] = psi(point (c, r), times_s[it])   [u/m^2]
    -- the result of dd_field_at_times on those points in row-major order, without a point
-   buffer.  In FP32-mixed precision the grid lets a tile of 128 columns x 4 rows split the
-   low-degree pair terms into column and row factors (fewer exponentials per pair); and on
-   grids of at least 64 x 64 points, the visits whose pair terms are on the degree-2 series
-   at every point of the grid (the older ones) are summed as a matrix product of those
-   factors on the tensor cores (BF16 pieces of the FP32 factors, FP32 accumulation); the
-   result then differs from dd_field_at_times by the FP32 rounding, within the same error
+   buffer.  In FP32-mixed precision, on grids of at least 32 x 32 and 4096 points, every
+   visit but the last few is a short sum of Gaussians (Gauss-Legendre nodes) that split into
+   column and row factors, and their sum over visits is a matrix product on the tensor cores
+   (two FP16 pieces of each FP32 factor, FP32 accumulation); smaller grids split the
+   low-degree pair terms into column and row factors on the CUDA cores.  The result then
+   differs from dd_field_at_times by the FP32 rounding, within the same error
    budget.  times_s and out as in dd_field_at_times.  A grid with no columns, rows or
    snapshots is a no-op.
    Errors: DD_EINVAL (NULL scan/buffer, negative sizes, non-finite origin or spacing, more
@@ -159,19 +159,18 @@ dd_status dd_field_on_grid(const dd_scan *scan, double x0_m, double y0_m, double
                            int64_t n_cols, int64_t n_rows, const double *times_s, int64_t n_t,
                            dd_precision prec, double *out, void *cuda_stream);
 
-/* The split dd_field_on_grid makes in FP32-mixed precision, host-only (no GPU work):
+/* How many of a snapshot's visits are smooth over a whole grid, host-only (no GPU work):
    prefix[it] = the number of leading visits (in visit order) whose pair terms at snapshot
-   times_s[it] (host array) are summed on the tensor cores, and prefix_deg2[it] (NULL: not
-   wanted) how many of them in the degree-2 form; the visits after prefix[it] go to the
-   CUDA-core tile kernel.  A visit qualifies when its pair term is on the degree-2 (degree-4)
-   series at every point of the grid: h = rho^2 dq <= 0.04 (0.33) for rho^2 up to the
+   times_s[it] (host array) are on the degree-4 exponent series at every point of the grid,
+   and prefix_deg2[it] (NULL: not wanted) how many of them on the degree-2 series.  A visit
+   qualifies when h = rho^2 dq <= 0.04 (0.33) for rho^2 up to the
    largest squared distance between the grid's box and the visits' box, with dq bounded
    through the scan's longest dwell (dq <= c / ((w1 - c) w1), c = 4 D tau_max, at
    w1 = 2 sigma^2 + 4 D (t - t_i)), so the qualifying visits are those started by
-   t - dT*: prefixes.  0 for grids smaller than 64 x 64 points and for snapshots with no
-   qualifying visit; the degree-4 band is left out where its coefficients of (rho^2)^4
-   would leave the FP32 normal range, and the path falls back to 0 everywhere if the
-   split's partial sums would exceed its 1 GiB workspace budget.
+   t - dT*: prefixes.  dd_field_on_grid in FP32-mixed precision sums all of them on the
+   tensor cores (and the visits after them up to h = 218, too).  0 for grids smaller than
+   64 x 64 points and for snapshots with no qualifying visit; the degree-4 band is left out
+   where its coefficients of (rho^2)^4 would leave the FP32 normal range.
    Errors: DD_EINVAL (NULL scan or buffers, negative sizes, non-finite grid or times,
    device arrays). */
 dd_status dd_field_grid_split(const dd_scan *scan, double x0_m, double y0_m, double dx_m, double dy_m,
@@ -255,12 +254,9 @@ typedef struct dd_batch dd_batch;
    grid_wh[2k], grid_wh[2k+1] = (columns W_k, rows H_k) of scan k; point (c, r) of scan k
    sits at (x0 + c dx, y0 + r dy) (one product and one sum each, no fused multiply-add) and
    its field goes to out[off_k + r W_k + c], off_k = sum over the earlier scans of W H.
-   dd_batch_run and dd_batch_tune then take pts_xy_m = NULL.  In FP32-mixed precision the
-   grid lets tiles of 32 x 32 points split the low-degree pair terms into column and row
-   factors (as dd_field_on_grid does), and for grids of at least 64 x 64 points each scan's
-   visits on the degree-2 (then degree-4) series at every point of its grid are summed as
-   matrix products on the tensor cores, the prefixes dd_field_grid_split reports, with the
-   same completion waits and NaN-on-timeout rule as dd_field_on_grid (dd_field_check); the
+   dd_batch_run and dd_batch_tune then take pts_xy_m = NULL.  In FP32-mixed precision every
+   scan is summed as dd_field_on_grid sums it on large grids, with the
+   same completion waits and NaN-on-timeout rule (dd_field_check); the
    result differs from the point-list plan by FP32 rounding only.  Errors: DD_EINVAL (sizes,
    non-finite origin or spacing, more than 2^31 points), DD_ENOMEM, DD_ECUDA. */
 dd_status dd_batch_create_grid(const dd_scan *const *scans, int32_t n_scans, const double *grid_xy,

@@ -13,6 +13,7 @@
 // threads x points-per-thread) by timing each once; choices are cached in-process and,
 // when DD_TUNE_CACHE names a file, in that JSON file.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -26,11 +27,10 @@
 #include <type_traits>
 #include <vector>
 
-#include "dd_batch_grid.cuh"
 #include "dd_coef.cuh"
 #include "dd_e1.cuh"
 #include "dd_field_impl.cuh"
-#include "dd_field_tc.cuh"
+#include "dd_grid.h"
 #include "dd_internal.h"
 
 namespace ddk {
@@ -47,12 +47,7 @@ struct BScan {
     // a grid of points (dd_batch_create_grid): point r W + c at (x0 + c dx, y0 + r dy) [m];
     // W = 0 for an explicit point list
     double gx0, gy0, gdx, gdy;
-    int64_t gW, gH, n_tc;
-    // grid plans in FP32-mixed: visits [0, k_tc) are summed by the tensor-core contraction
-    // into nq_tc FP32 rows of t_stride points at t_off (dd_field_tc.cuh); the CUDA-core tile
-    // kernel takes visits [k_tc, nact), in the blocks [blk0, nblk)
-    int k_tc, nq_tc, blk0;
-    int64_t t_off, t_stride;
+    int64_t gW, gH;
 };
 
 __device__ __forceinline__ int find_segment(const int64_t *__restrict__ offs, int n, int64_t g) {
@@ -146,49 +141,15 @@ batch_field_kernel(const BScan *__restrict__ sc, const int4 *__restrict__ items,
     }
 }
 
-// Persistent CTAs over grid tiles of 32 x 32 points (FP32-mixed): item (scan, tile, block).
-__global__ void __launch_bounds__(kBgThreads, 8)
-batch_grid_kernel(const BScan *__restrict__ sc, const int4 *__restrict__ items, int n_items,
-                  unsigned *__restrict__ counter, const float4 *__restrict__ F, const RecF32 *__restrict__ rec,
-                  int sb, double *__restrict__ partial) {
-    __shared__ BGridSmem sm;
-    __shared__ int s_item;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = (int)atomicAdd(counter, 1u);
-        __syncthreads();
-        const int it = s_item;
-        __syncthreads();
-        if (it >= n_items) break;
-        const int4 item = items[it];
-        const BScan &S = sc[item.x];
-        const int s_begin = max(item.z * sb, S.k_tc);
-        const int s_end = min(item.z * sb + sb, S.nact);
-        field_tile_bgrid(sm, S.srcF, F + S.pt_off, S.gW, S.gH, item.y % S.n_tc, item.y / S.n_tc,
-                         rec + S.rec_off, s_begin, s_end, partial + S.part_off + (int64_t)item.z * S.n_pts);
-    }
-}
-
 __global__ void batch_reduce_kernel(const BScan *__restrict__ sc, const int64_t *__restrict__ pt_offs, int n_scans,
-                                    int64_t total, const double *__restrict__ partial, const float *__restrict__ tpart,
-                                    bool mixed_grid, double *__restrict__ out) {
+                                    int64_t total, const double *__restrict__ partial, double *__restrict__ out) {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= total) return;
     const BScan &S = sc[find_segment(pt_offs, n_scans, g)];
     const int64_t p = g - S.pt_off;
-    // the tensor-core rows first, then the CUDA-core blocks from the first one past k_tc.
-    // Grid plans in FP32-mixed hold FP32 sums (the block sums exactly, in FP64 storage):
-    // a compensated FP32 sum (FP64 arithmetic is 64 times slower on this part); the others
-    // sum in FP64.
-    if (S.nq_tc > 0 || mixed_grid) {
-        BlockSum<float> acc;
-        for (int q = 0; q < S.nq_tc; ++q) acc.add(tpart[S.t_off + (int64_t)q * S.t_stride + p]);
-        for (int b = S.blk0; b < S.nblk; ++b) acc.add((float)partial[S.part_off + (int64_t)b * S.n_pts + p]);
-        out[g] = S.pref * acc.value();
-    } else {
-        double acc = 0.0;
-        for (int b = 0; b < S.nblk; ++b) acc += partial[S.part_off + (int64_t)b * S.n_pts + p];
-        out[g] = S.pref * acc;
-    }
+    double acc = 0.0;
+    for (int b = 0; b < S.nblk; ++b) acc += partial[S.part_off + (int64_t)b * S.n_pts + p];
+    out[g] = S.pref * acc;
 }
 
 // Kernel variants with the same 512-point tile (so they share one work list).
@@ -223,19 +184,15 @@ struct dd_batch {
     double *d_X = nullptr, *d_Y = nullptr, *d_part = nullptr;
     float4 *d_F = nullptr;
     void *d_rec = nullptr;
-    // tensor-core contraction of grid plans: scan table, work items (degree 2, then
-    // degree 4), their CTA counts and FP32 partial rows
-    ddk::TcScan *d_tcs = nullptr;
-    ddk::TcItem *d_titems = nullptr;
-    int n_t2 = 0, n_t4 = 0, cta_t2 = 0, cta_t4 = 0;
-    float *d_tpart = nullptr;
     double *d_pts = nullptr, *d_out = nullptr;   // staging for host buffers
     cudaStream_t cap = nullptr;
-    cudaStream_t side = nullptr;        // the graph's second branch (coefficients, contraction)
-    cudaEvent_t ev_fork = nullptr, ev_coef = nullptr, ev_join = nullptr;
+    cudaStream_t side = nullptr;        // the graph's second branch (coefficients)
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaGraphExec_t exec = nullptr;
     bool on_grid = false;               // points formed from per-scan grids (no point buffer)
-    bool grid_tiles = false;            // ... and evaluated by the grid tile kernel (FP32-mixed)
+    // ... and evaluated by the grid contraction (FP32-mixed; its tables and buffers are the
+    // plan's workspace)
+    std::unique_ptr<dd::GridEngine> engine;
     const double *g_pts = nullptr;
     double *g_out = nullptr;
     int g_variant = -1;
@@ -273,10 +230,13 @@ void launch_field(dd_batch *b, int grid, cudaStream_t st) {
 
 // Enqueue the whole batch evaluation on `st` (used for capture and for tuning).
 dd_status enqueue(dd_batch *b, const double *pts, double *out, int variant, cudaStream_t st) {
+    if (b->engine) {
+        DD_CUDA_TRY(b->engine->enqueue(out, st, nullptr, nullptr, nullptr, false, false));
+        return DD_OK;
+    }
     const unsigned nb_pts = (unsigned)((b->total_pts + 255) / 256);
     // two branches: the points on `st`, the coefficient records beside them on `side`
-    // (they only read the scans); with the tensor-core contraction, it follows the records
-    // on `side` while the grid tiles run on `st`; both join before the reduce
+    // (they only read the scans), joined before the field kernel
     DD_CUDA_TRY(cudaEventRecord(b->ev_fork, st));
     DD_CUDA_TRY(cudaStreamWaitEvent(b->side, b->ev_fork, 0));
     DD_CUDA_TRY(cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned), st));
@@ -290,23 +250,9 @@ dd_status enqueue(dd_batch *b, const double *pts, double *out, int variant, cuda
             ddk::batch_coef_kernel<ddk::RecF64><<<nb, 128, 0, b->side>>>(b->d_sc, b->d_rec_offs, b->n_scans,
                                                                        b->total_rec, (ddk::RecF64 *)b->d_rec);
     }
-    DD_CUDA_TRY(cudaEventRecord(b->ev_coef, b->side));
-    DD_CUDA_TRY(cudaStreamWaitEvent(st, b->ev_coef, 0));
-    if (b->n_t2 + b->n_t4 > 0) {
-        // the older visits of the larger grids on the tensor cores (after the points)
-        DD_CUDA_TRY(cudaEventRecord(b->ev_fork, st));
-        DD_CUDA_TRY(cudaStreamWaitEvent(b->side, b->ev_fork, 0));
-        DD_CUDA_TRY(dd::launch_field_tc(2, b->d_tcs, (const ddk::RecF32 *)b->d_rec, b->d_titems, b->n_t2, b->cta_t2,
-                                        b->side));
-        DD_CUDA_TRY(dd::launch_field_tc(4, b->d_tcs, (const ddk::RecF32 *)b->d_rec, b->d_titems + b->n_t2, b->n_t4,
-                                        b->cta_t4, b->side));
-    }
     DD_CUDA_TRY(cudaEventRecord(b->ev_join, b->side));
-    if (b->n_items > 0 && b->grid_tiles) {
-        ddk::batch_grid_kernel<<<b->grid[0], ddk::kBgThreads, 0, st>>>(b->d_sc, b->d_items, b->n_items, b->d_counter,
-                                                                      b->d_F, (const ddk::RecF32 *)b->d_rec, b->sb,
-                                                                      b->d_part);
-    } else if (b->n_items > 0) {
+    DD_CUDA_TRY(cudaStreamWaitEvent(st, b->ev_join, 0));
+    if (b->n_items > 0) {
         const int g = b->grid[variant];
         if (b->prec == DD_MIXED) {
             if (variant == 0) launch_field<ddk::CfgMixed>(b, g, st);
@@ -319,9 +265,7 @@ dd_status enqueue(dd_batch *b, const double *pts, double *out, int variant, cuda
             else launch_field<ddk::CfgF64>(b, g, st);
         }
     }
-    DD_CUDA_TRY(cudaStreamWaitEvent(st, b->ev_join, 0));
-    ddk::batch_reduce_kernel<<<nb_pts, 256, 0, st>>>(b->d_sc, b->d_pt_offs, b->n_scans, b->total_pts, b->d_part,
-                                                     b->d_tpart, b->grid_tiles, out);
+    ddk::batch_reduce_kernel<<<nb_pts, 256, 0, st>>>(b->d_sc, b->d_pt_offs, b->n_scans, b->total_pts, b->d_part, out);
     DD_CUDA_TRY(cudaGetLastError());
     return DD_OK;
 }
@@ -352,17 +296,6 @@ void tune_cache_store() {
     size_t k = 0;
     for (auto &kv : g_tune) f << "  \"" << kv.first << "\": " << kv.second << (++k < g_tune.size() ? ",\n" : "\n");
     f << "}\n";
-}
-
-int grid_kernel_ctas() {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaFuncSetAttribute(ddk::batch_grid_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess)
-        cudaGetLastError();
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ddk::batch_grid_kernel, ddk::kBgThreads, 0);
-    return std::max(1, sms * std::max(1, std::min(per, 8)));
 }
 
 // Plan of a batch: explicit points (grid_xy == NULL, pt_offsets given) or per-scan grids
@@ -397,17 +330,12 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
     b->prec = prec;
     b->n_scans = n_scans;
     b->on_grid = grid_xy != nullptr;
-    b->grid_tiles = b->on_grid && prec == DD_MIXED;
+    if (b->on_grid && prec == DD_MIXED) b->engine.reset(new dd::GridEngine());
     DD_CUDA_TRY(cudaGetDevice(&b->device));
     const int tile = prec == DD_MIXED ? kTile : ddk::CfgF64::kThreads * ddk::CfgF64::kPPT;
     std::vector<ddk::BScan> sc((size_t)n_scans);
     std::vector<int64_t> pt_offs((size_t)n_scans), rec_offs((size_t)n_scans);
     std::vector<std::pair<int64_t, int4>> items;
-    // tensor-core work items (FP32-mixed grid plans): degree 2 and degree 4, each at most
-    // kTcMaxItemStages stages long (the FP32 accumulation's error budget), times the tiles
-    std::vector<std::pair<int64_t, ddk::TcItem>> titems2, titems4;
-    std::vector<ddk::TcScan> tcs((size_t)n_scans, ddk::TcScan{});
-    int64_t tpart_total = 0;
     int64_t rec = 0, part = 0;
     for (int k = 0; k < n_scans; ++k) {
         const dd_scan *s = scans[k];
@@ -429,79 +357,73 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
         S.rec_off = rec;
         S.part_off = part;
         S.gx0 = S.gy0 = S.gdx = S.gdy = 0.0;
-        S.gW = S.gH = S.n_tc = 0;
+        S.gW = S.gH = 0;
         if (grid_xy) {
             S.gx0 = grid_xy[4 * k]; S.gy0 = grid_xy[4 * k + 1];
             S.gdx = grid_xy[4 * k + 2]; S.gdy = grid_xy[4 * k + 3];
             S.gW = grid_wh[2 * k]; S.gH = grid_wh[2 * k + 1];
-            S.n_tc = (S.gW + ddk::kBgCols - 1) / ddk::kBgCols;
         }
-        S.k_tc = S.nq_tc = 0;
-        S.t_off = S.t_stride = 0;
-        if (b->grid_tiles && S.nact > 0) {
-            int K2 = 0, K = 0;
-            dd::tc_prefixes(s, S.gx0, S.gy0, S.gdx, S.gdy, S.gW, S.gH, S.tdim, S.nact, &K2, &K);
-            if (K > 0) {
-                const int64_t n_tcols = (S.gW + ddk::kTcTile - 1) / ddk::kTcTile;
-                const int n_ttiles = (int)(n_tcols * ((S.gH + ddk::kTcTile - 1) / ddk::kTcTile));
-                constexpr int kPiece = ddk::kTcMaxItemStages * ddk::kTcStage;
-                int row = 0;
-                auto pieces = [&](int lo, int hi, std::vector<std::pair<int64_t, ddk::TcItem>> &list) {
-                    for (int vb = lo; vb < hi; vb += kPiece, ++row) {
-                        const int ve = std::min(hi, vb + kPiece);
-                        for (int t = 0; t < n_ttiles; ++t)
-                            list.push_back({(int64_t)(ve - vb), ddk::TcItem{vb, ve, t, row, S.rec_off, k, 0}});
-                    }
-                };
-                pieces(0, K2, titems2);
-                pieces(K2, K, titems4);
-                S.k_tc = K;
-                S.nq_tc = row;
-                S.t_stride = (S.n_pts + 3) / 4 * 4;             // 16-byte aligned rows
-                S.t_off = tpart_total;
-                tpart_total += (int64_t)row * S.t_stride;
-                // the points and partial rows are filled in once the plan's buffers exist
-                tcs[(size_t)k] = ddk::TcScan{S.gW, S.gH, n_tcols, S.srcF, nullptr, nullptr, S.t_stride};
-            }
+        if (b->engine) {
+            if (S.n_pts == 0) continue;
+            const dd::GridBox box{S.gx0, S.gy0, S.gdx, S.gdy, S.gW, S.gH};
+            const int g = b->engine->add_grid(s, box);
+            const int t = b->engine->add_table(s, box, src, S.tdim, S.nact);
+            b->engine->add_job(s, S.srcF, g, t, S.nact, 0, S.pt_off);
+            continue;
         }
-        S.blk0 = S.k_tc >= S.nact ? S.nblk : S.k_tc / b->sb;
         pt_offs[(size_t)k] = S.pt_off;
         rec_offs[(size_t)k] = rec;
         rec += S.nact;
         part += (int64_t)S.nblk * S.n_pts;
-        // grid tiles of 32 x 32 points (items cost by their valid points), else point tiles
-        const int64_t n_tr = b->grid_tiles ? (S.gH + ddk::kBgRows - 1) / ddk::kBgRows : 0;
-        const int64_t tiles = S.n_pts == 0 ? 0 : b->grid_tiles ? S.n_tc * n_tr : (S.n_pts + tile - 1) / tile;
-        for (int blk = S.blk0; blk < S.nblk; ++blk) {
-            const int64_t nsrc = std::min<int64_t>(S.nact, (int64_t)(blk + 1) * b->sb) -
-                                 std::max<int64_t>((int64_t)blk * b->sb, S.k_tc);
-            for (int64_t t = 0; t < tiles; ++t) {
-                int64_t npt;
-                if (b->grid_tiles) {
-                    const int64_t tc = t % S.n_tc, tr = t / S.n_tc;
-                    npt = std::min<int64_t>(ddk::kBgCols, S.gW - tc * ddk::kBgCols) *
-                          std::min<int64_t>(ddk::kBgRows, S.gH - tr * ddk::kBgRows);
-                } else {
-                    npt = std::min<int64_t>(tile, S.n_pts - t * tile);
-                }
-                items.push_back({nsrc * npt, make_int4(k, (int)t, blk, 0)});
-            }
+        const int64_t tiles = (S.n_pts + tile - 1) / tile;
+        for (int blk = 0; blk < S.nblk; ++blk) {
+            const int64_t nsrc = std::min<int64_t>(S.nact, (int64_t)(blk + 1) * b->sb) - (int64_t)blk * b->sb;
+            for (int64_t t = 0; t < tiles; ++t)
+                items.push_back({nsrc * std::min<int64_t>(tile, S.n_pts - t * tile), make_int4(k, (int)t, blk, 0)});
         }
     }
     std::stable_sort(items.begin(), items.end(),
                      [](const std::pair<int64_t, int4> &x, const std::pair<int64_t, int4> &y) { return x.first > y.first; });
-    auto longest_first = [](const std::pair<int64_t, ddk::TcItem> &x, const std::pair<int64_t, ddk::TcItem> &y) {
-        return x.first > y.first;
-    };
-    std::stable_sort(titems2.begin(), titems2.end(), longest_first);
-    std::stable_sort(titems4.begin(), titems4.end(), longest_first);
-    b->n_t2 = (int)titems2.size();
-    b->n_t4 = (int)titems4.size();
     b->total_pts = pt_offsets[n_scans];
     b->total_rec = rec;
     b->total_part = part;
     b->n_items = (int)items.size();
     const size_t rec_size = prec == DD_MIXED ? sizeof(ddk::RecF32) : sizeof(ddk::RecF64);
+    int64_t pairs = 0;
+    for (auto &S : sc) pairs += (int64_t)S.nact * S.n_pts;
+    b->pairs = pairs;
+    // tuning key: device name, precision and a log2 bucket of the pair count
+    cudaDeviceProp prop;
+    DD_CUDA_TRY(cudaGetDeviceProperties(&prop, b->device));
+    int bucket = 0;
+    while ((int64_t(1) << bucket) < pairs && bucket < 62) ++bucket;
+    std::ostringstream key;
+    key << prop.name << "/sm" << prop.major << prop.minor << "/" << (prec == DD_MIXED ? "mixed" : "fp64")
+        << (b->on_grid ? "/grid" : "") << "/2^" << bucket;
+    b->tune_key = key.str();
+    {
+        std::lock_guard<std::mutex> lock(g_tune_mu);
+        tune_cache_load();
+        auto f = g_tune.find(b->tune_key);
+        b->variant = f != g_tune.end() ? std::min(std::max(f->second, 0), kVariants - 1) : 0;
+    }
+    if (b->engine) {
+        b->variant = 0;                                  // one kernel for grids
+        DD_CUDA_TRY(b->engine->finish(false));
+        b->n_items = (int)std::min<int64_t>(b->engine->n_runs() + b->engine->n_tiles(), INT_MAX);
+        cudaError_t err = cudaMalloc(&b->ws, b->engine->workspace_bytes());
+        if (err != cudaSuccess) {
+            cudaGetLastError();
+            return dd::fail(DD_ENOMEM, std::string("dd_batch_create_grid: cudaMalloc: ") + cudaGetErrorString(err));
+        }
+        b->engine->bind(b->ws);
+        std::vector<char> tables(b->engine->table_bytes());
+        b->engine->write_tables(tables.data());
+        DD_CUDA_TRY(cudaMemcpy(b->ws, tables.data(), tables.size(), cudaMemcpyHostToDevice));
+        DD_CUDA_TRY(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
+        *out = b.release();
+        return DD_OK;
+    }
     size_t bytes = 0;
     auto add = [&](size_t x) { size_t o = (bytes + 255) & ~size_t(255); bytes = o + x; return o; };
     const size_t o_sc = add(sc.size() * sizeof(ddk::BScan));
@@ -513,9 +435,6 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
     const size_t o_f = add((size_t)std::max<int64_t>(1, b->total_pts) * sizeof(float4));
     const size_t o_rec = add((size_t)std::max<int64_t>(1, rec) * rec_size);
     const size_t o_part = add((size_t)std::max<int64_t>(1, part) * sizeof(double));
-    const size_t o_tcs = add(tcs.size() * sizeof(ddk::TcScan));
-    const size_t o_ti = add((size_t)std::max(1, b->n_t2 + b->n_t4) * sizeof(ddk::TcItem));
-    const size_t o_tp = add((size_t)std::max<int64_t>(4, tpart_total) * sizeof(float));
     cudaError_t err = cudaMalloc(&b->ws, bytes);
     if (err != cudaSuccess) {
         cudaGetLastError();
@@ -532,25 +451,6 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
     b->d_F = (float4 *)(base + o_f);
     b->d_rec = base + o_rec;
     b->d_part = (double *)(base + o_part);
-    b->d_tcs = (ddk::TcScan *)(base + o_tcs);
-    b->d_titems = (ddk::TcItem *)(base + o_ti);
-    b->d_tpart = (float *)(base + o_tp);
-    if (b->n_t2 + b->n_t4 > 0) {
-        for (int k = 0; k < n_scans; ++k) {
-            if (sc[(size_t)k].nq_tc == 0) continue;
-            tcs[(size_t)k].ptsF = b->d_F + sc[(size_t)k].pt_off;
-            tcs[(size_t)k].partial = b->d_tpart + sc[(size_t)k].t_off;
-        }
-        std::vector<ddk::TcItem> ti;
-        ti.reserve(titems2.size() + titems4.size());
-        for (auto &x : titems2) ti.push_back(x.second);
-        for (auto &x : titems4) ti.push_back(x.second);
-        DD_CUDA_TRY(cudaMemcpy(b->d_tcs, tcs.data(), tcs.size() * sizeof(ddk::TcScan), cudaMemcpyHostToDevice));
-        DD_CUDA_TRY(cudaMemcpy(b->d_titems, ti.data(), ti.size() * sizeof(ddk::TcItem), cudaMemcpyHostToDevice));
-        DD_CUDA_TRY(dd::prepare_field_tc());
-        b->cta_t2 = (int)std::min<int64_t>(b->n_t2, std::max<int64_t>(1, dd::field_tc_resident(2)));
-        b->cta_t4 = (int)std::min<int64_t>(b->n_t4, std::max<int64_t>(1, dd::field_tc_resident(4)));
-    }
     std::vector<int4> it(items.size());
     for (size_t k = 0; k < items.size(); ++k) it[k] = items[k].second;
     DD_CUDA_TRY(cudaMemcpy(b->d_sc, sc.data(), sc.size() * sizeof(ddk::BScan), cudaMemcpyHostToDevice));
@@ -560,35 +460,13 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
     DD_CUDA_TRY(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
     DD_CUDA_TRY(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
     DD_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
-    DD_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_coef, cudaEventDisableTiming));
     DD_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming));
-    if (b->grid_tiles)
-        b->grid = {grid_kernel_ctas(), grid_kernel_ctas(), grid_kernel_ctas(), grid_kernel_ctas()};
-    else if (prec == DD_MIXED)
+    if (prec == DD_MIXED)
         b->grid = {persistent_grid<ddk::CfgMixed>(), persistent_grid<ddk::CfgMixed256>(), persistent_grid<ddk::CfgMixed64>(),
                    persistent_grid<ddk::CfgMixed64x12>()};
     else
         b->grid = {persistent_grid<ddk::CfgF64>(), persistent_grid<ddk::CfgF64x256>(), persistent_grid<ddk::CfgF64>(),
                    persistent_grid<ddk::CfgF64>()};
-    // tuning key: device name, precision and a log2 bucket of the pair count
-    cudaDeviceProp prop;
-    DD_CUDA_TRY(cudaGetDeviceProperties(&prop, b->device));
-    int64_t pairs = 0;
-    for (auto &S : sc) pairs += (int64_t)S.nact * S.n_pts;
-    b->pairs = pairs;
-    int bucket = 0;
-    while ((int64_t(1) << bucket) < pairs && bucket < 62) ++bucket;
-    std::ostringstream key;
-    key << prop.name << "/sm" << prop.major << prop.minor << "/" << (prec == DD_MIXED ? "mixed" : "fp64")
-        << (b->on_grid ? "/grid" : "") << "/2^" << bucket;
-    b->tune_key = key.str();
-    {
-        std::lock_guard<std::mutex> lock(g_tune_mu);
-        tune_cache_load();
-        auto f = g_tune.find(b->tune_key);
-        b->variant = f != g_tune.end() ? std::min(std::max(f->second, 0), kVariants - 1) : 0;
-    }
-    if (b->grid_tiles) b->variant = 0;                  // one kernel for grid tiles
     *out = b.release();
     return DD_OK;
 }
@@ -628,7 +506,7 @@ dd_status dd_batch_tune(dd_batch *b, const double *pts_xy_m, int32_t *chosen) {
     DD_CUDA_TRY(cudaEventCreate(&e1));
     float best = 1e30f;
     int best_v = 0;
-    const int nv = b->grid_tiles ? 1 : b->prec == DD_MIXED ? kVariants : 2;
+    const int nv = b->engine ? 1 : b->prec == DD_MIXED ? kVariants : 2;
     for (int v = 0; v < nv; ++v) {
         dd_status st = enqueue(b, pts_xy_m, tmp, v, b->cap);           // warm
         if (st != DD_OK) { cudaFree(tmp); return st; }
@@ -689,7 +567,7 @@ dd_status dd_batch_run(dd_batch *b, const double *pts_xy_m, double *out, void *c
         b->g_variant = b->variant;
     }
     {
-        dd::ProfScope ps(b->grid_tiles ? "batch_grid_mixed_32x32" : variant_name(b->prec, b->variant), stream);
+        dd::ProfScope ps(b->engine ? "batch_grid_mixed" : variant_name(b->prec, b->variant), stream);
         DD_CUDA_TRY(cudaGraphLaunch(b->exec, stream));
     }
     if (out_host)
@@ -705,7 +583,6 @@ void dd_batch_destroy(dd_batch *b) {
     if (b->cap) cudaStreamDestroy(b->cap);
     if (b->side) cudaStreamDestroy(b->side);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-    if (b->ev_coef) cudaEventDestroy(b->ev_coef);
     if (b->ev_join) cudaEventDestroy(b->ev_join);
     cudaFree(b->ws);
     cudaFree(b->d_pts);

@@ -28,7 +28,7 @@
 #include "dd_e1.cuh"
 #include "dd_field_grid.cuh"
 #include "dd_field_impl.cuh"
-#include "dd_field_tc.cuh"
+#include "dd_grid.h"
 #include "dd_internal.h"
 
 namespace ddk {
@@ -81,32 +81,20 @@ __global__ void prep_points_lag_kernel(int nb_lag, int64_t M, double s, double k
         prep_point((int64_t)(blockIdx.x - nb_lag) * blockDim.x + threadIdx.x, xy, g, n, inv_p, X, Y, F);
 }
 
-// out[row[j]][p] = pref * (sum_{q < nq[j]} tpart[(trow0[j] + q) * pstride + p]
-//                          + sum_{kb0[j] <= k < nblk[j]} partial[(k * n_tg + j) * pstride + p]):
-// the tensor-core chunks of snapshot j (the older visits), then its visit blocks, in that
-// order (deterministic); four points per thread, so that each load moves 16 bytes or more.
-// kb0 and nq NULL: every block from 0, no tensor-core rows.
+// out[row[j]][p] = pref * sum_{k < nblk[j]} partial[(k * n_tg + j) * pstride + p], the visit
+// blocks of snapshot j in that order (deterministic); four points per thread, so that each
+// load moves 16 bytes or more.
 template <typename Part>
 __global__ void reduce_kernel(const Part *__restrict__ partial, const int *__restrict__ nblk_of_snap,
-                              const int *__restrict__ kb0_of_snap, const Part *__restrict__ tpart,
-                              const int *__restrict__ nq_of_snap, const int *__restrict__ trow0,
                               const int *__restrict__ row, int n_tg, int64_t n_pts, int64_t pstride, double pref,
                               double *__restrict__ out) {
     const int j = blockIdx.y;
     const int64_t p0 = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (p0 >= n_pts) return;
     const int nb = nblk_of_snap[j];
-    const int kb0 = kb0_of_snap ? kb0_of_snap[j] : 0;
-    const int nq = nq_of_snap ? nq_of_snap[j] : 0;
     BlockSum<Part> acc[4];
-    for (int k = 0; k < nq; ++k) {
-        Part v[4];
-        load4_cg(tpart + ((int64_t)trow0[j] + k) * pstride + p0, v);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q].add(v[q]);
-    }
 #pragma unroll 4
-    for (int k = kb0; k < nb; ++k) {
+    for (int k = 0; k < nb; ++k) {
         Part v[4];
         load4_cg(partial + ((int64_t)k * n_tg + j) * pstride + p0, v);
 #pragma unroll
@@ -160,7 +148,7 @@ struct HostTables {
 // Sizes of the workspace a call needs (the same function drives the carve).
 template <typename Cfg>
 size_t workspace_bytes(int64_t n_pts, int64_t n_src, int group, int sb, bool out_host, bool pts_host,
-                       int n_t, int64_t n_rec, int64_t trows, int64_t n_titems) {
+                       int n_t, int64_t n_rec) {
     using Rec = typename Cfg::Rec;
     const int nblk_max = (int)((n_src + sb - 1) / sb);
     const int n_chunks = (group + Cfg::kTCH - 1) / Cfg::kTCH;
@@ -171,13 +159,11 @@ size_t workspace_bytes(int64_t n_pts, int64_t n_src, int group, int sb, bool out
     add(2 * (size_t)n_pts * sizeof(double));                  // X, Y in pitch units
     add((size_t)n_pts * sizeof(float4));                      // the same as float-float
     add((size_t)group * sizeof(double));                      // snapshot times
-    add((size_t)group * sizeof(int) * 7);                     // nact, row, nblk, kst, kb0, nq, trow0 per snapshot
+    add((size_t)group * sizeof(int) * 3);                     // nact, row, nblk per snapshot
     add((size_t)group * sizeof(int64_t));                     // record row offset per snapshot
     add((size_t)n_chunks * nblk_max * sizeof(int2));          // (chunk, block) descriptors
-    add((size_t)n_titems * sizeof(ddk::TcItem));              // tensor-core work items
     add((size_t)n_rec * sizeof(Rec));                         // coefficient records
     add((size_t)nblk_max * group * ((n_pts + 3) / 4 * 4) * sizeof(typename Cfg::Real));   // partial sums
-    add((size_t)trows * ((n_pts + 3) / 4 * 4) * sizeof(float));                           // tensor-core partials
     return b + 256;
 }
 
@@ -236,24 +222,24 @@ int64_t resident_ctas() {
     return v;
 }
 
-// ---- the tensor-core part of the grid field (dd_field_tc.cuh)
+// ---- the prefixes that dd_field_grid_split reports
 //
-// A visit is handed to the contraction for snapshot j when its pair term is on the degree-2
-// (or degree-4) series at every point of the grid: h = rho^2 dq <= kL2H (kL4H) for rho^2 up
-// to R2, the largest squared distance between the grid's box and the box of the visits.
-// With c = 4 kappa tau_max, dq = 1/w0 - 1/w1 <= c / ((w1 - c) w1) for every visit of the
-// scan (dq grows with the dwell at a fixed w1 = 2s + 4 kappa (t - T_i)), so every visit
-// with w1 at or above the root w1* of (w1 - c) w1 = c R2 / h_limit (and its dwell over)
-// qualifies: the prefix of the visits that started by t_j - dT*, dT* = (w1* - 2s) /
-// (4 kappa), found by bisection of the start times.  The degree-2 prefix [0, K2) and the
-// degree-4 band [K2, K) go to the contraction (the degree-4 band only while its records'
-// g_4x = log2(e) l_4 dq^4 stay in the FP32 normal range, dq >= kMinDqX), the rest [K, nact)
-// to the CUDA-core tile.
+// A visit is on the degree-2 (degree-4) series at every point of the grid when
+// h = rho^2 dq <= kL2H (kL4H) for rho^2 up to R2, the largest squared distance between the
+// grid's box and the box of the visits.  With c = 4 kappa tau_max, dq = 1/w0 - 1/w1 <=
+// c / ((w1 - c) w1) for every visit of the scan (dq grows with the dwell at a fixed
+// w1 = 2s + 4 kappa (t - T_i)), so every visit with w1 at or above the root w1* of
+// (w1 - c) w1 = c R2 / h_limit (and its dwell over) qualifies: the prefix of the visits that
+// started by t_j - dT*, dT* = (w1* - 2s) / (4 kappa), found by bisection of the start times.
+// (The degree-4 band only while its records' coefficients of rho^8 stay in the FP32 normal
+// range, dq >= kMinDqX.)  All of them are among the visits that the contraction of dd_grid.cu
+// takes, whose bands reach h = 218.
+constexpr int64_t kSplitMinSide = 64;
+
 struct TcPlan {
     bool on = false;
-    int64_t n_tile_cols = 0, n_tiles = 0;
     std::vector<int> K2;         // per snapshot (time order): the degree-2 visits [0, K2)
-    std::vector<int> K;          // and the degree-4 band [K2, K); the CUDA-core tile from K
+    std::vector<int> K;          // and the degree-4 band [K2, K)
 };
 
 // Age (in dwells) from which every visit of the scan is on the series of the given h limit
@@ -274,8 +260,7 @@ TcPlan plan_tc(const dd_scan *scan, const ddk::GridDesc &grid, const std::vector
     const int n_t = (int)tdim.size();
     tp.K2.assign(n_t, 0);
     tp.K.assign(n_t, 0);
-    // tiles of 128 x 128 points: only grids that fill them reasonably
-    if (grid.W < ddk::kTcTile / 2 || grid.H < ddk::kTcTile / 2 || scan->n == 0) return tp;
+    if (grid.W < kSplitMinSide || grid.H < kSplitMinSide || scan->n == 0) return tp;
     const double ip = 1.0 / scan->pitch;
     const double xa = grid.x0 * ip, xb = (grid.x0 + (double)(grid.W - 1) * grid.dx) * ip;
     const double ya = grid.y0 * ip, yb = (grid.y0 + (double)(grid.H - 1) * grid.dy) * ip;
@@ -299,56 +284,15 @@ TcPlan plan_tc(const dd_scan *scan, const ddk::GridDesc &grid, const std::vector
         any += tp.K[k];
     }
     if (any == 0) return tp;
-    tp.n_tile_cols = (grid.W + ddk::kTcTile - 1) / ddk::kTcTile;
-    tp.n_tiles = tp.n_tile_cols * ((grid.H + ddk::kTcTile - 1) / ddk::kTcTile);
     tp.on = true;
     return tp;
 }
 
-// dynamic shared memory above 48 KB and the whole L1/shared array as shared memory, set
-// once per device
-template <int kDeg>
-cudaError_t prepare_tc_kernel() {
-    static std::atomic<uint64_t> done{0};
-    int dev = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err != cudaSuccess || dev >= 64) return err;
-    if (done.load() & (uint64_t(1) << dev)) return cudaSuccess;
-    err = cudaFuncSetAttribute(ddk::field_grid_tc_kernel<kDeg>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               ddk::TcConst<kDeg>::kSmemBytes);
-    if (err == cudaSuccess)
-        err = cudaFuncSetAttribute(ddk::field_grid_tc_kernel<kDeg>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                   (int)cudaSharedmemCarveoutMaxShared);
-    if (err == cudaSuccess) done.fetch_or(uint64_t(1) << dev);
-    return err;
-}
-
-// Tensor-core CTAs of the degree-kDeg kernel resident on the whole device at once (their
-// shared memory and tensor memory bound it per SM; 0 if unknown).
-template <int kDeg>
-int64_t tc_resident_ctas() {
-    static std::atomic<int64_t> cached[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 0;
-    int64_t v = cached[dev].load();
-    if (v > 0) return v;
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    v = (int64_t)ddk::TcShape<kDeg>::kCtasPerSm * sms;
-    cached[dev].store(v);
-    return v;
-}
-
-// The tensor-core contraction runs on a side stream of the calling thread, forked from the
-// caller's stream after the coefficients and joined back before the reduce, so that its CTAs
-// fill the SMs the CUDA-core tile kernel leaves idle.  One stream and two events per
+// The contraction's second launch runs on a side stream of the calling thread, forked from the
+// caller's stream after the coefficients and joined back before the final kernel, so that its
+// CTAs start as the first launch's leave their SMs.  One stream and two events per
 // (thread, device), created on first use (reusing an event is safe: a wait takes the state
 // of the event's latest record when it is issued).
-constexpr bool kTcBeforeCore = false;        // submission order of the two grid kernels
-constexpr bool kTcHighPriority = false;      // the side stream's priority (else the lowest)
 struct SideStream {
     cudaStream_t s = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
@@ -363,35 +307,13 @@ cudaError_t side_stream(SideStream **out) {
     if (!ss.s) {
         int lo = 0, hi = 0;
         if ((err = cudaDeviceGetStreamPriorityRange(&lo, &hi)) != cudaSuccess) return err;
-        if ((err = cudaStreamCreateWithPriority(&ss.s, cudaStreamNonBlocking, kTcHighPriority ? hi : lo)) != cudaSuccess)
+        if ((err = cudaStreamCreateWithPriority(&ss.s, cudaStreamNonBlocking, lo)) != cudaSuccess)
             return err;
         if ((err = cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming)) != cudaSuccess) return err;
         if ((err = cudaEventCreateWithFlags(&ss.join, cudaEventDisableTiming)) != cudaSuccess) return err;
     }
     *out = &ss;
     return cudaSuccess;
-}
-
-// Pieces of each snapshot's visit range [lo[j], hi[j]) for one launch over snapshots
-// [g0, g0 + ng): about one work item per resident CTA (every item the same number of 16-visit
-// stages, give or take the rounding), so that the launch is one wave and each CTA writes one
-// partial row per item; and no piece longer than kTcMaxItemStages stages (the accumulation's
-// error budget).
-std::vector<int> tc_pieces(const std::vector<int> &lo, const std::vector<int> &hi, int64_t n_tiles, int g0, int ng,
-                           int64_t slots) {
-    std::vector<int> pieces(ng, 0);
-    auto stages = [&](int j) { return (int64_t)((hi[g0 + j] - lo[g0 + j] + ddk::kTcStage - 1) / ddk::kTcStage); };
-    int64_t total = 0;
-    for (int j = 0; j < ng; ++j) total += stages(j) * n_tiles;
-    if (total == 0) return pieces;
-    const int64_t per = std::max<int64_t>(1, (total + std::max<int64_t>(slots, 1) - 1) / std::max<int64_t>(slots, 1));
-    for (int j = 0; j < ng; ++j) {
-        const int64_t S = stages(j);
-        if (S > 0) pieces[j] = (int)std::max<int64_t>(1, (S * n_tiles + per / 2) / per / std::max<int64_t>(n_tiles, 1));
-        if (S > 0) pieces[j] = (int)std::min<int64_t>(std::max<int64_t>({(int64_t)pieces[j], 1,
-                                                                        (S + ddk::kTcMaxItemStages - 1) / ddk::kTcMaxItemStages}), S);
-    }
-    return pieces;
 }
 
 // Snapshots in time order: order[k] = index into times of the k-th earliest, tdim[k] its time
@@ -448,13 +370,6 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
     std::vector<double> tdim;
     int64_t M = 0;
     const bool lattice = snapshot_dims(scan, times, order, tdim, nact, M);
-    // the degree-2 prefixes that the tensor-core contraction takes (grid tiles only)
-    TcPlan tp;
-    tp.K2.assign(n_t, 0);
-    tp.K.assign(n_t, 0);
-    if (grid_tiles) tp = plan_tc(scan, grid, tdim, nact);
-    const std::vector<int> zeros(n_t, 0);
-
     // visit block size and snapshot groups bound the partial and record buffers
     const int tile = Cfg::kThreads * Cfg::kPPT;
     // grid tiles: 128 columns x 4 rows (kThreads x kPPT); otherwise 512 consecutive points
@@ -470,9 +385,7 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
     // larger blocks only while the FP32 stage sums stay short (<= 32 stages)
     while ((size_t)((n_src + sb - 1) / sb) * group * ((n_pts + 3) / 4 * 4) * sizeof(typename Cfg::Real) > budget && sb < 32 * Cfg::kSTILE) sb *= 2;
     // smaller blocks (down to 128 visits, 64 for grid tiles) while one launch has fewer than
-    // 4 waves of resident CTAs, so that the last wave's stragglers cost little (on a grid the
-    // tile kernel takes only the visits the tensor-core contraction leaves, and 64-visit
-    // blocks measured 3 % faster there)
+    // 4 waves of resident CTAs, so that the last wave's stragglers cost little
     {
         constexpr int kWaves = 4;
         const int64_t waves4 = kWaves * (grid_tiles ? resident_ctas<Cfg, true>() : resident_ctas<Cfg>());
@@ -480,12 +393,9 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
         auto items_per_launch = [&](int b) {
             int64_t blocks = 0;
             for (int j0 = 0; j0 < n_t; j0 += Cfg::kTCH) {
-                int cmax = 0, kmin = INT_MAX;
-                for (int j = j0; j < std::min(n_t, j0 + Cfg::kTCH); ++j) {
-                    cmax = std::max(cmax, nact[j]);
-                    kmin = std::min(kmin, tp.K[j] / b);
-                }
-                blocks += std::max(0, (cmax + b - 1) / b - kmin);
+                int cmax = 0;
+                for (int j = j0; j < std::min(n_t, j0 + Cfg::kTCH); ++j) cmax = std::max(cmax, nact[j]);
+                blocks += (cmax + b - 1) / b;
             }
             return blocks * n_tiles / std::max(1, n_groups);
         };
@@ -496,33 +406,8 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
     }
     const int nblk_max = (int)((n_src + sb - 1) / sb);
     const int n_chunks_max = (group + Cfg::kTCH - 1) / Cfg::kTCH;
-    // tensor-core chunks: rows of partial sums per snapshot and work items per group, within
-    // the partial-sum budget (else the CUDA-core tile takes every visit)
-    int64_t trows_max = 0, n_titems_max = 0;
-    const int64_t tc_slots2 = tp.on ? std::max<int64_t>(1, tc_resident_ctas<2>()) : 1;
-    const int64_t tc_slots4 = tp.on ? std::max<int64_t>(1, tc_resident_ctas<4>()) : 1;
-    if (tp.on) {
-        for (int g0 = 0; g0 < n_t; g0 += group) {
-            const int ng = std::min(group, n_t - g0);
-            const std::vector<int> p2 = tc_pieces(zeros, tp.K2, tp.n_tiles, g0, ng, tc_slots2);
-            const std::vector<int> p4 = tc_pieces(tp.K2, tp.K, tp.n_tiles, g0, ng, tc_slots4);
-            int64_t rows = 0;
-            for (int j = 0; j < ng; ++j) rows += p2[j] + p4[j];
-            trows_max = std::max(trows_max, rows);
-            n_titems_max = std::max(n_titems_max, rows * tp.n_tiles);
-        }
-        if ((size_t)trows_max * ((n_pts + 3) / 4 * 4) * sizeof(float) > budget || n_titems_max > (int64_t(1) << 24)) {
-            tp.on = false;
-            std::fill(tp.K2.begin(), tp.K2.end(), 0);
-            std::fill(tp.K.begin(), tp.K.end(), 0);
-            trows_max = 0;
-            n_titems_max = 0;
-        }
-    }
-
     const int64_t n_rec = lattice ? M + 1 : (int64_t)group * n_src;
-    const size_t ws_bytes = workspace_bytes<Cfg>(n_pts, n_src, group, sb, out_copy, pts_copy, n_t, n_rec, trows_max,
-                                                 n_titems_max);
+    const size_t ws_bytes = workspace_bytes<Cfg>(n_pts, n_src, group, sb, out_copy, pts_copy, n_t, n_rec);
     dd_status st = DD_OK;
     const double *src = dd::device_sources(scan, stream, &st);
     if (!src) return st;
@@ -548,21 +433,15 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
     double *Y = X + n_pts;
     float4 *PF = cv.take<float4>((size_t)n_pts);
     double *d_t = cv.take<double>(group);
-    int *d_nact = cv.take<int>(7 * (size_t)group);
+    int *d_nact = cv.take<int>(3 * (size_t)group);
     int *d_row = d_nact + group;
     int *d_nblk = d_row + group;
-    int *d_kst = d_nblk + group;
-    int *d_kb0 = d_kst + group;
-    int *d_nq = d_kb0 + group;
-    int *d_trow0 = d_nq + group;
     int64_t *d_roff = cv.take<int64_t>(group);
     int2 *d_desc = cv.take<int2>((size_t)n_chunks_max * nblk_max);
-    ddk::TcItem *d_titems = cv.take<ddk::TcItem>((size_t)n_titems_max);
     Rec *d_rec = cv.take<Rec>((size_t)n_rec);
     using Part = typename Cfg::Real;
     const int64_t pstride = (n_pts + 3) / 4 * 4;            // 16-byte aligned partial rows
     Part *d_part = cv.take<Part>((size_t)nblk_max * group * pstride);
-    float *d_tpart = cv.take<float>((size_t)trows_max * pstride);
 
     if (!lattice) {
         DD_PROFILED("prep_points", stream,
@@ -586,10 +465,7 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
     for (int g0 = 0; g0 < n_t; g0 += group) {
         const int ng = std::min(group, n_t - g0);
         const int n_chunks = (ng + Cfg::kTCH - 1) / Cfg::kTCH;
-        std::vector<int> tabs(7 * (size_t)ng);
-        // tensor-core pieces: of the degree-2 prefix [0, K2) and of the degree-4 band [K2, K)
-        const std::vector<int> tp2 = tp.on ? tc_pieces(zeros, tp.K2, tp.n_tiles, g0, ng, tc_slots2) : std::vector<int>(ng, 0);
-        const std::vector<int> tp4 = tp.on ? tc_pieces(tp.K2, tp.K, tp.n_tiles, g0, ng, tc_slots4) : std::vector<int>(ng, 0);
+        std::vector<int> tabs(3 * (size_t)ng);
         std::vector<double> tg(ng);
         std::vector<int64_t> roff(ng);
         int max_nact = 0;
@@ -597,63 +473,27 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
             tg[j] = tdim[g0 + j];
             tabs[j] = nact[g0 + j];
             tabs[ng + j] = order[g0 + j];
-            tabs[3 * ng + j] = tp.K[g0 + j];                               // kst
-            tabs[4 * ng + j] = tp.K[g0 + j] / sb;                          // kb0
-            tabs[5 * ng + j] = tp2[j] + tp4[j];                            // nq
-            tabs[6 * ng + j] = j > 0 ? tabs[6 * ng + j - 1] + tabs[5 * ng + j - 1] : 0;   // trow0
             max_nact = std::max(max_nact, nact[g0 + j]);
             // lattice: snapshot t reads lag t - i at rev[M - t + i]; otherwise row j of the
             // per-(snapshot, visit) records
             roff[j] = lattice ? (tdim[g0 + j] > 0 ? M - (int64_t)tdim[g0 + j] : M) : (int64_t)j * n_src;
         }
         // work items: (tile, chunk, block) for every block below the chunk's largest
-        // n_active (from the first block that holds a visit past some snapshot's
-        // tensor-core prefix), longest first.  Every tile of a (chunk, block) costs the
+        // n_active, longest first.  Every tile of a (chunk, block) costs the
         // same, so the (chunk, block) descriptors are sorted (stable: ties keep chunk, block
         // order) and the kernel expands each into its tiles in tile order.
         std::vector<std::pair<int64_t, int2>> blocks;
         for (int c = 0; c < n_chunks; ++c) {
             const int j0 = c * Cfg::kTCH, j1 = std::min(ng, j0 + Cfg::kTCH);
-            int cmax = 0, kbmin = INT_MAX;
-            for (int j = j0; j < j1; ++j) {
-                cmax = std::max(cmax, nact[g0 + j]);
-                kbmin = std::min(kbmin, tp.K[g0 + j] / sb);
-            }
+            int cmax = 0;
+            for (int j = j0; j < j1; ++j) cmax = std::max(cmax, nact[g0 + j]);
             const int nb = (cmax + sb - 1) / sb;
             for (int j = j0; j < j1; ++j) tabs[2 * ng + j] = nb;
-            for (int k = kbmin; k < nb; ++k) {
+            for (int k = 0; k < nb; ++k) {
                 int64_t cost = 0;
-                for (int j = j0; j < j1; ++j)
-                    cost += std::max(0, std::min(nact[g0 + j], (k + 1) * sb) - std::max(k * sb, tp.K[g0 + j]));
+                for (int j = j0; j < j1; ++j) cost += std::max(0, std::min(nact[g0 + j], (k + 1) * sb) - k * sb);
                 blocks.push_back({cost, make_int2(c, k)});
             }
-        }
-        // tensor-core items: piece p of a snapshot's range [lo, hi) (stages [p S / P,
-        // (p + 1) S / P) of its S 16-visit stages) on each tile; degree-2 items (partial rows
-        // trow0[j] + p) then degree-4 items (rows trow0[j] + P2 + p), each list longest first
-        std::vector<ddk::TcItem> titems;
-        size_t n_t2 = 0;
-        if (tp.on) {
-            auto add_items = [&](const std::vector<int> &lo, const std::vector<int> &hi, const std::vector<int> &pc,
-                                 bool deg4) {
-                const size_t first = titems.size();
-                for (int j = 0; j < ng; ++j) {
-                    const int v0 = lo[g0 + j], P = pc[j];
-                    const int64_t S = (hi[g0 + j] - v0 + ddk::kTcStage - 1) / ddk::kTcStage;
-                    for (int p = 0; p < P; ++p) {
-                        const int vb = v0 + (int)(S * p / P) * ddk::kTcStage;
-                        const int ve = std::min(hi[g0 + j], v0 + (int)(S * (p + 1) / P) * ddk::kTcStage);
-                        const int row = tabs[6 * ng + j] + (deg4 ? tp2[j] : 0) + p;
-                        for (int64_t t = 0; t < tp.n_tiles; ++t) titems.push_back({vb, ve, (int)t, row, roff[j], 0, 0});
-                    }
-                }
-                std::stable_sort(titems.begin() + first, titems.end(), [](const ddk::TcItem &a, const ddk::TcItem &b) {
-                    return a.v_end - a.v_begin > b.v_end - b.v_begin;
-                });
-            };
-            add_items(zeros, tp.K2, tp2, false);
-            n_t2 = titems.size();
-            add_items(tp.K2, tp.K, tp4, true);
         }
         std::stable_sort(blocks.begin(), blocks.end(),
                          [](const std::pair<int64_t, int2> &a, const std::pair<int64_t, int2> &b) { return a.first > b.first; });
@@ -661,19 +501,15 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
         for (size_t q = 0; q < blocks.size(); ++q) it[q] = blocks[q].second;
 
         // the group's tables in one copy: a host image of the device span d_t .. the end of
-        // the descriptors (of the tensor-core items, if any)
+        // the descriptors
         {
             char *const d0 = reinterpret_cast<char *>(d_t);
-            const size_t span = titems.empty() ? reinterpret_cast<char *>(d_desc + it.size()) - d0
-                                               : reinterpret_cast<char *>(d_titems + titems.size()) - d0;
+            const size_t span = reinterpret_cast<char *>(d_desc + it.size()) - d0;
             std::vector<char> img(span);
             std::memcpy(img.data(), tg.data(), ng * sizeof(double));
-            std::memcpy(img.data() + (reinterpret_cast<char *>(d_nact) - d0), tabs.data(), 7 * (size_t)ng * sizeof(int));
+            std::memcpy(img.data() + (reinterpret_cast<char *>(d_nact) - d0), tabs.data(), 3 * (size_t)ng * sizeof(int));
             std::memcpy(img.data() + (reinterpret_cast<char *>(d_roff) - d0), roff.data(), ng * sizeof(int64_t));
             std::memcpy(img.data() + (reinterpret_cast<char *>(d_desc) - d0), it.data(), it.size() * sizeof(int2));
-            if (!titems.empty())
-                std::memcpy(img.data() + (reinterpret_cast<char *>(d_titems) - d0), titems.data(),
-                            titems.size() * sizeof(ddk::TcItem));
             DD_CUDA_TRY(keep->staging.upload(d0, img.data(), span, stream));
             keep->images.push_back(std::move(img));
         }
@@ -683,47 +519,6 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
                         (ddk::coef_kernel<Rec><<<cg, 128, 0, stream>>>(srcT, srcTAU, d_t, d_nact, scan->s, scan->kappa, d_rec, n_src)));
             DD_CUDA_TRY(cudaGetLastError());
         }
-        // the tensor-core contraction's fork point: after the coefficients
-        SideStream *side = nullptr;
-        if (kMixed && !titems.empty()) {
-            DD_CUDA_TRY(side_stream(&side));
-            DD_CUDA_TRY(cudaEventRecord(side->fork, stream));
-        }
-        // the contraction on the side stream (after the CUDA-core tile kernel is submitted,
-        // so that the latter's CTAs are placed first and the contraction's fill what they leave)
-        auto launch_tc = [&]() -> cudaError_t {
-            if constexpr (kMixed) {
-                if (side) {
-                    cudaError_t e = cudaStreamWaitEvent(side->s, side->fork, 0);
-                    if (e != cudaSuccess) return e;
-                    // DD_FAULT=field_tc_wait (tests): no MMA is issued, so the completion waits
-                    // run out and the kernel reports it (dd_field_check)
-                    const int withhold = dd::fault_injected("field_tc_wait") ? 1 : 0;
-                    // persistent CTAs: as many as are resident at once, at most one per item
-                    auto launch = [&](auto deg, const ddk::TcItem *items, size_t n_items, int64_t resident,
-                                      const char *name) -> cudaError_t {
-                        constexpr int kDeg = decltype(deg)::value;
-                        if (n_items == 0) return cudaSuccess;
-                        cudaError_t e2 = prepare_tc_kernel<kDeg>();
-                        if (e2 != cudaSuccess) return e2;
-                        const unsigned n_cta = (unsigned)std::min<int64_t>((int64_t)n_items, resident);
-                        DD_PROFILED(name, side->s,
-                                    (ddk::field_grid_tc_kernel<kDeg><<<n_cta, ddk::kTcThreads, ddk::TcConst<kDeg>::kSmemBytes, side->s>>>(
-                                        ddk::TcScan{grid.W, grid.H, tp.n_tile_cols, srcF, PF, d_tpart, pstride}, nullptr,
-                                        d_rec, items, (int)n_items, withhold)));
-                        return cudaGetLastError();
-                    };
-                    if ((e = launch(std::integral_constant<int, 2>(), d_titems, n_t2, tc_slots2, "field_grid_tc")) != cudaSuccess)
-                        return e;
-                    if ((e = launch(std::integral_constant<int, 4>(), d_titems + n_t2, titems.size() - n_t2, tc_slots4,
-                                    "field_grid_tc4")) != cudaSuccess)
-                        return e;
-                    if ((e = cudaEventRecord(side->join, side->s)) != cudaSuccess) return e;
-                }
-            }
-            return cudaSuccess;
-        };
-        if (kTcBeforeCore) DD_CUDA_TRY(launch_tc());
         if (!it.empty()) {
             if (grid_tiles) DD_CUDA_TRY((prefer_shared<Cfg, true>()));
             else DD_CUDA_TRY(prefer_shared<Cfg>());
@@ -735,7 +530,7 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
                     if (grid_tiles) {
                         DD_PROFILED("field_grid_mixed", stream,
                                     (ddk::field_grid_kernel<GridCfg><<<nctas, Cfg::kThreads, 0, stream>>>(
-                                        grid.W, grid.H, n_tc, d_rec, d_roff, d_nact, tp.on ? d_kst : nullptr, d_desc,
+                                        grid.W, grid.H, n_tc, d_rec, d_roff, d_nact, d_desc,
                                         n_tiles, item0, ng, sb, d_part, pstride, srcF, PF)));
                         DD_CUDA_TRY(cudaGetLastError());
                         continue;
@@ -748,13 +543,10 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
                 DD_CUDA_TRY(cudaGetLastError());
             }
         }
-        if (!kTcBeforeCore) DD_CUDA_TRY(launch_tc());
-        if (side) DD_CUDA_TRY(cudaStreamWaitEvent(stream, side->join, 0));
         dim3 rg((unsigned)((n_pts + 1023) / 1024), (unsigned)ng);
         DD_PROFILED("field_reduce", stream,
                     (ddk::reduce_kernel<Part><<<rg, 256, 0, stream>>>(
-                        d_part, d_nblk, tp.on ? d_kb0 : nullptr, reinterpret_cast<const Part *>(d_tpart),
-                        tp.on ? d_nq : nullptr, d_trow0, d_row, ng, n_pts, pstride, scan->pref, out_dev)));
+                        d_part, d_nblk, d_row, ng, n_pts, pstride, scan->pref, out_dev)));
         DD_CUDA_TRY(cudaGetLastError());
         keep->items.push_back(std::move(it));
         keep->ints.push_back(std::move(tabs));
@@ -766,6 +558,85 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
     DD_CUDA_TRY(dd::workspace_release(ws, stream));
     DD_CUDA_TRY(dd::defer_release(stream, keep, HostTables::release));
     if (dd::host_sync_needed(stream, {pts_kind, out_kind})) DD_CUDA_TRY(cudaStreamSynchronize(stream));
+    return DD_OK;
+}
+
+// FP32-mixed grids of at least this many columns, rows and points take the contraction
+// (dd_grid.cu); thinner ones leave most of its 128-row tiles empty and take the CUDA-core grid
+// tile.
+constexpr int64_t kQuadMinSide = 32, kQuadMinPts = 4096, kQuadMaxSide = int64_t(1) << 30;
+
+dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const std::vector<double> &times, double *out,
+                         cudaStream_t stream) {
+    const int n_t = (int)times.size();
+    const int64_t n_pts = grid.W * grid.H;
+    const dd::MemKind out_kind = dd::memory_kind(out);
+    const bool out_copy = out_kind != dd::MemKind::Device;
+    std::vector<int> order, nact;
+    std::vector<double> tdim;
+    int64_t M = 0;
+    const bool lattice = snapshot_dims(scan, times, order, tdim, nact, M);
+    const dd::GridBox box{grid.x0, grid.y0, grid.dx, grid.dy, grid.W, grid.H};
+    dd_status st = DD_OK;
+    const double *src = dd::device_sources(scan, stream, &st);
+    if (!src) return st;
+    const dd::ScanUse use{scan, stream};
+    const float4 *srcF = dd::device_sources_ff(scan, stream, &st);
+    // snapshots per pass: rows of k (off the lattice, a table per snapshot) and partial rows
+    // within about 1 GiB
+    int group = std::min(n_t, 4096);
+    while (group > 1 && (double)group * ((lattice ? 0.0 : 48.0 * (double)scan->n) + 16.0 * (double)n_pts) > (double)(int64_t(1) << 30))
+        group = (group + 1) / 2;
+    double *out_dev = out;
+    void *out_ws = nullptr;
+    auto no_memory = [](cudaError_t err) {
+        cudaGetLastError();
+        return dd::fail(err == cudaErrorMemoryAllocation ? DD_ENOMEM : DD_ECUDA,
+                        std::string("field workspace allocation: ") + cudaGetErrorString(err));
+    };
+    if (out_copy) {
+        const cudaError_t err = dd::workspace_alloc(&out_ws, (size_t)n_t * n_pts * sizeof(double), stream);
+        if (err != cudaSuccess) return no_memory(err);
+        out_dev = static_cast<double *>(out_ws);
+    }
+    auto *keep = new HostTables();
+    for (int g0 = 0; g0 < n_t; g0 += group) {
+        const int ng = std::min(group, n_t - g0);
+        dd::GridEngine eng;
+        const int gi = eng.add_grid(scan, box);
+        const int lag = lattice ? eng.add_lag_table(scan, box, M) : -1;
+        for (int j = g0; j < g0 + ng; ++j) {
+            // on the lattice, snapshot t sees visit v at lag t - v: table visit M - t + v
+            const int table = lattice ? lag : eng.add_table(scan, box, src, tdim[j], nact[j]);
+            const int shift = lattice ? (int)(tdim[j] > 0 ? M - (int64_t)tdim[j] : M) : 0;
+            eng.add_job(scan, srcF, gi, table, nact[j], shift, (int64_t)order[j] * n_pts);
+        }
+        DD_CUDA_TRY(eng.finish(true));
+        void *ws = nullptr;
+        const cudaError_t err = dd::fault_injected("alloc") ? cudaErrorMemoryAllocation
+                                                            : dd::workspace_alloc(&ws, eng.workspace_bytes(), stream);
+        if (err != cudaSuccess) {
+            dd::defer_release(stream, keep, HostTables::release);   // earlier groups may be in flight
+            if (out_ws) dd::workspace_release(out_ws, stream);
+            return no_memory(err);
+        }
+        eng.bind(ws);
+        keep->images.emplace_back(eng.table_bytes());
+        eng.write_tables(keep->images.back().data());
+        DD_CUDA_TRY(keep->staging.upload(ws, keep->images.back().data(), keep->images.back().size(), stream));
+        SideStream *side = nullptr;
+        DD_CUDA_TRY(side_stream(&side));
+        // DD_FAULT=field_tc_wait (tests): no MMA is issued, so the completion waits run out and
+        // the kernel reports it (dd_field_check)
+        DD_CUDA_TRY(eng.enqueue(out_dev, stream, side->s, side->fork, side->join, dd::fault_injected("field_tc_wait"), true));
+        DD_CUDA_TRY(dd::workspace_release(ws, stream));
+    }
+    if (out_copy) {
+        DD_CUDA_TRY(cudaMemcpyAsync(out, out_dev, (size_t)n_t * n_pts * sizeof(double), cudaMemcpyDeviceToHost, stream));
+        DD_CUDA_TRY(dd::workspace_release(out_ws, stream));
+    }
+    DD_CUDA_TRY(dd::defer_release(stream, keep, HostTables::release));
+    if (dd::host_sync_needed(stream, {out_kind})) DD_CUDA_TRY(cudaStreamSynchronize(stream));
     return DD_OK;
 }
 
@@ -824,6 +695,8 @@ extern "C" dd_status dd_field_on_grid(const dd_scan *scan, double x0_m, double y
     ddk::GridDesc g;
     g.x0 = x0_m; g.y0 = y0_m; g.dx = dx_m; g.dy = dy_m; g.W = n_cols; g.H = n_rows;
     const int64_t n_pts = n_cols * n_rows;
+    if (prec == DD_MIXED && std::min(n_cols, n_rows) >= kQuadMinSide && n_pts >= kQuadMinPts && std::max(n_cols, n_rows) < kQuadMaxSide)
+        return run_grid_mixed(scan, g, times, out, stream);
     if (prec == DD_MIXED) return run_field<ddk::CfgMixed>(scan, nullptr, n_pts, g, times, out, stream);
     return run_field<ddk::CfgF64>(scan, nullptr, n_pts, g, times, out, stream);
 }
@@ -831,50 +704,11 @@ extern "C" dd_status dd_field_on_grid(const dd_scan *scan, double x0_m, double y
 extern "C" dd_status dd_field_check(void) {
     dd::clear_error();
     DD_CUDA_TRY(cudaDeviceSynchronize());
-    int flag = 0;
-    DD_CUDA_TRY(cudaMemcpyFromSymbol(&flag, ddk::g_field_tc_timeout, sizeof(int)));
-    if (!flag) return DD_OK;
-    const int zero = 0;
-    DD_CUDA_TRY(cudaMemcpyToSymbol(ddk::g_field_tc_timeout, &zero, sizeof(int)));
+    bool timed_out = false;
+    DD_CUDA_TRY(dd::grid_engine_timed_out(&timed_out));
+    if (!timed_out) return DD_OK;
     return dd::fail(DD_ETIMEOUT, "dd_field_check: a tensor-core contraction of the grid field gave up waiting for its MMAs");
 }
-
-namespace dd {
-
-void tc_prefixes(const dd_scan *scan, double x0, double y0, double dx, double dy, int64_t W, int64_t H, double tdim,
-                 int nact, int *K2, int *K) {
-    *K2 = *K = 0;
-    if (W <= 0 || H <= 0 || nact <= 0) return;
-    ddk::GridDesc g;
-    g.x0 = x0; g.y0 = y0; g.dx = dx; g.dy = dy; g.W = W; g.H = H;
-    const TcPlan tp = plan_tc(scan, g, std::vector<double>{tdim}, std::vector<int>{nact});
-    if (!tp.on) return;
-    *K2 = tp.K2[0];
-    *K = tp.K[0];
-}
-
-cudaError_t prepare_field_tc() {
-    cudaError_t err = prepare_tc_kernel<2>();
-    return err == cudaSuccess ? prepare_tc_kernel<4>() : err;
-}
-
-int64_t field_tc_resident(int deg) { return deg == 2 ? tc_resident_ctas<2>() : tc_resident_ctas<4>(); }
-
-cudaError_t launch_field_tc(int deg, const ddk::TcScan *scans, const ddk::RecF32 *rec, const ddk::TcItem *items,
-                            int n_items, int n_ctas, cudaStream_t stream) {
-    if (n_items <= 0) return cudaSuccess;
-    // (no profiling scope: batch plans capture this launch into a CUDA graph)
-    const ddk::TcScan none{};
-    if (deg == 2)
-        ddk::field_grid_tc_kernel<2><<<(unsigned)n_ctas, ddk::kTcThreads, ddk::TcConst<2>::kSmemBytes, stream>>>(
-            none, scans, rec, items, n_items, 0);
-    else
-        ddk::field_grid_tc_kernel<4><<<(unsigned)n_ctas, ddk::kTcThreads, ddk::TcConst<4>::kSmemBytes, stream>>>(
-            none, scans, rec, items, n_items, 0);
-    return cudaGetLastError();
-}
-
-}  // namespace dd
 
 extern "C" dd_status dd_field_grid_split(const dd_scan *scan, double x0_m, double y0_m, double dx_m, double dy_m,
                                          int64_t n_cols, int64_t n_rows, const double *times_s, int64_t n_t,

@@ -1,0 +1,361 @@
+// dd_grid.cu -- the FP32-mixed field on grids of points: visits in bands of Gauss-Legendre nodes
+// on the tensor cores, the last few on the CUDA cores (dd_grid_quad.cuh), for one scan's
+// snapshots (dd_field_on_grid) or a batch of scans (dd_batch_create_grid).
+//
+// Launches: prep (axes, rows of k, records of the recent visits), the contraction, and the final
+// kernel (recent visits, partial rows, prefactor).
+#include "dd_grid.h"
+
+#include <algorithm>
+#include <atomic>
+#include <cmath>
+#include <cstring>
+#include <queue>
+#include <utility>
+
+#include "dd_grid_quad.cuh"
+
+namespace {
+
+using ddk::kGqBands;
+using ddk::kGqNodes;
+
+// Ages (in dwells) from which every visit of the scan takes each band at every point of the
+// grid (+inf: none): h = rho^2 dq <= kGqH for rho^2 up to R2, the largest squared distance
+// between the grid's box and the visits' box, r = w1/w0 - 1 <= kGqR, and the dwell over.  With
+// c = 4 kappa tau_max, dq <= c / ((w1 - c) w1) and r <= c / (w1 - c) for every visit (both grow
+// with the dwell at a fixed w1 = 2s + 4 kappa (t - T_i)).
+void band_ages(const dd_scan *scan, const dd::GridBox &g, double (&age)[kGqBands]) {
+    const double ip = 1.0 / scan->pitch;
+    const double xa = g.x0 * ip, xb = (g.x0 + (double)(g.W - 1) * g.dx) * ip;
+    const double ya = g.y0 * ip, yb = (g.y0 + (double)(g.H - 1) * g.dy) * ip;
+    const double ex = std::max(std::max(xa, xb) - scan->x_lo, scan->x_hi - std::min(xa, xb));
+    const double ey = std::max(std::max(ya, yb) - scan->y_lo, scan->y_hi - std::min(ya, yb));
+    // margins for the points' own rounding
+    const double R2 = (ex * ex + ey * ey) * (1.0 + 1e-6) + 1e-6;
+    const double c = 4.0 * scan->kappa * scan->tau_max;
+    double prev = INFINITY;
+    for (int b = 0; b < kGqBands; ++b) {
+        const double dq = ddk::kGqH[b] * (1.0 - 1e-4) / R2;
+        double w1 = 0.5 * (c + std::sqrt(c * c + 4.0 * c / dq));
+        w1 = std::max({w1, c + c / ddk::kGqR[b], 2.0 * scan->s + c}) * (1.0 + 1e-9);
+        const double a = (w1 - 2.0 * scan->s) / (4.0 * scan->kappa) * (1.0 + 1e-9);
+        prev = age[b] = std::isfinite(a) && a > 0.0 ? std::min(prev, a) : INFINITY;
+    }
+}
+
+// Rows of k of the table visits before i.
+int64_t rows_before(const ddk::GqTable &t, int64_t i) {
+    int64_t k = 0;
+    for (int b = 0; b < kGqBands; ++b)
+        k += std::max<int64_t>(0, std::min<int64_t>(i, t.vb[b + 1]) - t.vb[b]) * kGqNodes[b];
+    return k;
+}
+
+int sm_count() {
+    static std::atomic<int> cached[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 1;
+    int v = cached[dev].load();
+    if (v > 0) return v;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) {
+        cudaGetLastError();
+        return 1;
+    }
+    cached[dev].store(v);
+    return v;
+}
+
+cudaError_t prepare_kernel() {
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess || dev >= 64) return err;
+    if (done.load() & (uint64_t(1) << dev)) return cudaSuccess;
+    err = cudaFuncSetAttribute(ddk::grid_quad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ddk::kGqSmemBytes);
+    if (err == cudaSuccess) done.fetch_or(uint64_t(1) << dev);
+    return err;
+}
+
+}  // namespace
+
+namespace dd {
+
+struct GridEngine::Tables {
+    std::vector<ddk::GqGrid> grids;
+    std::vector<ddk::GqTable> tabs;
+    std::vector<ddk::GqJob> jobs;
+    std::vector<ddk::GqRun> runs;                        // CTA by CTA, launch by launch
+    std::vector<int> cta_off;                            // first run of each CTA, per launch n_cta + 1
+    std::vector<int64_t> ax_offs, vis_offs, rec_offs, tile_offs;
+    struct Span { int64_t k0, k1, split; };              // rows of k of a job; from split on: n > 2
+    std::vector<Span> spans;
+    int n_cta[2] = {0, 0};
+    int64_t n_ax = 0, n_vis = 0, n_rows = 0, n_rec = 0, n_part = 0;
+    // device
+    char *base = nullptr;
+    ddk::GqRow *rows = nullptr;
+    ddk::RecF32 *rec = nullptr;
+    float2 *ax = nullptr;
+    float *part = nullptr;
+
+    struct Layout { size_t grids, tabs, jobs, runs, cta, axo, viso, reco, tileo, end; };
+    Layout layout() const {
+        Layout l;
+        size_t b = 0;
+        auto add = [&](size_t n) { const size_t o = b; b = (b + n + 255) & ~size_t(255); return o; };
+        l.grids = add(grids.size() * sizeof(ddk::GqGrid));
+        l.tabs = add(tabs.size() * sizeof(ddk::GqTable));
+        l.jobs = add(jobs.size() * sizeof(ddk::GqJob));
+        l.runs = add(runs.size() * sizeof(ddk::GqRun));
+        l.cta = add(cta_off.size() * sizeof(int));
+        l.axo = add(ax_offs.size() * sizeof(int64_t));
+        l.viso = add(vis_offs.size() * sizeof(int64_t));
+        l.reco = add(rec_offs.size() * sizeof(int64_t));
+        l.tileo = add(tile_offs.size() * sizeof(int64_t));
+        l.end = b;
+        return l;
+    }
+};
+
+GridEngine::GridEngine() : t(new Tables()) {}
+GridEngine::~GridEngine() { delete t; }
+
+int GridEngine::add_grid(const dd_scan *scan, const GridBox &g) {
+    t->grids.push_back({g.x0, g.y0, g.dx, g.dy, 1.0 / scan->pitch, t->n_ax, (int)g.W, (int)g.H});
+    t->ax_offs.push_back(t->n_ax);
+    t->n_ax += g.W + g.H;
+    return (int)t->grids.size() - 1;
+}
+
+int GridEngine::add_table(const dd_scan *scan, const GridBox &g, const double *src, double tdim, int nact) {
+    double age[kGqBands];
+    band_ages(scan, g, age);
+    ddk::GqTable tb{src + 2 * scan->n, src + 3 * scan->n, scan->s, scan->kappa, tdim, t->n_vis, t->n_rows, t->n_rec, nact, 0, {}};
+    tb.vb[0] = 0;
+    for (int b = 0; b < kGqBands; ++b) {
+        const int64_t k = std::upper_bound(scan->T.begin(), scan->T.end(), tdim - age[b]) - scan->T.begin();
+        tb.vb[b + 1] = std::max(tb.vb[b], (int)std::min<int64_t>(k, nact));
+    }
+    t->tabs.push_back(tb);
+    t->vis_offs.push_back(t->n_vis);
+    t->rec_offs.push_back(t->n_rec);
+    t->n_vis += nact;
+    t->n_rows += rows_before(tb, nact);
+    t->n_rec += nact - tb.vb[kGqBands];
+    return (int)t->tabs.size() - 1;
+}
+
+int GridEngine::add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M) {
+    double age[kGqBands];
+    band_ages(scan, g, age);
+    ddk::GqTable tb{nullptr, nullptr, scan->s, scan->kappa, 0.0, t->n_vis, t->n_rows, t->n_rec, (int)M, 0, {}};
+    tb.vb[0] = 0;
+    for (int b = 0; b < kGqBands; ++b) {
+        const double last = std::floor((double)M - age[b]);             // lag M - i >= age
+        tb.vb[b + 1] = last >= 0.0 ? std::max(tb.vb[b], (int)std::min((double)M, last + 1.0)) : tb.vb[b];
+    }
+    t->tabs.push_back(tb);
+    t->vis_offs.push_back(t->n_vis);
+    t->rec_offs.push_back(t->n_rec);
+    t->n_vis += M;
+    t->n_rows += rows_before(tb, M);
+    t->n_rec += M - tb.vb[kGqBands];
+    return (int)t->tabs.size() - 1;
+}
+
+void GridEngine::add_job(const dd_scan *scan, const float4 *srcF, int grid, int table, int nact, int shift,
+                         int64_t out_off) {
+    const ddk::GqGrid &g = t->grids[grid];
+    const ddk::GqTable &tb = t->tabs[table];
+    ddk::GqJob j{};
+    j.srcF = srcF;
+    j.ax_off = g.ax_off;
+    j.W = g.W;
+    j.H = g.H;
+    j.n_tc = (g.W + ddk::kGqTile - 1) / ddk::kGqTile;
+    j.tw = ((g.W + j.n_tc - 1) / j.n_tc + 15) / 16 * 16;               // even widths: less padding
+    j.shift = shift;
+    const int i0 = shift, i1 = shift + nact, kc = std::min(std::max(tb.vb[kGqBands], i0), i1);
+    j.r0 = kc - shift;
+    j.r1 = nact;
+    j.rec0 = tb.rec_off + (kc - tb.vb[kGqBands]);
+    j.t_stride = ((int64_t)g.W * g.H + 3) / 4 * 4;
+    j.out_off = out_off;
+    j.pref = scan->pref;
+    t->jobs.push_back(j);
+    const int mid = std::min(std::max(tb.vb[2], i0), kc);
+    t->spans.push_back({tb.k_off + rows_before(tb, i0), tb.k_off + rows_before(tb, kc), tb.k_off + rows_before(tb, mid)});
+}
+
+cudaError_t GridEngine::finish(bool two_launches) {
+    const int sms = sm_count();
+    t->tile_offs.assign(1, 0);
+    for (const ddk::GqJob &j : t->jobs)
+        t->tile_offs.push_back(t->tile_offs.back() + (int64_t)((j.W + 31) / 32) * ((j.H + ddk::kGqFinRows - 1) / ddk::kGqFinRows));
+    // Cost of a run: its rows of k times the factors formed per row (32 positions at a time),
+    // plus about 500 rows' worth of factors for its start, drain and output.
+    auto row_cost = [](const ddk::GqJob &j, int tile) {
+        const int nc = std::min(j.tw, j.W - (tile % j.n_tc) * j.tw);
+        const int nr = std::min(ddk::kGqTile, j.H - (tile / j.n_tc) * ddk::kGqTile);
+        return (int64_t)((nc + 31) / 32 + (nr + 31) / 32 + 1);
+    };
+    constexpr int64_t kRunCost = 2000;
+    for (int launch = 0; launch < (two_launches ? 2 : 1); ++launch) {
+        auto span = [&](size_t j, int64_t &k0, int64_t &k1) {
+            const Tables::Span &s = t->spans[j];
+            k0 = launch == 0 ? s.k0 : s.split;
+            k1 = launch == 0 && two_launches ? s.split : s.k1;
+        };
+        int64_t total = 0;
+        for (size_t j = 0; j < t->jobs.size(); ++j) {
+            int64_t k0, k1;
+            span(j, k0, k1);
+            const ddk::GqJob &J = t->jobs[j];
+            const int n_tiles = J.n_tc * ((J.H + ddk::kGqTile - 1) / ddk::kGqTile);
+            for (int q = 0; q < n_tiles && k1 > k0; ++q) total += (k1 - k0) * row_cost(J, q);
+        }
+        if (total == 0) continue;
+        // about two runs per CTA, so that dealing them out longest first evens the CTAs' shares
+        const int64_t per = std::max<int64_t>(total / (2 * sms), 2 * kRunCost);
+        std::vector<std::pair<int64_t, ddk::GqRun>> list;
+        for (size_t j = 0; j < t->jobs.size(); ++j) {
+            int64_t k0, k1;
+            span(j, k0, k1);
+            if (k1 <= k0) continue;
+            ddk::GqJob &J = t->jobs[j];
+            const int n_tiles = J.n_tc * ((J.H + ddk::kGqTile - 1) / ddk::kGqTile);
+            // every tile of the job in the same number of pieces (whole partial rows)
+            const int64_t cost = (k1 - k0) * row_cost(J, 0), steps = (k1 - k0 + 15) / 16;
+            const int64_t P = std::min(std::max<int64_t>(1, (cost + per / 2) / per), steps);
+            for (int64_t p = 0; p < P; ++p) {
+                const int64_t a = k0 + steps * p / P * 16, b = std::min(k1, k0 + steps * (p + 1) / P * 16);
+                for (int q = 0; q < n_tiles; ++q)
+                    list.push_back({(b - a) * row_cost(J, q) + kRunCost,
+                                    ddk::GqRun{a, (int)(b - a), (int)j, q, J.nq + (int)p}});
+            }
+            J.nq += (int)P;
+        }
+        std::stable_sort(list.begin(), list.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
+        const int n_cta = (int)std::min<int64_t>(sms, (int64_t)list.size());
+        std::vector<std::vector<int>> of((size_t)n_cta);
+        std::priority_queue<std::pair<int64_t, int>, std::vector<std::pair<int64_t, int>>, std::greater<std::pair<int64_t, int>>> load;
+        for (int c = 0; c < n_cta; ++c) load.push({0, c});
+        for (size_t k = 0; k < list.size(); ++k) {
+            const std::pair<int64_t, int> top = load.top();
+            load.pop();
+            of[(size_t)top.second].push_back((int)k);
+            load.push({top.first + list[k].first, top.second});
+        }
+        t->n_cta[launch] = n_cta;
+        for (int c = 0; c < n_cta; ++c) {
+            t->cta_off.push_back((int)t->runs.size());
+            for (int k : of[(size_t)c]) t->runs.push_back(list[(size_t)k].second);
+        }
+        t->cta_off.push_back((int)t->runs.size());
+    }
+    for (ddk::GqJob &j : t->jobs) {
+        j.t_off = t->n_part;
+        t->n_part += (int64_t)j.nq * j.t_stride;
+    }
+    return t->runs.empty() ? cudaSuccess : prepare_kernel();
+}
+
+size_t GridEngine::table_bytes() const { return t->layout().end; }
+
+size_t GridEngine::workspace_bytes() const {
+    auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
+    return up(table_bytes()) + up((size_t)t->n_rows * sizeof(ddk::GqRow)) + up((size_t)t->n_rec * sizeof(ddk::RecF32)) +
+           up((size_t)t->n_ax * sizeof(float2)) + up((size_t)t->n_part * sizeof(float)) + 256;
+}
+
+void GridEngine::write_tables(char *dst) const {
+    const Tables::Layout l = t->layout();
+    auto put = [&](size_t off, const auto &v) {
+        if (!v.empty()) std::memcpy(dst + off, v.data(), v.size() * sizeof(v[0]));
+    };
+    put(l.grids, t->grids);
+    put(l.tabs, t->tabs);
+    put(l.jobs, t->jobs);
+    put(l.runs, t->runs);
+    put(l.cta, t->cta_off);
+    put(l.axo, t->ax_offs);
+    put(l.viso, t->vis_offs);
+    put(l.reco, t->rec_offs);
+    put(l.tileo, t->tile_offs);
+}
+
+void GridEngine::bind(void *workspace) {
+    char *p = static_cast<char *>(workspace);
+    auto take = [&](size_t b) { char *q = p; p += (b + 255) & ~size_t(255); return q; };
+    t->base = take(table_bytes());
+    t->rows = reinterpret_cast<ddk::GqRow *>(take((size_t)t->n_rows * sizeof(ddk::GqRow)));
+    t->rec = reinterpret_cast<ddk::RecF32 *>(take((size_t)t->n_rec * sizeof(ddk::RecF32)));
+    t->ax = reinterpret_cast<float2 *>(take((size_t)t->n_ax * sizeof(float2)));
+    t->part = reinterpret_cast<float *>(take((size_t)t->n_part * sizeof(float)));
+}
+
+int64_t GridEngine::n_tiles() const { return t->tile_offs.empty() ? 0 : t->tile_offs.back(); }
+int64_t GridEngine::n_runs() const { return (int64_t)t->runs.size(); }
+
+cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t side, cudaEvent_t fork,
+                                cudaEvent_t join, bool withhold, bool profile) {
+    if (t->jobs.empty() || n_tiles() == 0) return cudaSuccess;
+    const Tables::Layout l = t->layout();
+    const ddk::GqJob *jobs = reinterpret_cast<const ddk::GqJob *>(t->base + l.jobs);
+    const ddk::GqRun *runs = reinterpret_cast<const ddk::GqRun *>(t->base + l.runs);
+    const int *cta = reinterpret_cast<const int *>(t->base + l.cta);
+    cudaError_t err;
+    auto scoped = [&](const char *name, cudaStream_t s, auto &&launch) {
+        if (profile) {
+            dd::ProfScope ps(name, s);
+            launch();
+        } else {
+            launch();
+        }
+        return cudaGetLastError();
+    };
+    const int64_t n_prep = ddk::gq_warps(t->n_rec) + ddk::gq_warps(t->n_vis) + t->n_ax;
+    auto offs = [&](size_t o) { return reinterpret_cast<const int64_t *>(t->base + o); };
+    const ddk::GqPrep prep{reinterpret_cast<const ddk::GqTable *>(t->base + l.tabs), offs(l.reco), offs(l.viso), offs(l.axo),
+                           reinterpret_cast<const ddk::GqGrid *>(t->base + l.grids), t->n_rec, t->n_vis, t->n_ax,
+                           (int)t->tabs.size(), (int)t->grids.size(), t->rows, t->rec, t->ax};
+    if ((err = scoped("coef_mixed", stream, [&] {
+             ddk::grid_quad_prep_kernel<<<(unsigned)((n_prep + 63) / 64), 64, 0, stream>>>(prep);
+         })) != cudaSuccess)
+        return err;
+    const bool both = t->n_cta[0] > 0 && t->n_cta[1] > 0 && side != nullptr;
+    if (both) {
+        if ((err = cudaEventRecord(fork, stream)) != cudaSuccess) return err;
+        if ((err = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return err;
+    }
+    auto contraction = [&](int k, const char *name, cudaStream_t s) -> cudaError_t {
+        if (t->n_cta[k] == 0) return cudaSuccess;
+        const int *off = cta + (k == 0 || t->n_cta[0] == 0 ? 0 : t->n_cta[0] + 1);
+        return scoped(name, s, [&] {
+            ddk::grid_quad_kernel<<<(unsigned)t->n_cta[k], ddk::kGqThreads, ddk::kGqSmemBytes, s>>>(
+                jobs, runs, off, t->rows, t->ax, t->part, withhold ? 1 : 0);
+        });
+    };
+    if ((err = contraction(0, "field_grid_tc", stream)) != cudaSuccess) return err;
+    if ((err = contraction(1, "field_grid_tc4", both ? side : stream)) != cudaSuccess) return err;
+    if (both) {
+        if ((err = cudaEventRecord(join, side)) != cudaSuccess) return err;
+        if ((err = cudaStreamWaitEvent(stream, join, 0)) != cudaSuccess) return err;
+    }
+    return scoped("field_grid_mixed", stream, [&] {
+        ddk::grid_quad_final_kernel<<<(unsigned)n_tiles(), ddk::kGqFinThreads, 0, stream>>>(
+            jobs, reinterpret_cast<const int64_t *>(t->base + l.tileo), (int)t->jobs.size(), t->rec, t->ax, t->part, out);
+    });
+}
+
+cudaError_t grid_engine_timed_out(bool *timed_out) {
+    int flag = 0;
+    cudaError_t err = cudaMemcpyFromSymbol(&flag, ddk::g_grid_quad_timeout, sizeof(int));
+    *timed_out = err == cudaSuccess && flag != 0;
+    if (!*timed_out) return err;
+    const int zero = 0;
+    return cudaMemcpyToSymbol(ddk::g_grid_quad_timeout, &zero, sizeof(int));
+}
+
+}  // namespace dd

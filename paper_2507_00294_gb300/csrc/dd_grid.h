@@ -1,0 +1,67 @@
+// dd_grid.h -- host side of the FP32-mixed field on grids of points (dd_grid.cu): the tables,
+// workspace layout and launches of a set of jobs, one job = one snapshot of one scan on one grid.
+// Used per call by dd_field_on_grid and per plan by the grid batches.
+#pragma once
+#include <cstdint>
+#include <vector>
+
+#include <cuda_runtime.h>
+
+#include "dd_internal.h"
+
+namespace ddk {
+struct GqGrid;
+struct GqTable;
+struct GqJob;
+struct GqRun;
+struct GqRow;
+}  // namespace ddk
+
+namespace dd {
+
+// A grid of evaluation points [m].
+struct GridBox {
+    double x0 = 0, y0 = 0, dx = 0, dy = 0;
+    int64_t W = 0, H = 0;
+};
+
+class GridEngine {
+  public:
+    GridEngine();
+    ~GridEngine();
+    GridEngine(const GridEngine &) = delete;
+    GridEngine &operator=(const GridEngine &) = delete;
+
+    // Axes of a grid (W, H < 2^30) in the scan's pitch units; returns its index.
+    int add_grid(const dd_scan *scan, const GridBox &g);
+    // Coefficients of the visits [0, nact) of a scan at tdim (dwells), or of the lags M .. 1 of a
+    // uniform scan; src: the scan's device block.  Returns the table's index.
+    int add_table(const dd_scan *scan, const GridBox &g, const double *src, double tdim, int nact);
+    int add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M);
+    // The scan's snapshot with nact started visits, table visit = visit + shift; its field goes to
+    // out + out_off (W H values).
+    void add_job(const dd_scan *scan, const float4 *srcF, int grid, int table, int nact, int shift, int64_t out_off);
+    // Splits the contraction into runs for the device's SMs: the rows of k of one and two nodes
+    // and the rest as two launches (two_launches), or all in one.
+    cudaError_t finish(bool two_launches);
+
+    size_t table_bytes() const;          // host tables, uploaded to the workspace's first bytes
+    size_t workspace_bytes() const;
+    void write_tables(char *dst) const;
+    void bind(void *workspace);
+    // Launches on `stream`; the second contraction launch goes to `side` (may be NULL), forked and
+    // joined by the two events.  withhold: testing hook of the bounded waits.
+    cudaError_t enqueue(double *out, cudaStream_t stream, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join,
+                        bool withhold, bool profile);
+    int64_t n_tiles() const;             // tiles of the recent visits' kernel
+    int64_t n_runs() const;
+
+  private:
+    struct Tables;
+    Tables *t;
+};
+
+// Whether a contraction gave up waiting since the last call (clears the flag).
+cudaError_t grid_engine_timed_out(bool *timed_out);
+
+}  // namespace dd

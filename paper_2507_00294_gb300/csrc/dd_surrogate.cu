@@ -13,6 +13,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include "dd_internal.h"
@@ -144,10 +145,35 @@ conv3x3_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const fl
 // canonical K-major layout without swizzle: "core matrices" of 8 rows x 16 bytes.
 //   input row [c8][px][8]: pixel rows 16 bytes apart, so the 128 pixels of any tap
 //          (shifted by kx*dil columns) form 16 core matrices 128 bytes apart (SBO), and
-//          the next 8 channels sit one channel-group plane further (LBO = cols*16 bytes);
+//          the next 8 channels sit one channel-group plane further (LBO = plane*16 bytes);
 //   weight [tap][c8][co][8]: SBO 128 bytes (next 8 outputs), LBO Cout*16 bytes.
 constexpr int kTW5 = 128;
 static __device__ int g_tc_timeout;       // set when an MMA completion wait gives up
+
+// Pixels per channel-group plane of a staged row: the row's, padded to 2 mod 8, so that the copies of
+// a pixel's channel groups (consecutive threads, whole sectors of global memory) land in
+// different banks.
+__host__ __device__ constexpr int conv_plane(int dil) { return kTW5 + 2 * dil + (2 - (kTW5 + 2 * dil) % 8 + 8) % 8; }
+
+// 32 bytes in one access (a whole sector; the address a multiple of 32), else in two
+__device__ __forceinline__ void store32(void *p, uint4 a, uint4 b, bool wide) {
+    if (wide) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                     :: "l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
+    } else {
+        reinterpret_cast<uint4 *>(p)[0] = a;
+        reinterpret_cast<uint4 *>(p)[1] = b;
+    }
+}
+__device__ __forceinline__ void load32(const void *p, uint4 &a, uint4 &b, bool wide) {
+    if (wide) {
+        asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
+    } else {
+        a = reinterpret_cast<const uint4 *>(p)[0];
+        b = reinterpret_cast<const uint4 *>(p)[1];
+    }
+}
 
 // 16-byte global -> shared copy that completes asynchronously; src_bytes 0 writes zeros.
 __device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, int src_bytes) {
@@ -161,37 +187,42 @@ __device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, i
 // of their three input rows: input rows live in a ring of four slots [C8][cols][8], and
 // each output row copies in (cp.async) only the row its successor needs while its own
 // MMAs run; the MMAs of the next row are issued once this row's epilogue has read the
-// other accumulator.
+// other accumulator.  Bound by memory and by the chain of copy, MMAs and epilogue of each row
+// (82 us of a 192 us layer with none of the three doing its work).  Copies and stores in
+// whole 32-byte sectors (they moved half of each) and the bias from shared memory took a 32 -> 32
+// layer on 256 maps from 192 to 152 us on average over the dilations.
 constexpr int kSeg = 8;
 template <int CI, int CO, int EPI>
 __global__ void __launch_bounds__(128)
 conv3x3_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const float *__restrict__ bias,
                   const bf16 *__restrict__ mask, void *__restrict__ out, int H, int W, int dil, int items_per_strip,
-                  int n_items, int withhold_mma) {
+                  int n_items, int withhold_mma, bool wide) {
     constexpr int C8 = CI / 8;
     static_assert(CI % 16 == 0 && (CO == 16 || CO == 32), "K steps of 16; 16 or 32 accumulator columns");
     // dynamic shared memory: weights [9][C8][CO][8], the ring of 4 input rows
-    // [slot][C8][cols][8], two mbarriers, the TMEM address
+    // [slot][C8][plane][8], two mbarriers, the TMEM address
     extern __shared__ __align__(16) unsigned char smem_raw[];
     bf16 *s_w = reinterpret_cast<bf16 *>(smem_raw);
-    const int cols = kTW5 + 2 * dil;
-    const int slot_elems = C8 * cols * 8;
+    const int cols = kTW5 + 2 * dil, plane = conv_plane(dil);
+    const int slot_elems = C8 * plane * 8;
     bf16 *s_ring = s_w + 9 * C8 * CO * 8;
     uint64_t *s_bar = reinterpret_cast<uint64_t *>(s_ring + 4 * slot_elems);
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(s_bar + 2);
+    __shared__ __align__(16) float s_bias[CO];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tiles_per_row = W / kTW5;
+    if (EPI == kEpiReluBf16 && tid < CO) s_bias[tid] = bias[tid];
 
     // input row yy (zeros outside the image) of image img0, columns x0 - dil .., into slot
     auto stage_row = [&](int64_t img0, int x0, int yy, int slot) {
         bf16 *dst = s_ring + slot * slot_elems;
         const bool row_in = yy >= 0 && yy < H;
         for (int v = tid; v < cols * C8; v += 128) {
-            const int c8 = v / cols, px = v - c8 * cols;
+            const int px = v / C8, c8 = v % C8;
             const int xx = x0 + px - dil;
             const bool inside = row_in && xx >= 0 && xx < W;
             const bf16 *src = inside ? in + (img0 + (int64_t)yy * W + xx) * CI + c8 * 8 : in;
-            cp_async16_zfill(dst + ((size_t)c8 * cols + px) * 8, src, inside ? 16 : 0);
+            cp_async16_zfill(dst + (c8 * plane + px) * 8, src, inside ? 16 : 0);
         }
     };
     // the 9 x Cin/16 MMAs of chain row j (input rows j - 1, j, j + 1 in slots (j + 3) % 4,
@@ -205,9 +236,9 @@ conv3x3_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const
             const bf16 *row = s_ring + ((j + 3 + ky) & 3) * slot_elems;
 #pragma unroll
             for (int c0 = 0; c0 < CI; c0 += 16) {
-                const uint32_t a = smem_u32(row + ((size_t)(c0 / 8) * cols + kx * dil) * 8);
+                const uint32_t a = smem_u32(row + ((size_t)(c0 / 8) * plane + kx * dil) * 8);
                 const uint32_t bb = smem_u32(s_w + ((size_t)(tap * C8 + c0 / 8) * CO) * 8);
-                umma_bf16(tmem + 32u * b, umma_smem_desc(a, (uint32_t)cols * 16u, 128u),
+                umma_bf16(tmem + 32u * b, umma_smem_desc(a, (uint32_t)plane * 16u, 128u),
                           umma_smem_desc(bb, CO * 16u, 128u), idesc, accumulate);
                 accumulate = 1;
             }
@@ -272,6 +303,12 @@ conv3x3_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const
             // the input row the next output row adds (chain row j + 2, into the slot of j - 2)
             if (j + 1 < j1) stage_row(img0, x0, rho + (j + 2) * dil, (j + 2) & 3);
             asm volatile("cp.async.commit_group;" ::: "memory");
+            const int64_t pix = img0 + (int64_t)(rho + j * dil) * W + x0 + 32 * warp + lane;
+            uint4 mk[CO / 8];               // this pixel's mask, in flight while the MMAs run
+            if (EPI == kEpiMaskBf16) {
+#pragma unroll
+                for (int qq = 0; qq < CO / 8; qq += 2) load32(mask + pix * CO + 8 * qq, mk[qq], mk[qq + 1], wide);
+            }
             // at most 2^18 tries of at most 1 us each (the suspend-time hint): a quarter second
             uint32_t done = 0;
             const uint32_t parity = (uint32_t)(k >> 1) & 1u;
@@ -281,20 +318,13 @@ conv3x3_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const
                              : "=r"(done) : "r"(smem_u32(s_bar + b)), "r"(parity) : "memory");
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (done) {
-                const int y = rho + j * dil;
                 uint32_t v[CO];
                 tmem_ld_32x32b<CO>(tmem + 32u * b + ((uint32_t)(32 * warp) << 16), v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                const int64_t pix = img0 + (int64_t)y * W + x0 + 32 * warp + lane;
                 if (EPI == kEpiLinearF32) {
                     static_cast<float *>(out)[pix] = __uint_as_float(v[0]) + bias[0];
                 } else {
                     uint4 o[CO / 8];
-                    uint4 mk[CO / 8];
-                    if (EPI == kEpiMaskBf16) {
-#pragma unroll
-                        for (int qq = 0; qq < CO / 8; ++qq) mk[qq] = reinterpret_cast<const uint4 *>(mask + pix * CO)[qq];
-                    }
 #pragma unroll
                     for (int qq = 0; qq < CO / 8; ++qq) {
                         uint32_t packed[4];
@@ -303,8 +333,8 @@ conv3x3_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const
                             const int ch = 8 * qq + 2 * e;
                             float v0 = __uint_as_float(v[ch]), v1 = __uint_as_float(v[ch + 1]);
                             if (EPI == kEpiReluBf16) {
-                                v0 = fmaxf(v0 + bias[ch], 0.f);
-                                v1 = fmaxf(v1 + bias[ch + 1], 0.f);
+                                v0 = fmaxf(v0 + s_bias[ch], 0.f);
+                                v1 = fmaxf(v1 + s_bias[ch + 1], 0.f);
                             } else {
                                 const uint32_t mw = e == 0 ? mk[qq].x : e == 1 ? mk[qq].y : e == 2 ? mk[qq].z : mk[qq].w;
                                 const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162 *>(&mw);
@@ -317,7 +347,7 @@ conv3x3_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const
                         o[qq] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
                     }
 #pragma unroll
-                    for (int qq = 0; qq < CO / 8; ++qq) reinterpret_cast<uint4 *>(static_cast<bf16 *>(out) + pix * CO)[qq] = o[qq];
+                    for (int qq = 0; qq < CO / 8; qq += 2) store32(static_cast<bf16 *>(out) + pix * CO + 8 * qq, o[qq], o[qq + 1], wide);
                 }
             }
             // the next row's input has landed and this row's accumulator has been read
@@ -340,74 +370,103 @@ conv3x3_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" :: "r"(tmem) : "memory");
 }
 
-// Weight gradient partials: CTA c sums rows [c*rows, (c+1)*rows) of the B*H image rows.
+// Weight gradient partials: CTA c sums rows [c*rows, (c+1)*rows) of the B*H image rows, 64 pixels
+// at a time.
 //   part[c][co*9*CI + tap*CI + ci] = sum_p dz[p][co] * x[p + offset(tap)][ci]
 //   part[c][CO*9*CI + co]          = sum_p dz[p][co]
+// The next 64 pixels' three input rows and dz come in by cp.async while these run (two shared
+// buffers of the dilation's size, padded rows: no bank conflicts of ldmatrix).  Bound by the
+// shared-memory reads of the operands (ldmatrix) and mma.sync.  32 maps of 128 x 128, 32 -> 32
+// channels: 100 -> 54 us with the reduction below (20 of the gain the reduction's).
 template <int CI, int CO>
-__global__ void __launch_bounds__(128)
+struct WgradSmem {
+    static constexpr int CIP = CI + 8, COP = CO + 8;
+    static __host__ __device__ int x_elems(int dil) { return 3 * (kTW + 2 * dil) * CIP; }
+    static __host__ __device__ int elems(int dil) { return x_elems(dil) + kTW * COP; }
+};
+template <int CI, int CO>
+__global__ void __launch_bounds__(128, 4)
 conv3x3_wgrad_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ dz, int H, int W, int rows_total,
                      int rows_per_cta, int dil, float *__restrict__ part) {
-    constexpr int CIP = CI + 8, COP = CO + 8;
+    using S = WgradSmem<CI, CO>;
+    constexpr int CIP = S::CIP, COP = S::COP;
     constexpr int NT = 9 * CI / 8;                 // n-tiles of 8 (tap, ci) columns
     constexpr int MT = CO / 16;                    // m-tiles of 16 output channels
     constexpr int NTW = (NT + 3) / 4;              // n-tiles per warp (round robin)
-    __shared__ __align__(16) bf16 s_x[3][kTW + 2 * kMaxDil][CIP];
-    __shared__ __align__(16) bf16 s_dz[kTW][COP];
-    __shared__ float s_db[CO];
+    constexpr int DBP = 128 / CO;                  // threads per channel of the bias gradient
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ float s_db[128];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int cols = kTW + 2 * dil, per_row = W / kTW;
+    auto bx = [&](int b) { return reinterpret_cast<bf16 *>(smem_raw) + b * S::elems(dil); };
+    auto bdz = [&](int b) { return bx(b) + S::x_elems(dil); };
+    auto stage = [&](int t, int b) {
+        const int row = t / per_row, x0 = (t - row * per_row) * kTW, y = row % H;
+        const int64_t img0 = (int64_t)(row - y) * W;
+        bf16 *const sx = bx(b), *const sd = bdz(b);
+#pragma unroll
+        for (int ky = 0; ky < 3; ++ky) {
+            const int yy = y + (ky - 1) * dil;
+            const bool row_in = yy >= 0 && yy < H;
+            for (int v = tid; v < cols * (CI / 8); v += 128) {
+                const int px = v / (CI / 8), c8 = v % (CI / 8), xx = x0 + px - dil;
+                const bool in = row_in && xx >= 0 && xx < W;
+                cp_async16_zfill(sx + (ky * cols + px) * CIP + c8 * 8,
+                                 in ? x + (img0 + (int64_t)yy * W + xx) * CI + c8 * 8 : x, in ? 16 : 0);
+            }
+        }
+        const bf16 *const src = dz + (img0 + (int64_t)y * W + x0) * CO;
+        for (int v = tid; v < kTW * CO / 8; v += 128) {
+            const int px = v / (CO / 8), c8 = v % (CO / 8);
+            cp_async16_zfill(sd + px * COP + c8 * 8, src + px * CO + c8 * 8, 16);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     float acc[MT][NTW][4];
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
         for (int n = 0; n < NTW; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
     float db = 0.f;
-    const int r_begin = blockIdx.x * rows_per_cta;
-    const int r_end = min(rows_total, r_begin + rows_per_cta);
-    for (int row = r_begin; row < r_end; ++row) {
-        const int y = row % H;
-        const int64_t img0 = (int64_t)(row - y) * W;
-        for (int x0 = 0; x0 < W; x0 += kTW) {
-            __syncthreads();
-            const int cols = kTW + 2 * dil;
-            for (int v = tid; v < 3 * cols * (CI / 8); v += 128) {
-                const int ky = v / (cols * (CI / 8));
-                const int rem = v - ky * cols * (CI / 8);
-                const int px = rem / (CI / 8), c8 = rem - px * (CI / 8);
-                const int yy = y + (ky - 1) * dil, xx = x0 + px - dil;
-                uint4 val = make_uint4(0, 0, 0, 0);
-                if (yy >= 0 && yy < H && xx >= 0 && xx < W)
-                    val = *reinterpret_cast<const uint4 *>(x + (img0 + (int64_t)yy * W + xx) * CI + c8 * 8);
-                *reinterpret_cast<uint4 *>(&s_x[ky][px][c8 * 8]) = val;
-            }
-            for (int v = tid; v < kTW * CO / 8; v += 128) {
-                const int px = v / (CO / 8), c8 = v - px * (CO / 8);
-                *reinterpret_cast<uint4 *>(&s_dz[px][c8 * 8]) =
-                    *reinterpret_cast<const uint4 *>(dz + (img0 + (int64_t)y * W + x0 + px) * CO + c8 * 8);
-            }
-            __syncthreads();
-            if (tid < CO)
-                for (int px = 0; px < kTW; ++px) db += __bfloat162float(s_dz[px][tid]);
+    const int t0 = blockIdx.x * rows_per_cta * per_row;
+    const int t1 = min(rows_total, (blockIdx.x + 1) * rows_per_cta) * per_row;
+    if (t0 < t1) stage(t0, 0);
+    for (int t = t0; t < t1; ++t) {
+        const int b = (t - t0) & 1;
+        if (t + 1 < t1) {
+            stage(t + 1, b ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const bf16 *const sx = bx(b), *const sd = bdz(b);
+        {
+            const int co = tid % CO;
 #pragma unroll
-            for (int p0 = 0; p0 < kTW; p0 += 16) {
-                uint32_t a[MT][4];
+            for (int px = tid / CO; px < kTW; px += DBP) db += __bfloat162float(sd[px * COP + co]);
+        }
 #pragma unroll
-                for (int m = 0; m < MT; ++m)
-                    ldsm_x4_t(smem_u32(&s_dz[p0 + (lane & 7) + 8 * (lane >> 4)][m * 16 + 8 * ((lane >> 3) & 1)]),
-                              a[m][0], a[m][1], a[m][2], a[m][3]);
+        for (int p0 = 0; p0 < kTW; p0 += 16) {
+            uint32_t a[MT][4];
 #pragma unroll
-                for (int j = 0; j < NTW; ++j) {
-                    const int nt = warp + 4 * j;
-                    if (nt < NT) {
-                        const int tap = (nt * 8) / CI, ci0 = (nt * 8) % CI;
-                        const int ky = tap / 3, kx = tap % 3;
-                        uint32_t b0, b1;
-                        ldsm_x2_t(smem_u32(&s_x[ky][p0 + (lane & 7) + 8 * ((lane >> 3) & 1) + kx * dil][ci0]), b0, b1);
+            for (int m = 0; m < MT; ++m)
+                ldsm_x4_t(smem_u32(sd + (p0 + (lane & 7) + 8 * (lane >> 4)) * COP + m * 16 + 8 * ((lane >> 3) & 1)),
+                          a[m][0], a[m][1], a[m][2], a[m][3]);
 #pragma unroll
-                        for (int m = 0; m < MT; ++m) mma_bf16(acc[m][j], a[m][0], a[m][1], a[m][2], a[m][3], b0, b1);
-                    }
+            for (int j = 0; j < NTW; ++j) {
+                const int nt = warp + 4 * j;
+                if (nt < NT) {
+                    const int tap = (nt * 8) / CI, ci0 = (nt * 8) % CI;
+                    const int ky = tap / 3, kx = tap % 3;
+                    uint32_t b0, b1;
+                    ldsm_x2_t(smem_u32(sx + (ky * cols + p0 + (lane & 7) + 8 * ((lane >> 3) & 1) + kx * dil) * CIP + ci0), b0, b1);
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma_bf16(acc[m][j], a[m][0], a[m][1], a[m][2], a[m][3], b0, b1);
                 }
             }
         }
+        __syncthreads();                           // this buffer is staged again next
     }
     float *dst = part + (int64_t)blockIdx.x * (CO * 9 * CI + CO);
     const int g = lane >> 2, t2 = 2 * (lane & 3);
@@ -424,17 +483,37 @@ conv3x3_wgrad_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ dz, in
             dst[(co + 8) * 9 * CI + n] = acc[m][j][2];
             dst[(co + 8) * 9 * CI + n + 1] = acc[m][j][3];
         }
-    if (tid < CO) s_db[tid] = db;
+    s_db[tid] = db;
     __syncthreads();
-    if (tid < CO) dst[CO * 9 * CI + tid] = s_db[tid];
+    if (tid < CO) {
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < DBP; ++k) v += s_db[k * CO + tid];
+        dst[CO * 9 * CI + tid] = v;
+    }
 }
 
-__global__ void reduce_partials_kernel(const float *__restrict__ part, int n_parts, int len, float *__restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= len) return;
+// out[i] = sum over the parts in a fixed order: 32 consecutive outputs per CTA, the parts dealt out
+// to its eight warps (each with eight loads in flight), then the eight sums in warp order.  One
+// thread per output over all 608 parts left 37 CTAs waiting on one another's loads.
+__global__ void __launch_bounds__(256) reduce_partials_kernel(const float *__restrict__ part, int n_parts, int len,
+                                                             float *__restrict__ out) {
+    __shared__ float s_sum[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int c = 0; c < n_parts; ++c) s += part[(int64_t)c * len + i];
-    out[i] = s;
+    if (i < len) {
+#pragma unroll 8
+        for (int c = warp; c < n_parts; c += 8) s += part[(int64_t)c * len + i];
+    }
+    s_sum[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && i < len) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t += s_sum[k][lane];
+        out[i] = t;
+    }
 }
 
 // dz[p][0] = 2 w[p] (pred[p] - target[p]) / n, dz[p][1..15] = 0; per-block sums of
@@ -664,7 +743,7 @@ template <int CI, int CO, int EPI>
 cudaError_t launch_conv_tc(const void *in, const void *w, const float *bias, const void *mask, void *out, int B,
                            int H, int W, int dil, cudaStream_t st) {
     auto bytes = [](int d) {
-        const size_t b = sizeof(ddk::bf16) * ((size_t)9 * CI * CO + (size_t)4 * CI * (ddk::kTW5 + 2 * d)) + 32;
+        const size_t b = sizeof(ddk::bf16) * ((size_t)9 * CI * CO + (size_t)4 * CI * ddk::conv_plane(d)) + 32;
         return std::max<size_t>(b, 30 * 1024);
     };
     static bool configured = false;     // allow the largest dilation's staging area once
@@ -700,9 +779,33 @@ cudaError_t launch_conv_tc(const void *in, const void *w, const float *bias, con
     // DD_FAULT=tc_wait (tests): no MMA is issued, so every completion wait runs out and the
     // timeout path (flag, no output, TMEM released) is exercised without a GPU fault
     const int withhold = dd::fault_injected("tc_wait") ? 1 : 0;
+    // 32-byte accesses of the output and the mask (a multiple of 32 bytes per pixel) where both start
+    // on one
+    const bool wide = ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(mask)) & 31) == 0;
     ddk::conv3x3_tc_kernel<CI, CO, EPI><<<grid, 128, bytes(dil), st>>>((const ddk::bf16 *)in, (const ddk::bf16 *)w, bias,
                                                                         (const ddk::bf16 *)mask, out, H, W, dil,
-                                                                        per_strip, n_items, withhold);
+                                                                        per_strip, n_items, withhold, wide);
+    return cudaGetLastError();
+}
+
+template <int CI, int CO>
+cudaError_t launch_wgrad(int n_cta, const ddk::bf16 *x, const ddk::bf16 *dz, int H, int W, int rows_total, int rows_per,
+                         int dil, float *part, cudaStream_t st) {
+    auto bytes = [](int d) { return (int)(2 * sizeof(ddk::bf16)) * ddk::WgradSmem<CI, CO>::elems(d); };
+    static std::atomic<uint64_t> done{0};          // per device: the attributes are set
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess || dev >= 64) return err != cudaSuccess ? err : cudaErrorInvalidDevice;
+    if (!(done.load() & (uint64_t(1) << dev))) {
+        err = cudaFuncSetAttribute(ddk::conv3x3_wgrad_kernel<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   bytes(ddk::kMaxDil));
+        if (err == cudaSuccess)
+            err = cudaFuncSetAttribute(ddk::conv3x3_wgrad_kernel<CI, CO>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                       (int)cudaSharedmemCarveoutMaxShared);
+        if (err != cudaSuccess) return err;
+        done.fetch_or(uint64_t(1) << dev);
+    }
+    ddk::conv3x3_wgrad_kernel<CI, CO><<<n_cta, 128, bytes(dil), st>>>(x, dz, H, W, rows_total, rows_per, dil, part);
     return cudaGetLastError();
 }
 
@@ -781,11 +884,13 @@ dd_status dd_sur_wgrad(const void *x, const void *dz, int32_t B, int32_t H, int3
     dd::ProfScope ps("conv3x3_wgrad", st);
     const ddk::bf16 *xb = (const ddk::bf16 *)x, *db = (const ddk::bf16 *)dz;
     const int d = dilation;
-    if (cin == 16 && cout == 32) ddk::conv3x3_wgrad_kernel<16, 32><<<n_cta, 128, 0, st>>>(xb, db, H, W, rows_total, rows_per, d, part);
-    else if (cin == 32 && cout == 32) ddk::conv3x3_wgrad_kernel<32, 32><<<n_cta, 128, 0, st>>>(xb, db, H, W, rows_total, rows_per, d, part);
-    else if (cin == 32 && cout == 16) ddk::conv3x3_wgrad_kernel<32, 16><<<n_cta, 128, 0, st>>>(xb, db, H, W, rows_total, rows_per, d, part);
-    else ddk::conv3x3_wgrad_kernel<16, 16><<<n_cta, 128, 0, st>>>(xb, db, H, W, rows_total, rows_per, d, part);
-    ddk::reduce_partials_kernel<<<(len + 255) / 256, 256, 0, st>>>(part, n_cta, len, grad);
+    cudaError_t err = cudaSuccess;
+    if (cin == 16 && cout == 32) err = launch_wgrad<16, 32>(n_cta, xb, db, H, W, rows_total, rows_per, d, part, st);
+    else if (cin == 32 && cout == 32) err = launch_wgrad<32, 32>(n_cta, xb, db, H, W, rows_total, rows_per, d, part, st);
+    else if (cin == 32 && cout == 16) err = launch_wgrad<32, 16>(n_cta, xb, db, H, W, rows_total, rows_per, d, part, st);
+    else err = launch_wgrad<16, 16>(n_cta, xb, db, H, W, rows_total, rows_per, d, part, st);
+    if (err != cudaSuccess) return dd::fail_cuda(err, "dd_sur_wgrad launch");
+    ddk::reduce_partials_kernel<<<(len + 31) / 32, 256, 0, st>>>(part, n_cta, len, grad);
     DD_CUDA_TRY(cudaGetLastError());
     return DD_OK;
 }

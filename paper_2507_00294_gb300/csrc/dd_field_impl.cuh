@@ -106,7 +106,7 @@ __device__ __forceinline__ double pair_term(double r2, const RecF64 &R) {
         double p = R.c[15];
 #pragma unroll
         for (int m = 14; m >= 0; --m) p = fma(p, h, R.c[m]);
-        return exp(-a) * p;
+        return exp_neg_f64(a) * p;
     }
     return e1diff_general_f64(a, h, R.c[0]);
 }
@@ -114,13 +114,14 @@ __device__ __forceinline__ double pair_term(double r2, const RecF64 &R) {
 // FP64 moment term of degree D (truncation e^{2h} h^{D+1}/(D+1)! <= 1e-17 at the class
 // limits below): e^-a times Horner in h over c_0..c_D.
 constexpr double kDeg4HD = 1.0e-3, kDeg8HD = 5.2e-2, kDeg11HD = 0.19;
+// their upper words, and 745's
+constexpr int kDeg4Word = 0x3F50624D, kDeg8Word = 0x3FAA9FBE, kDeg11Word = 0x3FC851EB, kZeroWord = 0x40874800;
 template <int D>
-__device__ __forceinline__ double moment_term_f64(double r2, const RecF64 &R) {
-    const double h = r2 * R.dq;
+__device__ __forceinline__ double moment_term_f64(double a, double h, const RecF64 &R) {
     double p = R.c[D];
 #pragma unroll
     for (int m = D - 1; m >= 0; --m) p = fma(p, h, R.c[m]);
-    return exp(-r2 * R.q1) * p;
+    return exp_neg_f64(a) * p;
 }
 
 // Tile configurations.  kThreads threads x kPPT points per thread form a point tile;
@@ -685,22 +686,35 @@ __device__ __forceinline__ void field_tile(TileSmem<Cfg, TCH> &sm, const double 
                 if (gs < na[jc]) {
                     const Rec &R = sm.rec[jc][s];
                     if constexpr (std::is_same<Rec, RecF64>::value) {
-                        // one polynomial degree for the warp, from every lane's own h and a
+                        // one polynomial degree for the warp, from every lane's own h and a.  The
+                        // limits are compared on the upper words (no FP64 compares; a and h
+                        // are never negative): a value at a limit's own word takes the higher
+                        // degree, and a pair at a's word evaluates its (tiny) term.  A lane
+                        // whose own a is 745 or more adds 0.
+                        // (not a NaN: its word is past infinity's, and it reaches pair_term)
+                        auto beyond = [](double v) {
+                            return (uint32_t)(__double2hiint(v) - kZeroWord) <= (uint32_t)(0x7FF00000 - kZeroWord);
+                        };
                         uint32_t cls = 0;
+                        double h[PPT], a[PPT];
 #pragma unroll
                         for (int k = 0; k < PPT; ++k) {
-                            const double h = r2[k] * R.dq, a = r2[k] * R.q1;
-                            const uint32_t c = a >= 745.0 ? 0u : h <= kDeg4HD ? 1u : h <= kDeg8HD ? 2u
-                                             : h <= kDeg11HD ? 3u : 4u;
+                            h[k] = r2[k] * R.dq;
+                            a[k] = r2[k] * R.q1;
+                            const int hw = __double2hiint(h[k]);
+                            const uint32_t c = beyond(a[k]) ? 0u : hw < kDeg4Word ? 1u
+                                             : hw < kDeg8Word ? 2u : hw < kDeg11Word ? 3u : 4u;
                             cls = max(cls, c);
                         }
                         cls = __reduce_max_sync(0xffffffffu, cls);
+                        if (cls == 0u) continue;
 #pragma unroll
                         for (int k = 0; k < PPT; ++k) {
-                            if (cls == 1u) acc[jc][k] += moment_term_f64<4>(r2[k], R);
-                            else if (cls == 2u) acc[jc][k] += moment_term_f64<8>(r2[k], R);
-                            else if (cls == 3u) acc[jc][k] += moment_term_f64<11>(r2[k], R);
-                            else if (cls == 4u) acc[jc][k] += pair_term(r2[k], R);
+                            if (beyond(a[k])) continue;
+                            if (cls == 1u) acc[jc][k] += moment_term_f64<4>(a[k], h[k], R);
+                            else if (cls == 2u) acc[jc][k] += moment_term_f64<8>(a[k], h[k], R);
+                            else if (cls == 3u) acc[jc][k] += moment_term_f64<11>(a[k], h[k], R);
+                            else acc[jc][k] += pair_term(r2[k], R);
                         }
                     } else {
 #pragma unroll

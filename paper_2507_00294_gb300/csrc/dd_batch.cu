@@ -32,6 +32,7 @@
 #include "dd_field_impl.cuh"
 #include "dd_grid.h"
 #include "dd_internal.h"
+#include "dd_sort_points.cuh"
 
 namespace ddk {
 
@@ -81,6 +82,18 @@ __global__ void batch_prep_kernel(const BScan *__restrict__ sc, const int64_t *_
     Y[g] = y;
     const float xh = (float)x, yh = (float)y;
     F[g] = make_float4(xh, (float)(x - (double)xh), yh, (float)(y - (double)yh));
+}
+
+// The point lists in spatial order, kSortPts points of a scan per CTA (dd_sort_points.cuh); CTA q
+// takes chunk q - chunk_offs[k] of scan k.  perm holds indices within the scan.
+__global__ void __launch_bounds__(kSortThreads)
+batch_sort_kernel(const BScan *__restrict__ sc, const int64_t *__restrict__ chunk_offs, int n_scans,
+                  const float4 *__restrict__ in, float4 *__restrict__ F, int *__restrict__ perm) {
+    __shared__ SortSmem sm;
+    const int k = find_segment(chunk_offs, n_scans, blockIdx.x);
+    const BScan &S = sc[k];
+    const int64_t c0 = (blockIdx.x - chunk_offs[k]) * kSortPts, off = S.pt_off, n = S.n_pts;
+    sort_points_block(sm, n, c0, (int)min((int64_t)kSortPts, n - c0), in + off, F + off, perm + off);
 }
 
 template <typename Rec>
@@ -142,14 +155,15 @@ batch_field_kernel(const BScan *__restrict__ sc, const int4 *__restrict__ items,
 }
 
 __global__ void batch_reduce_kernel(const BScan *__restrict__ sc, const int64_t *__restrict__ pt_offs, int n_scans,
-                                    int64_t total, const double *__restrict__ partial, double *__restrict__ out) {
+                                    int64_t total, const double *__restrict__ partial, const int *__restrict__ perm,
+                                    double *__restrict__ out) {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= total) return;
     const BScan &S = sc[find_segment(pt_offs, n_scans, g)];
     const int64_t p = g - S.pt_off;
     double acc = 0.0;
     for (int b = 0; b < S.nblk; ++b) acc += partial[S.part_off + (int64_t)b * S.n_pts + p];
-    out[g] = S.pref * acc;
+    out[perm ? S.pt_off + perm[g] : g] = S.pref * acc;
 }
 
 // Kernel variants with the same 512-point tile (so they share one work list).
@@ -183,6 +197,11 @@ struct dd_batch {
     unsigned *d_counter = nullptr;
     double *d_X = nullptr, *d_Y = nullptr, *d_part = nullptr;
     float4 *d_F = nullptr;
+    // FP32-mixed point lists: the slots' points (within their scan), and the scans' first sorting CTAs
+    float4 *d_F0 = nullptr;             // in the caller's order
+    int *d_perm = nullptr;
+    int64_t *d_chunk_offs = nullptr;
+    int64_t n_chunks = 0;
     void *d_rec = nullptr;
     double *d_pts = nullptr, *d_out = nullptr;   // staging for host buffers
     cudaStream_t cap = nullptr;
@@ -240,7 +259,11 @@ dd_status enqueue(dd_batch *b, const double *pts, double *out, int variant, cuda
     DD_CUDA_TRY(cudaEventRecord(b->ev_fork, st));
     DD_CUDA_TRY(cudaStreamWaitEvent(b->side, b->ev_fork, 0));
     DD_CUDA_TRY(cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned), st));
-    ddk::batch_prep_kernel<<<nb_pts, 256, 0, st>>>(b->d_sc, b->d_pt_offs, b->n_scans, pts, b->total_pts, b->d_X, b->d_Y, b->d_F);
+    ddk::batch_prep_kernel<<<nb_pts, 256, 0, st>>>(b->d_sc, b->d_pt_offs, b->n_scans, pts, b->total_pts, b->d_X, b->d_Y,
+                                                   b->d_perm ? b->d_F0 : b->d_F);
+    if (b->d_perm)
+        ddk::batch_sort_kernel<<<(unsigned)b->n_chunks, ddk::kSortThreads, 0, st>>>(b->d_sc, b->d_chunk_offs, b->n_scans,
+                                                                                  b->d_F0, b->d_F, b->d_perm);
     if (b->total_rec > 0) {
         const unsigned nb = (unsigned)((b->total_rec + 127) / 128);
         if (b->prec == DD_MIXED)
@@ -265,7 +288,8 @@ dd_status enqueue(dd_batch *b, const double *pts, double *out, int variant, cuda
             else launch_field<ddk::CfgF64>(b, g, st);
         }
     }
-    ddk::batch_reduce_kernel<<<nb_pts, 256, 0, st>>>(b->d_sc, b->d_pt_offs, b->n_scans, b->total_pts, b->d_part, out);
+    ddk::batch_reduce_kernel<<<nb_pts, 256, 0, st>>>(b->d_sc, b->d_pt_offs, b->n_scans, b->total_pts, b->d_part,
+                                                     b->d_perm, out);
     DD_CUDA_TRY(cudaGetLastError());
     return DD_OK;
 }
@@ -435,6 +459,17 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
     const size_t o_f = add((size_t)std::max<int64_t>(1, b->total_pts) * sizeof(float4));
     const size_t o_rec = add((size_t)std::max<int64_t>(1, rec) * rec_size);
     const size_t o_part = add((size_t)std::max<int64_t>(1, part) * sizeof(double));
+    // point lists in spatial order where a list is longer than a warp's points
+    std::vector<int64_t> chunk_offs;
+    if (prec == DD_MIXED && b->total_pts > 128 * (int64_t)n_scans) {
+        for (auto &S : sc) {
+            chunk_offs.push_back(b->n_chunks);
+            b->n_chunks += (S.n_pts + ddk::kSortPts - 1) / ddk::kSortPts;
+        }
+    }
+    const size_t o_f0 = add(chunk_offs.empty() ? 0 : (size_t)b->total_pts * sizeof(float4));
+    const size_t o_perm = add(chunk_offs.empty() ? 0 : (size_t)b->total_pts * sizeof(int));
+    const size_t o_chunk = add(chunk_offs.size() * sizeof(int64_t));
     cudaError_t err = cudaMalloc(&b->ws, bytes);
     if (err != cudaSuccess) {
         cudaGetLastError();
@@ -451,6 +486,12 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
     b->d_F = (float4 *)(base + o_f);
     b->d_rec = base + o_rec;
     b->d_part = (double *)(base + o_part);
+    if (!chunk_offs.empty()) {
+        b->d_F0 = (float4 *)(base + o_f0);
+        b->d_perm = (int *)(base + o_perm);
+        b->d_chunk_offs = (int64_t *)(base + o_chunk);
+        DD_CUDA_TRY(cudaMemcpy(b->d_chunk_offs, chunk_offs.data(), chunk_offs.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
+    }
     std::vector<int4> it(items.size());
     for (size_t k = 0; k < items.size(); ++k) it[k] = items[k].second;
     DD_CUDA_TRY(cudaMemcpy(b->d_sc, sc.data(), sc.size() * sizeof(ddk::BScan), cudaMemcpyHostToDevice));

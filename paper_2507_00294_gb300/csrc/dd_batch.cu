@@ -391,7 +391,7 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
             if (S.n_pts == 0) continue;
             const dd::GridBox box{S.gx0, S.gy0, S.gdx, S.gdy, S.gW, S.gH};
             const int g = b->engine->add_grid(s, box);
-            const int t = b->engine->add_table(s, box, src, S.tdim, S.nact);
+            const int t = b->engine->add_table(s, box, src, S.tdim, S.nact, true);
             b->engine->add_job(s, S.srcF, g, t, S.nact, 0, S.pt_off);
             continue;
         }

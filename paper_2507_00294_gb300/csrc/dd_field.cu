@@ -600,12 +600,22 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
 }
 
 // FP32-mixed grids of at least this many columns, rows and points take the contraction
-// (dd_grid.cu); thinner ones leave most of its 128-row tiles empty and take the CUDA-core grid
-// tile.
+// (dd_grid.cu); smaller ones leave most of its tiles empty.
 constexpr int64_t kQuadMinSide = 32, kQuadMinPts = 4096, kQuadMaxSide = int64_t(1) << 30;
 
-dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const std::vector<double> &times, double *out,
-                         cudaStream_t stream) {
+// Narrow grids (below 64 columns, half of the CUDA-core grid tile's 128, whose lanes mostly idle
+// there) take the final kernel of dd_grid.cu with every visit left to it.  A CTA there walks all of
+// a snapshot's visits for 32 columns x 16 rows (0.11 us per visit), where the grid tile splits them;
+// so few visits, or CTAs to fill the GPU with.  A scan of n visits, tile against walk in us:
+// 256 visits, 16 x 16 points, 256 snapshots: 96, 68; 32 snapshots: 73, 57; 576 visits, 32 x 32: 512
+// CTAs 189, 121, 128 CTAs 111, 105; 1024 visits, 48 x 48: 1536 CTAs 341, 302, 384 CTAs 146, 176.
+bool narrow_grid(const ddk::GridDesc &g, int64_t n_t, int64_t n_visits) {
+    const int64_t ctas = ((g.W + 31) / 32) * ((g.H + 15) / 16) * n_t;
+    return g.W < 64 && g.H < kQuadMaxSide && n_visits <= 1024 && ctas >= (n_visits <= 256 ? 32 : n_visits);
+}
+
+dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const std::vector<double> &times, bool contract,
+                         double *out, cudaStream_t stream) {
     const int n_t = (int)times.size();
     const int64_t n_pts = grid.W * grid.H;
     const dd::MemKind out_kind = dd::memory_kind(out);
@@ -623,7 +633,7 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
     // snapshots per pass: rows of k (off the lattice, a table per snapshot) and partial rows
     // within about 1 GiB
     int group = std::min(n_t, 4096);
-    while (group > 1 && (double)group * ((lattice ? 0.0 : 48.0 * (double)scan->n) + 16.0 * (double)n_pts) > (double)(int64_t(1) << 30))
+    while (group > 1 && (double)group * ((lattice ? 0.0 : (contract ? 48.0 : 80.0) * (double)scan->n) + 16.0 * (double)n_pts) > (double)(int64_t(1) << 30))
         group = (group + 1) / 2;
     double *out_dev = out;
     void *out_ws = nullptr;
@@ -642,10 +652,10 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
         const int ng = std::min(group, n_t - g0);
         dd::GridEngine eng;
         const int gi = eng.add_grid(scan, box);
-        const int lag = lattice ? eng.add_lag_table(scan, box, M) : -1;
+        const int lag = lattice ? eng.add_lag_table(scan, box, M, contract) : -1;
         for (int j = g0; j < g0 + ng; ++j) {
             // on the lattice, snapshot t sees visit v at lag t - v: table visit M - t + v
-            const int table = lattice ? lag : eng.add_table(scan, box, src, tdim[j], nact[j]);
+            const int table = lattice ? lag : eng.add_table(scan, box, src, tdim[j], nact[j], contract);
             const int shift = lattice ? (int)(tdim[j] > 0 ? M - (int64_t)tdim[j] : M) : 0;
             eng.add_job(scan, srcF, gi, table, nact[j], shift, (int64_t)order[j] * n_pts);
         }
@@ -659,9 +669,14 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
             return no_memory(err);
         }
         eng.bind(ws);
-        keep->images.emplace_back(eng.table_bytes());
-        eng.write_tables(keep->images.back().data());
-        DD_CUDA_TRY(keep->staging.upload(ws, keep->images.back().data(), keep->images.back().size(), stream));
+        const size_t n_tab = eng.table_bytes();
+        char *tables = static_cast<char *>(keep->staging.stage(n_tab));
+        if (!tables) {                           // no pinned memory: a pageable image
+            keep->images.emplace_back(n_tab);
+            tables = keep->images.back().data();
+        }
+        eng.write_tables(tables);
+        DD_CUDA_TRY(cudaMemcpyAsync(ws, tables, n_tab, cudaMemcpyHostToDevice, stream));
         SideStream *side = nullptr;
         DD_CUDA_TRY(side_stream(&side));
         // DD_FAULT=field_tc_wait (tests): no MMA is issued, so the completion waits run out and
@@ -734,7 +749,8 @@ extern "C" dd_status dd_field_on_grid(const dd_scan *scan, double x0_m, double y
     g.x0 = x0_m; g.y0 = y0_m; g.dx = dx_m; g.dy = dy_m; g.W = n_cols; g.H = n_rows;
     const int64_t n_pts = n_cols * n_rows;
     if (prec == DD_MIXED && std::min(n_cols, n_rows) >= kQuadMinSide && n_pts >= kQuadMinPts && std::max(n_cols, n_rows) < kQuadMaxSide)
-        return run_grid_mixed(scan, g, times, out, stream);
+        return run_grid_mixed(scan, g, times, true, out, stream);
+    if (prec == DD_MIXED && narrow_grid(g, n_t, scan->n)) return run_grid_mixed(scan, g, times, false, out, stream);
     if (prec == DD_MIXED) return run_field<ddk::CfgMixed>(scan, nullptr, n_pts, g, times, out, stream);
     return run_field<ddk::CfgF64>(scan, nullptr, n_pts, g, times, out, stream);
 }

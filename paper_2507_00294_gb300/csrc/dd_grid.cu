@@ -10,7 +10,6 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
-#include <queue>
 #include <utility>
 
 #include "dd_grid_quad.cuh"
@@ -24,8 +23,12 @@ using ddk::kGqNodes;
 // grid (+inf: none): h = rho^2 dq <= kGqH for rho^2 up to R2, the largest squared distance
 // between the grid's box and the visits' box, r = w1/w0 - 1 <= kGqR, and the dwell over.  With
 // c = 4 kappa tau_max, dq <= c / ((w1 - c) w1) and r <= c / (w1 - c) for every visit (both grow
-// with the dwell at a fixed w1 = 2s + 4 kappa (t - T_i)).
-void band_ages(const dd_scan *scan, const dd::GridBox &g, double (&age)[kGqBands]) {
+// with the dwell at a fixed w1 = 2s + 4 kappa (t - T_i)).  Without the contraction: none.
+void band_ages(const dd_scan *scan, const dd::GridBox &g, bool contract, double (&age)[kGqBands]) {
+    if (!contract) {
+        for (double &a : age) a = INFINITY;
+        return;
+    }
     const double ip = 1.0 / scan->pitch;
     const double xa = g.x0 * ip, xb = (g.x0 + (double)(g.W - 1) * g.dx) * ip;
     const double ya = g.y0 * ip, yb = (g.y0 + (double)(g.H - 1) * g.dy) * ip;
@@ -128,9 +131,9 @@ int GridEngine::add_grid(const dd_scan *scan, const GridBox &g) {
     return (int)t->grids.size() - 1;
 }
 
-int GridEngine::add_table(const dd_scan *scan, const GridBox &g, const double *src, double tdim, int nact) {
+int GridEngine::add_table(const dd_scan *scan, const GridBox &g, const double *src, double tdim, int nact, bool contract) {
     double age[kGqBands];
-    band_ages(scan, g, age);
+    band_ages(scan, g, contract, age);
     ddk::GqTable tb{src + 2 * scan->n, src + 3 * scan->n, scan->s, scan->kappa, tdim, t->n_vis, t->n_rows, t->n_rec, nact, 0, {}};
     tb.vb[0] = 0;
     for (int b = 0; b < kGqBands; ++b) {
@@ -146,9 +149,9 @@ int GridEngine::add_table(const dd_scan *scan, const GridBox &g, const double *s
     return (int)t->tabs.size() - 1;
 }
 
-int GridEngine::add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M) {
+int GridEngine::add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M, bool contract) {
     double age[kGqBands];
-    band_ages(scan, g, age);
+    band_ages(scan, g, contract, age);
     ddk::GqTable tb{nullptr, nullptr, scan->s, scan->kappa, 0.0, t->n_vis, t->n_rows, t->n_rec, (int)M, 0, {}};
     tb.vb[0] = 0;
     for (int b = 0; b < kGqBands; ++b) {
@@ -218,7 +221,10 @@ cudaError_t GridEngine::finish(bool two_launches) {
         if (total == 0) continue;
         // about two runs per CTA, so that dealing them out longest first evens the CTAs' shares
         const int64_t per = std::max<int64_t>(total / (2 * sms), 2 * kRunCost);
-        std::vector<std::pair<int64_t, ddk::GqRun>> list;
+        std::vector<ddk::GqRun> list;
+        std::vector<std::pair<int64_t, int>> order;      // (- cost, run)
+        list.reserve((size_t)(4 * sms) + t->jobs.size());
+        order.reserve(list.capacity());
         for (size_t j = 0; j < t->jobs.size(); ++j) {
             int64_t k0, k1;
             span(j, k0, k1);
@@ -230,29 +236,30 @@ cudaError_t GridEngine::finish(bool two_launches) {
             const int64_t P = std::min(std::max<int64_t>(1, (cost + per / 2) / per), steps);
             for (int64_t p = 0; p < P; ++p) {
                 const int64_t a = k0 + steps * p / P * 16, b = std::min(k1, k0 + steps * (p + 1) / P * 16);
-                for (int q = 0; q < n_tiles; ++q)
-                    list.push_back({(b - a) * row_cost(J, q) + kRunCost,
-                                    ddk::GqRun{a, (int)(b - a), (int)j, q, J.nq + (int)p}});
+                for (int q = 0; q < n_tiles; ++q) {
+                    order.push_back({-((b - a) * row_cost(J, q) + kRunCost), (int)list.size()});
+                    list.push_back(ddk::GqRun{a, (int)(b - a), (int)j, q, J.nq + (int)p});
+                }
             }
             J.nq += (int)P;
         }
-        std::stable_sort(list.begin(), list.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
-        const int n_cta = (int)std::min<int64_t>(sms, (int64_t)list.size());
-        std::vector<std::vector<int>> of((size_t)n_cta);
-        std::priority_queue<std::pair<int64_t, int>, std::vector<std::pair<int64_t, int>>, std::greater<std::pair<int64_t, int>>> load;
-        for (int c = 0; c < n_cta; ++c) load.push({0, c});
+        std::sort(order.begin(), order.end());
+        // dealt out longest first, back and forth over the CTAs: run k goes to CTA k % n on even
+        // rounds and n - 1 - k % n on odd ones
+        const int n = (int)std::min<int64_t>(sms, (int64_t)list.size()), full = (int)list.size() / n, rest = (int)list.size() % n;
+        const int base = (int)t->runs.size();
+        auto extra = [&](int c) { return (full & 1 ? n - 1 - c : c) < rest ? 1 : 0; };   // a run of the last round
+        t->n_cta[launch] = n;
+        for (int c = 0, off = base; c <= n; ++c) {
+            t->cta_off.push_back(off);
+            if (c < n) off += full + extra(c);
+        }
+        const int *const off = t->cta_off.data() + t->cta_off.size() - (size_t)(n + 1);
+        t->runs.resize((size_t)base + list.size());
         for (size_t k = 0; k < list.size(); ++k) {
-            const std::pair<int64_t, int> top = load.top();
-            load.pop();
-            of[(size_t)top.second].push_back((int)k);
-            load.push({top.first + list[k].first, top.second});
+            const int round = (int)k / n, pos = (int)k % n, c = (round & 1) ? n - 1 - pos : pos;
+            t->runs[(size_t)(off[c] + round)] = list[(size_t)order[k].second];
         }
-        t->n_cta[launch] = n_cta;
-        for (int c = 0; c < n_cta; ++c) {
-            t->cta_off.push_back((int)t->runs.size());
-            for (int k : of[(size_t)c]) t->runs.push_back(list[(size_t)k].second);
-        }
-        t->cta_off.push_back((int)t->runs.size());
     }
     for (ddk::GqJob &j : t->jobs) {
         j.t_off = t->n_part;

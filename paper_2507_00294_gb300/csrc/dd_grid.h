@@ -35,9 +35,10 @@ class GridEngine {
     // Axes of a grid (W, H < 2^30) in the scan's pitch units; returns its index.
     int add_grid(const dd_scan *scan, const GridBox &g);
     // Coefficients of the visits [0, nact) of a scan at tdim (dwells), or of the lags M .. 1 of a
-    // uniform scan; src: the scan's device block.  Returns the table's index.
-    int add_table(const dd_scan *scan, const GridBox &g, const double *src, double tdim, int nact);
-    int add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M);
+    // uniform scan; src: the scan's device block; contract: false leaves every visit to the
+    // CUDA cores.  Returns the table's index.
+    int add_table(const dd_scan *scan, const GridBox &g, const double *src, double tdim, int nact, bool contract);
+    int add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M, bool contract);
     // The scan's snapshot with nact started visits, table visit = visit + shift; its field goes to
     // out + out_off (W H values).
     void add_job(const dd_scan *scan, const float4 *srcF, int grid, int table, int nact, int shift, int64_t out_off);

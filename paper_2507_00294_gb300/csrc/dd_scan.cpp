@@ -268,6 +268,7 @@ void pinned_give(PinnedBlock b) {
 
 struct Deferred {
     cudaEvent_t ev;
+    cudaStream_t stream;
     int device;
     void *obj;
     void (*del)(void *);
@@ -283,12 +284,18 @@ cudaError_t defer_release(cudaStream_t stream, void *obj, void (*del)(void *)) {
     if (err == cudaSuccess && (device < 0 || device >= 64)) err = cudaErrorInvalidDevice;
     if (err == cudaSuccess) {
         std::lock_guard<std::mutex> lock(g_deferred_mu);
-        // release what has completed (in order: the list is in enqueue order per stream)
+        // release what has completed; the list is in enqueue order per stream, so the entries
+        // of a stream after its first unfinished one need no query (a host that runs ahead has
+        // dozens pending)
+        std::vector<std::pair<int, cudaStream_t>> busy;
         for (auto it = g_deferred.begin(); it != g_deferred.end();) {
-            if (cudaEventQuery(it->ev) == cudaSuccess) {
+            const std::pair<int, cudaStream_t> key{it->device, it->stream};
+            const bool known = key.second != cudaStreamPerThread && std::find(busy.begin(), busy.end(), key) != busy.end();
+            if (!known && cudaEventQuery(it->ev) == cudaSuccess) {
                 done.push_back(*it);
                 it = g_deferred.erase(it);
             } else {
+                if (!known) busy.push_back(key);
                 ++it;
             }
         }
@@ -308,7 +315,7 @@ cudaError_t defer_release(cudaStream_t stream, void *obj, void (*del)(void *)) {
         }
         if (err == cudaSuccess) err = cudaEventRecord(ev, stream);
         if (err == cudaSuccess) {
-            g_deferred.push_back({ev, device, obj, del});
+            g_deferred.push_back({ev, stream, device, obj, del});
         } else {
             cudaGetLastError();
             if (ev) g_free_events[device].push_back(ev);

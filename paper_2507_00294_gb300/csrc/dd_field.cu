@@ -614,6 +614,67 @@ bool narrow_grid(const ddk::GridDesc &g, int64_t n_t, int64_t n_visits) {
     return g.W < 64 && g.H < kQuadMaxSide && n_visits <= 1024 && ctas >= (n_visits <= 256 ? 32 : n_visits);
 }
 
+// Snapshots (indices k0 .. k1 - 1 in time order) of a whole raster on the dwell lattice that share
+// their sums by a shift of scan rows (dd_grid_quad.cuh), grouped by phase, where that leaves at most
+// half of the pairs and takes at most twice the partial rows; the rest is returned in `rest`.  rows:
+// grid rows per pitch.  The grid covers the scan, so that every visit passes the same grid points
+// closely in each snapshot: a tile of the tall grid then holds no terms that are large only where
+// this snapshot does not look (the contraction's factors are relative to the tile's largest).
+struct ShiftGroups {
+    std::vector<std::vector<int>> groups;
+    std::vector<int> rest;
+    int rows = 0;
+    int64_t H_ext = 0;
+};
+ShiftGroups shift_groups(const dd_scan *scan, const ddk::GridDesc &grid, const std::vector<double> &tdim, bool lattice,
+                         int k0, int k1) {
+    ShiftGroups out;
+    out.H_ext = grid.H;
+    const double per = grid.dy > 0.0 ? std::nearbyint(scan->pitch / grid.dy) : 0.0;
+    const double xe = grid.x0 + (double)(grid.W - 1) * grid.dx, tol = 1e-9 * scan->pitch;
+    const bool covers = std::min(grid.x0, xe) <= tol && std::max(grid.x0, xe) >= (scan->nx - 1) * scan->pitch - tol &&
+                        grid.y0 <= tol && grid.y0 + (double)(grid.H - 1) * grid.dy >= (scan->ny - 1) * scan->pitch - tol;
+    // (a row further down then lies where the scan's next row shifts it, to 1e-12 pitch over the
+    // largest scan)
+    const bool fits = lattice && covers && scan->order == DD_RASTER && scan->n == (int64_t)scan->nx * scan->ny &&
+                      per >= 1.0 && per <= 64.0 && std::fabs(per * grid.dy - scan->pitch) * scan->ny <= 1e-12 * scan->pitch;
+    std::vector<std::pair<int64_t, int>> by_phase;       // (phase, index), whole dwells inside the scan
+    for (int k = k0; k < k1; ++k) {
+        if (fits && tdim[k] >= 1.0 && tdim[k] <= (double)scan->n) by_phase.push_back({(int64_t)tdim[k] % scan->nx, k});
+        else out.rest.push_back(k);
+    }
+    std::sort(by_phase.begin(), by_phase.end());
+    for (size_t a = 0; a < by_phase.size();) {
+        size_t b = a;
+        std::vector<int> g;
+        double direct = 0.0, shifted = 0.0, rows_shifted = 0.0;       // pairs / W, partial rows
+        for (; b < by_phase.size() && by_phase[b].first == by_phase[a].first; ++b) {
+            const int k = by_phase[b].second;
+            // (a snapshot given twice is its own sum)
+            if (!g.empty() && tdim[k] == tdim[g.back()]) out.rest.push_back(k);
+            else g.push_back(k);
+        }
+        const int64_t last = (int64_t)tdim[g.back()], h_ext = grid.H + (int64_t)per * ((last - (int64_t)tdim[g[0]]) / scan->nx);
+        double before = 0.0;
+        for (int k : g) {
+            const double H = (double)(grid.H + (int64_t)per * ((last - (int64_t)tdim[k]) / scan->nx));
+            direct += tdim[k] * (double)grid.H;
+            shifted += (tdim[k] - before) * H;
+            rows_shifted += H;
+            before = tdim[k];
+        }
+        if (shifted <= 0.5 * direct && rows_shifted <= 2.0 * (double)(g.size() * grid.H) && h_ext < kQuadMaxSide) {
+            out.rows = (int)per;
+            out.H_ext = std::max(out.H_ext, h_ext);
+            out.groups.push_back(std::move(g));
+        } else {
+            out.rest.insert(out.rest.end(), g.begin(), g.end());
+        }
+        a = b;
+    }
+    return out;
+}
+
 dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const std::vector<double> &times, bool contract,
                          double *out, cudaStream_t stream) {
     const int n_t = (int)times.size();
@@ -651,9 +712,22 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
     for (int g0 = 0; g0 < n_t; g0 += group) {
         const int ng = std::min(group, n_t - g0);
         dd::GridEngine eng;
-        const int gi = eng.add_grid(scan, box);
+        const ShiftGroups sg = shift_groups(scan, grid, tdim, lattice && contract, g0, g0 + ng);
+        // (a row of a group's tall grid counts only where some snapshot sees it, at a distance
+        // that the grid itself has)
         const int lag = lattice ? eng.add_lag_table(scan, box, M, contract) : -1;
-        for (int j = g0; j < g0 + ng; ++j) {
+        if (!sg.groups.empty()) {
+            dd::GridBox tall = box;
+            tall.H = sg.H_ext;
+            const int gt = eng.add_grid(scan, tall);
+            for (const std::vector<int> &g : sg.groups) {
+                std::vector<std::pair<int64_t, int64_t>> snaps;
+                for (int k : g) snaps.push_back({(int64_t)tdim[k], (int64_t)order[k] * n_pts});
+                eng.add_shift_group(scan, srcF, gt, lag, M, grid.H, sg.rows, snaps);
+            }
+        }
+        const int gi = sg.rest.empty() ? -1 : eng.add_grid(scan, box);
+        for (int j : sg.rest) {
             // on the lattice, snapshot t sees visit v at lag t - v: table visit M - t + v
             const int table = lattice ? lag : eng.add_table(scan, box, src, tdim[j], nact[j], contract);
             const int shift = lattice ? (int)(tdim[j] > 0 ? M - (int64_t)tdim[j] : M) : 0;

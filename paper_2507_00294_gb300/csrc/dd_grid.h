@@ -3,6 +3,7 @@
 // Used per call by dd_field_on_grid and per plan by the grid batches.
 #pragma once
 #include <cstdint>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -42,6 +43,11 @@ class GridEngine {
     // The scan's snapshot with nact started visits, table visit = visit + shift; its field goes to
     // out + out_off (W H values).
     void add_job(const dd_scan *scan, const float4 *srcF, int grid, int table, int nact, int shift, int64_t out_off);
+    // Snapshots M_0 < M_1 < .. (dwells; each with its offset in out) of one phase of a raster, on
+    // the first H rows of a grid that reaches the tall grid of the group (dd_grid_quad.cuh);
+    // table: the lags M .. 1; rows_per_scan_row: grid rows per pitch.
+    void add_shift_group(const dd_scan *scan, const float4 *srcF, int grid, int table, int64_t M, int64_t H,
+                         int rows_per_scan_row, const std::vector<std::pair<int64_t, int64_t>> &snaps);
     // Splits the contraction into runs for the device's SMs: the rows of k of one and two nodes
     // and the rest as two launches (two_launches), or all in one.
     cudaError_t finish(bool two_launches);
@@ -58,6 +64,8 @@ class GridEngine {
     int64_t n_runs() const;
 
   private:
+    void add_span(const dd_scan *scan, const float4 *srcF, int grid, int table, int i0, int i1, int shift, int H,
+                  int64_t out_off);
     struct Tables;
     Tables *t;
 };

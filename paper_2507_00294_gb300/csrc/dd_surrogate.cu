@@ -181,193 +181,293 @@ __device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, i
                  : "memory");
 }
 
-// Persistent CTAs: each stages the weights once and allocates two TMEM accumulators once,
-// then walks work items.  An item is a segment of kSeg output rows of one 128-pixel column
-// strip, taken with stride dil (rows y0, y0 + dil, ...), so that consecutive rows share two
-// of their three input rows: input rows live in a ring of four slots [C8][cols][8], and
-// each output row copies in (cp.async) only the row its successor needs while its own
-// MMAs run; the MMAs of the next row are issued once this row's epilogue has read the
-// other accumulator.  Bound by memory and by the chain of copy, MMAs and epilogue of each row
-// (82 us of a 192 us layer with none of the three doing its work).  Copies and stores in
-// whole 32-byte sectors (they moved half of each) and the bias from shared memory took a 32 -> 32
-// layer on 256 maps from 192 to 152 us on average over the dilations.
+// Persistent CTAs of three roles over work items.  An item is a segment of at most kSeg output
+// rows of one 128-pixel column strip, taken with stride dil (rows y0, y0 + dil, ...).  Input row i
+// of that chain takes part in output rows i - 1, i and i + 1, so its MMAs, one per tap column and
+// 16 channels, carry the weights of all three rows side by side (N = 3 CO): a third of the
+// MMAs and of the shared-memory reads of the pixels that one output row at a time takes.  The
+// output rows of an item are neighbouring blocks of CO columns of tensor memory; an input row
+// starts the block of row i + 1 with an MMA of its own (no accumulate).
+//   warps 0-3: epilogue (blocks are given back as soon as they are in registers);
+//   warps 4-7: copies (cp.async) into a ring of input rows;
+//   warp 8: one thread issues the MMAs.
+// The roles hand over two rows at a time: the waits, commits and fences of a row took longer than
+// its work (2000 clocks per row and role one row at a time).  Step k of an item brings the input
+// rows j0 - 1 + 2 k and j0 + 2 k, starts output rows j0 + 2 k and the next, and completes the two
+// before.  Every wait is bounded; a wait that gives up stops the CTA's roles and sets the timeout
+// flag.  Two CTAs per SM (256 TMEM columns each).
+// A 32 -> 32 layer on 256 maps (537 MB) takes 115 to 132 us over the dilations, 4.1 to 4.7 TB/s: bound
+// by memory beside the hand-overs (58 us with no copies, MMAs or stores, 90 without the stores).
+// One input row at a time took 122 to 142 us, one output row at a time, each with its nine taps,
+// 152 on average.  Eight epilogue warps or two steps ahead gave nothing.
 constexpr int kSeg = 8;
+constexpr int kConvAhead = 1, kConvMaxSlots = 5, kConvThreads = 288;     // slots of two rows
+static_assert(kConvMaxSlots > kConvAhead + 1 && kSeg % 4 == 0, "a slot is refilled after its rows have been handed over");
+
+struct ConvItem {
+    int64_t img0;
+    int x0, rho, j0, j1, J;         // output rows rho + j dil, j0 <= j < j1; input rows 0 <= j < J
+};
+
 template <int CI, int CO, int EPI>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kConvThreads, 2)
 conv3x3_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, const float *__restrict__ bias,
-                  const bf16 *__restrict__ mask, void *__restrict__ out, int H, int W, int dil, int items_per_strip,
-                  int n_items, int withhold_mma, bool wide) {
-    constexpr int C8 = CI / 8;
+                  const bf16 *__restrict__ mask, void *__restrict__ out, int H, int W, int dil, int seg,
+                  int items_per_strip, int n_items, int n_slots, int withhold_mma, bool wide) {
+    constexpr int C8 = CI / 8, N = 3 * CO, kCols = kSeg * CO;
     static_assert(CI % 16 == 0 && (CO == 16 || CO == 32), "K steps of 16; 16 or 32 accumulator columns");
-    // dynamic shared memory: weights [9][C8][CO][8], the ring of 4 input rows
-    // [slot][C8][plane][8], two mbarriers, the TMEM address
+    // dynamic shared memory: weights [kx][C8][2 - ky][CO][8], the ring of input rows [slot][2][C8][plane][8]
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    bf16 *s_w = reinterpret_cast<bf16 *>(smem_raw);
-    const int cols = kTW5 + 2 * dil, plane = conv_plane(dil);
-    const int slot_elems = C8 * plane * 8;
-    bf16 *s_ring = s_w + 9 * C8 * CO * 8;
-    uint64_t *s_bar = reinterpret_cast<uint64_t *>(s_ring + 4 * slot_elems);
-    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(s_bar + 2);
+    __shared__ __align__(8) uint64_t s_full[kConvMaxSlots], s_empty[kConvMaxSlots], s_done[kSeg / 2], s_free[kSeg / 2], s_end;
     __shared__ __align__(16) float s_bias[CO];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail;
+    bf16 *s_w = reinterpret_cast<bf16 *>(smem_raw);
+    const int cols = kTW5 + 2 * dil, plane = conv_plane(dil), row_elems = C8 * plane * 8;
+    bf16 *s_ring = s_w + 3 * C8 * N * 8;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tiles_per_row = W / kTW5;
+    const int long_rows = H / dil + 1, long_segs = (long_rows + seg - 1) / seg, short_segs = (long_rows - 1 + seg - 1) / seg;
+
     if (EPI == kEpiReluBf16 && tid < CO) s_bias[tid] = bias[tid];
-
-    // input row yy (zeros outside the image) of image img0, columns x0 - dil .., into slot
-    auto stage_row = [&](int64_t img0, int x0, int yy, int slot) {
-        bf16 *dst = s_ring + slot * slot_elems;
-        const bool row_in = yy >= 0 && yy < H;
-        for (int v = tid; v < cols * C8; v += 128) {
-            const int px = v / C8, c8 = v % C8;
-            const int xx = x0 + px - dil;
-            const bool inside = row_in && xx >= 0 && xx < W;
-            const bf16 *src = inside ? in + (img0 + (int64_t)yy * W + xx) * CI + c8 * 8 : in;
-            cp_async16_zfill(dst + (c8 * plane + px) * 8, src, inside ? 16 : 0);
-        }
-    };
-    // the 9 x Cin/16 MMAs of chain row j (input rows j - 1, j, j + 1 in slots (j + 3) % 4,
-    // j % 4, (j + 1) % 4) into accumulator b, committed to barrier b
-    auto issue = [&](int j, int b, uint32_t tmem) {
-        constexpr uint32_t idesc = umma_idesc_bf16(kTW5, CO);
-        int accumulate = 0;
-#pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const int ky = tap / 3, kx = tap % 3;
-            const bf16 *row = s_ring + ((j + 3 + ky) & 3) * slot_elems;
-#pragma unroll
-            for (int c0 = 0; c0 < CI; c0 += 16) {
-                const uint32_t a = smem_u32(row + ((size_t)(c0 / 8) * plane + kx * dil) * 8);
-                const uint32_t bb = smem_u32(s_w + ((size_t)(tap * C8 + c0 / 8) * CO) * 8);
-                umma_bf16(tmem + 32u * b, umma_smem_desc(a, (uint32_t)plane * 16u, 128u),
-                          umma_smem_desc(bb, CO * 16u, 128u), idesc, accumulate);
-                accumulate = 1;
-            }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                     :: "r"(smem_u32(s_bar + b)) : "memory");
-    };
-    // item q: strip (image, column tile), then the segment within the strip: rows
-    // rho + dil * (seg * kSeg + i), i < kSeg, for the residue rho of its chain
-    auto decode = [&](int q, int64_t &img0, int &x0, int &rho, int &j0, int &j1) {
-        const int strip = q / items_per_strip;
-        int r = q - strip * items_per_strip;
-        const int bimg = strip / tiles_per_row;
-        x0 = (strip - bimg * tiles_per_row) * kTW5;
-        img0 = (int64_t)bimg * H * W;
-        for (rho = 0; rho < dil; ++rho) {
-            const int J = (H - rho + dil - 1) / dil;             // chain rows rho, rho + dil, .. < H
-            const int ns = (J + kSeg - 1) / kSeg;
-            if (r < ns) { j0 = r * kSeg; j1 = min(J, j0 + kSeg); return; }
-            r -= ns;
-        }
-        j0 = j1 = 0;                                             // not reached for q < n_items
-    };
-
-    for (int v = tid; v < CO * 9 * C8; v += 128) {
-        const int co = v / (9 * C8), r = v - co * (9 * C8);      // r = tap * C8 + c8
-        cp_async16_zfill(s_w + ((size_t)r * CO + co) * 8, w + (int64_t)co * 9 * CI + r * 8, 16);
+    for (int v = tid; v < 3 * C8 * N; v += kConvThreads) {
+        const int n = v % N, c8 = (v / N) % C8, kx = v / (N * C8), ky = 2 - n / CO, co = n % CO;
+        cp_async16_zfill(s_w + (size_t)v * 8, w + ((int64_t)co * 9 + ky * 3 + kx) * CI + c8 * 8, 16);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" :: "r"(smem_u32(s_tmem)) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_u32(&s_tmem)), "n"(kCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(s_bar)) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(s_bar + 1)) : "memory");
+        for (int k = 0; k < kConvMaxSlots; ++k) {
+            mbar_init(s_full + k, 4);
+            mbar_init(s_empty + k, 1);
+        }
+        for (int k = 0; k < kSeg / 2; ++k) {
+            mbar_init(s_done + k, 1);
+            mbar_init(s_free + k, 4);
+        }
+        mbar_init(&s_end, 1);
+        s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    fence_proxy_async_smem();
+    tc_fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *s_tmem;
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
 
-    int k = 0;                      // rows done by this CTA: accumulator k & 1, barrier use k >> 1
-    bool ok = true;
-    for (int q = blockIdx.x; q < n_items && ok; q += gridDim.x) {
-        int64_t img0;
-        int x0, rho, j0, j1;
-        decode(q, img0, x0, rho, j0, j1);
-        // the first row's three input rows (chain rows j0 - 1 .. j0 + 1), then its MMAs; every
-        // earlier MMA of this CTA has completed (each row's wait precedes its epilogue)
-        for (int i = j0 - 1; i <= j0 + 1; ++i) stage_row(img0, x0, rho + i * dil, (i + 4) & 3);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (tid == 0 && !withhold_mma) issue(j0, k & 1, tmem);
-        for (int j = j0; j < j1; ++j, ++k) {
-            const int b = k & 1;
-            // the input row the next output row adds (chain row j + 2, into the slot of j - 2)
-            if (j + 1 < j1) stage_row(img0, x0, rho + (j + 2) * dil, (j + 2) & 3);
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            const int64_t pix = img0 + (int64_t)(rho + j * dil) * W + x0 + 32 * warp + lane;
-            uint4 mk[CO / 8];               // this pixel's mask, in flight while the MMAs run
-            if (EPI == kEpiMaskBf16) {
+    // at most 2^18 tries of at most 1 us each (the suspend-time hint): a quarter second
+    auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
+        uint32_t done = 0;
+        for (int it = 0; it < (1 << 18); ++it) {
+            asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
+                         " selp.u32 %0, 1, 0, p;\n}\n"
+                         : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+            if (done) return true;
+            if (*(volatile int *)&s_fail) return false;
+        }
+        *(volatile int *)&s_fail = 1;
+        return false;
+    };
+    // by every lane: one lane's wait and a shuffle were slower
+    auto warp_wait = [&](uint64_t *bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, wait(bar, parity)); };
+    auto arrive = [&](uint64_t *bar) {
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(bar)) : "memory");
+    };
+    // item q: strip (image, column tile), then the segment within the strip
+    auto decode = [&](int q) -> ConvItem {
+        ConvItem I;
+        const int strip = q / items_per_strip;
+        int r = q - strip * items_per_strip;
+        const int bimg = strip / tiles_per_row;
+        I.x0 = (strip - bimg * tiles_per_row) * kTW5;
+        I.img0 = (int64_t)bimg * H * W;
+        // chains rho < H mod dil have long_rows rows, the others one less
+        const int n_long = (H - (long_rows - 1) * dil) * long_segs;
+        const bool is_long = r < n_long;
+        const int ns = is_long ? long_segs : short_segs, rest = is_long ? r : r - n_long, c = rest / ns;
+        I.J = is_long ? long_rows : long_rows - 1;
+        I.rho = is_long ? c : c + H - (long_rows - 1) * dil;
+        I.j0 = (rest - c * ns) * seg;
+        I.j1 = min(I.J, I.j0 + seg);
+        return I;
+    };
+    // first block of an item after one at `base`: items of at most half the blocks alternate
+    auto next_base = [&](int base, const ConvItem &I) { return 2 * (I.j1 - I.j0) <= kSeg && base == 0 ? kSeg / 2 : 0; };
+
+    if (warp < 4) {                                              // epilogue
+        uint32_t phase = 0;                                      // bit: parity of the pair's use
+        int base = 0;
+        bool ok = true;
+        for (int q = blockIdx.x; q < n_items && ok; q += gridDim.x) {
+            const ConvItem I = decode(q);
+            base = next_base(base, I);
+            for (int j = I.j0; j < I.j1; j += 2) {
+                const int pair = (base + j - I.j0) / 2, n_out = min(2, I.j1 - j);
+                int64_t pix[2];
+                uint4 mk[2][CO / 8];            // the pixels' mask, in flight while the MMAs run
 #pragma unroll
-                for (int qq = 0; qq < CO / 8; qq += 2) load32(mask + pix * CO + 8 * qq, mk[qq], mk[qq + 1], wide);
-            }
-            // at most 2^18 tries of at most 1 us each (the suspend-time hint): a quarter second
-            uint32_t done = 0;
-            const uint32_t parity = (uint32_t)(k >> 1) & 1u;
-            for (int it = 0; it < (1 << 18) && !done; ++it)
-                asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
-                             " selp.u32 %0, 1, 0, p;\n}\n"
-                             : "=r"(done) : "r"(smem_u32(s_bar + b)), "r"(parity) : "memory");
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (done) {
-                uint32_t v[CO];
-                tmem_ld_32x32b<CO>(tmem + 32u * b + ((uint32_t)(32 * warp) << 16), v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (EPI == kEpiLinearF32) {
-                    static_cast<float *>(out)[pix] = __uint_as_float(v[0]) + bias[0];
-                } else {
-                    uint4 o[CO / 8];
+                for (int r = 0; r < 2; ++r) {
+                    pix[r] = I.img0 + (int64_t)(I.rho + (j + r) * dil) * W + I.x0 + 32 * warp + lane;
+                    if (EPI == kEpiMaskBf16 && r < n_out) {
 #pragma unroll
-                    for (int qq = 0; qq < CO / 8; ++qq) {
-                        uint32_t packed[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int ch = 8 * qq + 2 * e;
-                            float v0 = __uint_as_float(v[ch]), v1 = __uint_as_float(v[ch + 1]);
-                            if (EPI == kEpiReluBf16) {
-                                v0 = fmaxf(v0 + s_bias[ch], 0.f);
-                                v1 = fmaxf(v1 + s_bias[ch + 1], 0.f);
-                            } else {
-                                const uint32_t mw = e == 0 ? mk[qq].x : e == 1 ? mk[qq].y : e == 2 ? mk[qq].z : mk[qq].w;
-                                const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162 *>(&mw);
-                                v0 = __bfloat162float(m2.x) > 0.f ? v0 : 0.f;
-                                v1 = __bfloat162float(m2.y) > 0.f ? v1 : 0.f;
-                            }
-                            const __nv_bfloat162 h2 = __floats2bfloat162_rn(v0, v1);
-                            packed[e] = *reinterpret_cast<const uint32_t *>(&h2);
-                        }
-                        o[qq] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+                        for (int qq = 0; qq < CO / 8; qq += 2) load32(mask + pix[r] * CO + 8 * qq, mk[r][qq], mk[r][qq + 1], wide);
                     }
+                }
+                if (!(ok = warp_wait(s_done + pair, (phase >> pair) & 1u))) break;
+                phase ^= 1u << pair;
+                tc_fence_after();
 #pragma unroll
-                    for (int qq = 0; qq < CO / 8; qq += 2) store32(static_cast<bf16 *>(out) + pix * CO + 8 * qq, o[qq], o[qq + 1], wide);
+                for (int r = 0; r < 2; ++r) {
+                    if (r >= n_out) break;
+                    uint32_t v[CO];
+                    tmem_ld_32x32b<CO>(tmem + (uint32_t)(CO * (2 * pair + r)) + ((uint32_t)(32 * warp) << 16), v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (r == n_out - 1) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) arrive(s_free + pair);
+                    }
+                    if (EPI == kEpiLinearF32) {
+                        static_cast<float *>(out)[pix[r]] = __uint_as_float(v[0]) + bias[0];
+                    } else {
+                        uint4 o[CO / 8];
+#pragma unroll
+                        for (int qq = 0; qq < CO / 8; ++qq) {
+                            uint32_t packed[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const int ch = 8 * qq + 2 * e;
+                                float v0 = __uint_as_float(v[ch]), v1 = __uint_as_float(v[ch + 1]);
+                                if (EPI == kEpiReluBf16) {
+                                    v0 = fmaxf(v0 + s_bias[ch], 0.f);
+                                    v1 = fmaxf(v1 + s_bias[ch + 1], 0.f);
+                                } else {
+                                    const uint32_t mw = e == 0 ? mk[r][qq].x : e == 1 ? mk[r][qq].y : e == 2 ? mk[r][qq].z : mk[r][qq].w;
+                                    const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162 *>(&mw);
+                                    v0 = __bfloat162float(m2.x) > 0.f ? v0 : 0.f;
+                                    v1 = __bfloat162float(m2.y) > 0.f ? v1 : 0.f;
+                                }
+                                const __nv_bfloat162 h2 = __floats2bfloat162_rn(v0, v1);
+                                packed[e] = *reinterpret_cast<const uint32_t *>(&h2);
+                            }
+                            o[qq] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+                        }
+#pragma unroll
+                        for (int qq = 0; qq < CO / 8; qq += 2) store32(static_cast<bf16 *>(out) + pix[r] * CO + 8 * qq, o[qq], o[qq + 1], wide);
+                    }
                 }
             }
-            // the next row's input has landed and this row's accumulator has been read
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            const int all_done = __syncthreads_and((int)done);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (!all_done) {                    // a wait gave up: report and stop this CTA
-                if (tid == 0) atomicExch(&g_tc_timeout, 1);
-                ok = false;
-                break;
-            }
-            if (tid == 0 && j + 1 < j1 && !withhold_mma) issue(j + 1, (k + 1) & 1, tmem);
         }
+        if (!ok && lane == 0) atomicExch(&g_tc_timeout, 1);
+    } else if (warp < 8) {                                       // copies
+        // thread: channel group c8 of the pixels px0, px0 + kStep, ..
+        constexpr int kStep = 128 / C8;
+        const int t = tid - 128, c8 = t % C8, px0 = t / C8;
+        int n = 0, slot = 0, given = 0;                          // steps issued, the next one's slot; the next to hand over
+        uint32_t parity = 1;                                     // of the slots' last release (none yet: passes)
+        bool ok = true;
+        for (int q = blockIdx.x; q < n_items && ok; q += gridDim.x) {
+            const ConvItem I = decode(q);
+            for (int i = I.j0 - 1; i <= I.j1; i += 2) {
+                if (!(ok = warp_wait(s_empty + slot, parity))) break;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    if (i + r < 0 || i + r > I.j1 || i + r >= I.J) continue;
+                    int xx = I.x0 + px0 - dil;
+                    const bf16 *src = in + (I.img0 + (int64_t)(I.rho + (i + r) * dil) * W + xx) * CI + c8 * 8;
+                    bf16 *dst = s_ring + (2 * slot + r) * row_elems + (c8 * plane + px0) * 8;
+#pragma unroll 3
+                    for (int px = px0; px < cols; px += kStep) {
+                        const bool inside = (unsigned)xx < (unsigned)W;          // zeros beside the image
+                        cp_async16_zfill(dst, inside ? src : in, inside ? 16 : 0);
+                        xx += kStep;
+                        src += kStep * CI;
+                        dst += kStep * 8;
+                    }
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                if (++slot == n_slots) { slot = 0; parity ^= 1u; }
+                if (++n > kConvAhead) {                          // the step kConvAhead back has landed
+                    asm volatile("cp.async.wait_group %0;" :: "n"(kConvAhead) : "memory");
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) arrive(s_full + given);
+                    if (++given == n_slots) given = 0;
+                }
+            }
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        fence_proxy_async_smem();
+        __syncwarp();
+        for (int k = min(n, kConvAhead); k > 0; --k) {
+            if (lane == 0) arrive(s_full + given);
+            if (++given == n_slots) given = 0;
+        }
+        // the MMAs' releases of the last steps arrive before the CTA ends
+        for (int b = min(n, n_slots); b > 0 && ok; --b) {
+            const int s = slot - b;                              // step n - b; < 0: of the round before
+            ok = warp_wait(s_empty + (s < 0 ? s + n_slots : s), s < 0 ? parity : parity ^ 1u);
+        }
+        if (!ok && t == 0) atomicExch(&g_tc_timeout, 1);
+    } else if (lane == 0 && !withhold_mma) {                     // MMAs
+        int slot = 0, base = 0;
+        uint32_t parity = 0, phase = 0xFFFFFFFFu;                // phase: parity of the pair's last release
+        const uint64_t w0 = umma_smem_desc(smem_u32(s_w), N * 16u, 128u);
+        bool ok = true;
+        for (int q = blockIdx.x; q < n_items && ok; q += gridDim.x) {
+            const ConvItem I = decode(q);
+            base = next_base(base, I);
+            const int i0 = max(I.j0 - 1, 0), i1 = min(I.j1, I.J - 1);
+            for (int i = I.j0 - 1; i <= I.j1; i += 2) {
+                const int pair = (base + i + 1 - I.j0) / 2;      // the output rows this step starts
+                if (i + 1 < I.j1) {
+                    if (!(ok = wait(s_free + pair, (phase >> pair) & 1u))) break;
+                    phase ^= 1u << pair;
+                }
+                if (!(ok = wait(s_full + slot, parity))) break;
+                tc_fence_after();
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int ii = i + r;
+                    if (ii < i0 || ii > i1) continue;
+                    const int lo = max(I.j0, ii - 1), hi = min(I.j1 - 1, ii + 1);
+                    const int fresh = ii == i0 ? lo : ii + 1;    // blocks from here on start with this row
+                    const uint64_t a = umma_smem_desc(smem_u32(s_ring + (2 * slot + r) * row_elems), (uint32_t)plane * 16u, 128u);
+                    auto mma = [&](int kx, int c0, int ja, int jb, int accumulate) {
+                        umma_bf16(tmem + (uint32_t)(CO * (base + ja - I.j0)), a + (uint32_t)((c0 / 8) * plane + kx * dil),
+                                  w0 + (uint32_t)((kx * C8 + c0 / 8) * N + (ja - ii + 1) * CO),
+                                  umma_idesc_bf16(kTW5, (jb - ja + 1) * CO), accumulate);
+                    };
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) {
+#pragma unroll
+                        for (int c0 = 0; c0 < CI; c0 += 16) {
+                            if (kx == 0 && c0 == 0) {
+                                if (fresh > lo) mma(0, 0, lo, min(hi, fresh - 1), 1);
+                                if (fresh <= hi) mma(0, 0, fresh, hi, 0);
+                            } else {
+                                mma(kx, c0, lo, hi, 1);
+                            }
+                        }
+                    }
+                }
+                umma_commit(s_empty + slot);
+                if (++slot == n_slots) { slot = 0; parity ^= 1u; }
+                if (i >= I.j0) umma_commit(s_done + pair - 1);   // the two before are complete
+            }
+        }
+        umma_commit(&s_end);                                     // none in flight when the memory is given back
+        mbar_wait_bounded(&s_end, 0, 1 << 18);
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncwarp();
+    tc_fence_before();
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" :: "r"(tmem) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(kCols) : "memory");
 }
 
 // Weight gradient partials: CTA c sums rows [c*rows, (c+1)*rows) of the B*H image rows, 64 pixels
@@ -736,55 +836,56 @@ cudaError_t launch_conv(const void *in, const void *w, const float *bias, const 
 }
 
 // The tensor-memory variant (W a multiple of 128): persistent CTAs over segments of
-// dilation-strided row chains.  Each CTA holds 64 TMEM columns; its shared-memory request is
-// at least 30 KB, so that at most 7 CTAs share an SM (448 of its 512 columns: an
-// allocation never waits).
+// dilation-strided row chains.  Each CTA holds at most 256 TMEM columns and asks for more than a
+// third of an SM's shared memory, so that at most two share an SM and an allocation never waits.
 template <int CI, int CO, int EPI>
 cudaError_t launch_conv_tc(const void *in, const void *w, const float *bias, const void *mask, void *out, int B,
                            int H, int W, int dil, cudaStream_t st) {
-    auto bytes = [](int d) {
-        const size_t b = sizeof(ddk::bf16) * ((size_t)9 * CI * CO + (size_t)4 * CI * ddk::conv_plane(d)) + 32;
-        return std::max<size_t>(b, 30 * 1024);
-    };
-    static bool configured = false;     // allow the largest dilation's staging area once
-    if (!configured) {
-        cudaError_t err = cudaFuncSetAttribute(ddk::conv3x3_tc_kernel<CI, CO, EPI>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(ddk::kMaxDil));
-        // the whole L1/shared array as shared memory: without this preference the occupancy
-        // query below counts a small shared-memory carveout and allows one CTA (4 warps) per
-        // SM, leaving the tensor pipe idle behind each CTA's copy and MMA waits
+    constexpr size_t kLeast = 77 * 1024, kMost = 112 * 1024;
+    const size_t w_bytes = sizeof(ddk::bf16) * 9 * CI * CO, slot = 2 * sizeof(ddk::bf16) * CI * ddk::conv_plane(dil);
+    const int n_slots = std::min<int>(ddk::kConvMaxSlots, (int)((kMost - w_bytes) / slot));
+    static_assert((kMost - sizeof(ddk::bf16) * 9 * CI * CO) / (2 * sizeof(ddk::bf16) * CI * ddk::conv_plane(ddk::kMaxDil)) > ddk::kConvAhead + 1,
+                  "slots at the largest dilation");
+    const size_t bytes = std::max(kLeast, w_bytes + n_slots * slot);
+    static std::atomic<uint64_t> configured{0};    // per device: the attributes are set
+    int dev = 0, sms = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (err != cudaSuccess) return err;
+    if (dev >= 64 || !(configured.load() & (uint64_t(1) << dev))) {
+        err = cudaFuncSetAttribute(ddk::conv3x3_tc_kernel<CI, CO, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(ddk::conv3x3_tc_kernel<CI, CO, EPI>,
                                        cudaFuncAttributePreferredSharedMemoryCarveout,
                                        (int)cudaSharedmemCarveoutMaxShared);
         if (err != cudaSuccess) return err;
-        configured = true;
+        if (dev < 64) configured.fetch_or(uint64_t(1) << dev);
     }
-    int dev = 0, sms = 0, smem_sm = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    if (err != cudaSuccess) return err;
-    // CTAs that fit one SM's shared memory (each also costs the runtime's 1 KB reserve);
-    // the occupancy query was seen to answer 1 here, which left 4 warps per SM
-    const int per = (int)((size_t)smem_sm / (bytes(dil) + 1024));
-    // items per (image, column tile): the segments of every residue chain rho < dil
-    int per_strip = 0;
-    for (int rho = 0; rho < dil; ++rho) {
-        const int J = (H - rho + dil - 1) / dil;
-        per_strip += (J + ddk::kSeg - 1) / ddk::kSeg;
+    // Rows per item: the length at which the CTA with the most items has the least to do; an item
+    // also reads two rows beside it (most of them from L2)
+    int seg = ddk::kSeg, per_strip = 0;
+    int64_t best = INT64_MAX;
+    for (int s = ddk::kSeg; s >= 3; --s) {
+        int items = 0;                             // per (image, column tile): the segments of every chain rho < dil
+        for (int rho = 0; rho < dil; ++rho) items += ((H - rho + dil - 1) / dil + s - 1) / s;
+        const int64_t n = (int64_t)B * (W / ddk::kTW5) * items, cost = (n + 2 * sms - 1) / (2 * sms) * (s + 1);
+        if (s == ddk::kSeg || (cost < best && n <= INT32_MAX)) {
+            best = cost;
+            seg = s;
+            per_strip = items;
+        }
     }
     const int n_items = B * (W / ddk::kTW5) * per_strip;
-    const int grid = std::max(1, std::min(n_items, sms * std::min(per, 7)));
+    const int grid = std::max(1, std::min(n_items, 2 * sms));
     // DD_FAULT=tc_wait (tests): no MMA is issued, so every completion wait runs out and the
     // timeout path (flag, no output, TMEM released) is exercised without a GPU fault
     const int withhold = dd::fault_injected("tc_wait") ? 1 : 0;
     // 32-byte accesses of the output and the mask (a multiple of 32 bytes per pixel) where both start
     // on one
     const bool wide = ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(mask)) & 31) == 0;
-    ddk::conv3x3_tc_kernel<CI, CO, EPI><<<grid, 128, bytes(dil), st>>>((const ddk::bf16 *)in, (const ddk::bf16 *)w, bias,
-                                                                        (const ddk::bf16 *)mask, out, H, W, dil,
-                                                                        per_strip, n_items, withhold, wide);
+    ddk::conv3x3_tc_kernel<CI, CO, EPI><<<grid, ddk::kConvThreads, bytes, st>>>(
+        (const ddk::bf16 *)in, (const ddk::bf16 *)w, bias, (const ddk::bf16 *)mask, out, H, W, dil, seg, per_strip,
+        n_items, n_slots, withhold, wide);
     return cudaGetLastError();
 }
 

@@ -419,9 +419,16 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
             return blocks * n_tiles / std::max(1, n_groups);
         };
         const int sb_min = grid_tiles ? 64 : 128;
-        while (sb > sb_min && waves4 > 0 && items_per_launch(sb) < waves4 &&
-               (size_t)((n_src + sb / 2 - 1) / (sb / 2)) * group * ((n_pts + 3) / 4 * 4) * sizeof(typename Cfg::Real) <= budget)
-            sb /= 2;
+        auto fits = [&](int b) {
+            return (size_t)((n_src + b - 1) / b) * group * ((n_pts + 3) / 4 * 4) * sizeof(typename Cfg::Real) <= budget;
+        };
+        while (sb > sb_min && waves4 > 0 && items_per_launch(sb) < waves4 && fits(sb / 2)) sb /= 2;
+        // and down to one stage while the launch leaves a quarter of the resident CTAs' places
+        // empty: the call then takes as long as one CTA's visits.  128 or 64 visits against
+        // this, in us: FP64, 593 points, 4 snapshots of 308 visits 2288, 665; mixed, 1290 points, 5 of
+        // 816: 76, 55; 2000 points, 40 of 2458: 205, 144; 32 x 32 points, 16 of 576: 81, 56.
+        // Above the line it depends: 1000 of 1216 places, 10,007 points 168, 182, 2000 points 228, 196.
+        while (sb > Cfg::kSTILE && 16 * items_per_launch(sb) < 3 * waves4 && fits(sb / 2)) sb /= 2;
     }
     const int nblk_max = (int)((n_src + sb - 1) / sb);
     const int n_chunks_max = (group + Cfg::kTCH - 1) / Cfg::kTCH;

@@ -43,17 +43,6 @@ FLOPS_SERIES = {2: 6.25, 4: 10.25, 8: 19.25, 12: 27.25}
 FLOPS_GENERAL = 56.25
 FLOPS_ZERO = 1.25
 MUFU_SERIES, MUFU_GENERAL = 1.0, 4.0
-# The same on a grid tile (128 columns x 4 rows x 4 snapshots, dd_field_on_grid): dx and
-# dx^2 cost 2 flops per (column, visit), shared by 16 pairs (0.125); rho^2 = dx^2 + dy^2 one
-# FMA per (point, visit), shared by 4 snapshots (0.5).  A degree-2 pair is X Y (+ A B):
-# the column factor X = 2^(g_0 + g_1x dx^2 + g_2x dx^4) costs 2 FMAs and one ex2 per
-# (column, visit, snapshot), shared by the 4 rows (1 flop, 0.25 ex2 per pair); the row
-# factor Y is shared by 128 columns (~0.02 flops, 0.008 ex2); the pair itself one FMA (2
-# flops); where the cross term is needed, A = X (2 ln2 g_2x) dx^2 (3 multiplies per
-# column, visit and snapshot: 0.75) and one more FMA (2).  Higher degrees as above with
-# the grid's rho^2 (0.625 instead of 1.25).
-GRID_FLOPS_SEP1, GRID_FLOPS_SEP2, GRID_MUFU_SEP = 3.17, 5.92, 0.258
-GRID_FLOPS_RHO, GRID_FLOPS_ZERO = 0.625, 0.125
 # FP32 peak from the unit counts and the maximum clock: 152 SMs x 128 lanes x 2 x 2.07 GHz.
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # FP64 FMA peak: 1.6 per clock per SM (a microbenchmark on this GPU: 0.50 T DFMA/s at
@@ -188,9 +177,8 @@ def whole_job(job_pairs_per_step, steps, rank_total_ms, dist=None, device=None):
 # Per kernel: the ncu summary under profiles/ that records its DRAM traffic, and the
 # sources whose text fixes its code (the summary's source_sha is their hash).
 PROFILED = {
-    "field_mixed": ("field_mixed_raster64.md", ("dd_field_impl.cuh", "dd_e1.cuh", "dd_coef.cuh")),
-    "field_grid_mixed": ("field_grid_mixed_raster64.md",
-                         ("dd_field_grid.cuh", "dd_field_impl.cuh", "dd_e1.cuh", "dd_coef.cuh")),
+    "field_mixed": ("field_mixed_points64.md", ("dd_field_impl.cuh", "dd_e1.cuh", "dd_coef.cuh")),
+    "field_grid_tc": ("field_grid_quad_grid256.md", ("dd_grid_quad.cuh", "dd_umma.cuh")),
 }
 
 
@@ -227,69 +215,40 @@ def recorded_traffic(kernel):
 
 def recorded_pipes(kernel):
     """Pipe and issue utilisation of the committed ncu capture (fractions), if taken on this
-    source: what the kernel keeps busy, beside the algorithmic fraction of the roofline."""
+    source: what the kernel keeps busy."""
     vals = recorded_profile(kernel)
-    keys = {"fma_pipe_pct": "fma_pipe", "xu_pipe_pct": "xu_pipe", "issue_active_pct": "issue_active"}
-    try:
-        out = {name: float(vals[k]) / 100.0 for k, name in keys.items()}
-        out["thread_instructions_per_pair"] = float(vals["thread_instructions_per_pair"])
-    except (KeyError, ValueError):
+    keys = {"tensor_pipe_pct": "tensor_pipe", "fma_pipe_pct": "fma_pipe", "xu_pipe_pct": "xu_pipe",
+            "issue_active_pct": "issue_active"}
+    out = {name: float(vals[k]) / 100.0 for k, name in keys.items() if k in vals}
+    if not out:
         return None
     out["note"] = ("ncu --set full capture of one launch on this source (profiles/%s): pipe busy "
                    "fractions and issue-slot use per SM sub-partition" % PROFILED[kernel][0])
     return out
 
 
-# BF16 tensor-core peak: the measured cuBLAS burst figure, else the recipe's fallback
-def bf16_peak_tflops():
+def grid_kernel_lines(prof):
+    """The grid field's kernels by their own events: launches and mean time.  field_grid_tc and
+    field_grid_tc4 (the Gauss-Legendre contraction's two launches, the rows of k with one or two
+    nodes and the rest) and field_grid_mixed (the most recent visits) overlap one another on two
+    streams; field_reduce sums the segments of lags that the raster's snapshots share."""
+    names = ("coef_mixed", "field_grid_tc", "field_grid_tc4", "field_grid_mixed", "field_reduce")
+    return {k: {"launches": prof[k][0], "avg_launch_ms": prof[k][1] / prof[k][0]} for k in names if prof.get(k, (0,))[0]}
+
+
+def hbm_peak_gbs():
+    """The measured copy bandwidth, else the stated fallback (6.8 TB/s)."""
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-            return float(json.load(f)["bf16_tflops"]), "measured (cuBLAS bf16 burst, MEASURED_PEAKS.json)"
+            return float(json.load(f)["hbm_gbs"]), "measured copy bandwidth (MEASURED_PEAKS.json)"
     except (OSError, KeyError, ValueError):
-        return 1900.0, "fallback (1.9 PFLOP/s bf16)"
+        return 6800.0, "fallback (6.8 TB/s)"
 
 
-def tensor_core_line(prof, kernel, tc_pairs, flops_per_pair):
-    """A tensor-core contraction of the grid field: field_grid_tc (degree 2: 7 BF16 MMAs of 2
-    flops per (row, column, visit) triple, 14 tensor flops per pair-term) or field_grid_tc4
-    (degree 4: 12 MMAs, 24 flops).  Its event time runs from its launch on the side stream to
-    its end, overlapping the CUDA-core tile kernel (whose CTAs are placed first), so the rate
-    below is a lower bound of what it does alone."""
-    n, ms = prof.get(kernel, (0, 0.0))
-    if not n or not tc_pairs:
-        return None
-    avg = ms / n
-    peak, note = bf16_peak_tflops()
-    achieved = flops_per_pair * tc_pairs / (avg / 1e3) / 1e12
-    return {"kernel": kernel, "bound": "tensor", "pairs_per_launch": tc_pairs, "flops_per_pair": flops_per_pair,
-            "avg_launch_ms": avg, "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "peak_note": note, "note": "event time overlaps the CUDA-core tile kernel (side stream)"}
-
-
-def cumulant_l2(r):
-    """l_2 of the FP32 record's exponent series (half the variance of s under the weight
-    r / (1 + r s) on [0, 1]), by a 2000-node midpoint rule: enough to place a pair in the
-    degree-2 class with or without the cross term."""
-    sg = (np.arange(2000) + 0.5) / 2000
-    out = np.empty(len(r))
-    for k0 in range(0, len(r), 4096):
-        rr = r[k0:k0 + 4096, None]
-        wgt = rr / (1 + rr * sg[None, :])
-        m0 = wgt.mean(1)
-        m1 = (wgt * sg).mean(1) / m0
-        m2 = (wgt * sg ** 2).mean(1) / m0
-        out[k0:k0 + 4096] = 0.5 * (m2 - m1 ** 2)
-    return out
-
-
-def ops_per_pair(job, samples=400_000, seed=5, grid=False, prefix=None):
-    """Algorithmic FP32 FLOPs and MUFU operations per pair-term of the field kernel on this
-    workload: the cost of the cheapest path that meets the FP32 accuracy target for each
-    pair (series degree from that pair's own h, zero when a >= 87; on a grid, the degree-2
-    pairs in their separable form, with the cross term where its size 2 g_2x dx^2 dy^2
-    exceeds the 2.5e-7 budget), averaged over seeded pairs.  prefix[j]: visits of snapshot
-    j that the tensor-core contraction takes (the CUDA-core tile kernel sums the rest; the
-    pairs sampled here are its pairs)."""
+def ops_per_pair(job, samples=400_000, seed=5):
+    """Algorithmic FP32 FLOPs and MUFU operations per pair-term of the point-list field kernel on
+    this workload: the cost of the cheapest path that meets the FP32 accuracy target for each
+    pair (series degree from that pair's own h, zero when a >= 87), averaged over seeded pairs."""
     from paper_2507_00294_gb300 import workloads as w
     s = job.scan
     rng = np.random.default_rng(seed)
@@ -298,8 +257,7 @@ def ops_per_pair(job, samples=400_000, seed=5, grid=False, prefix=None):
     it = rng.integers(0, len(job.times), samples)
     t = job.times[it]
     nact = np.searchsorted(ts, t, side="left")
-    k0 = np.zeros(samples, np.int64) if prefix is None else np.asarray(prefix, np.int64)[it]
-    i = k0 + (rng.random(samples) * (nact - k0)).astype(np.int64)
+    i = (rng.random(samples) * nact).astype(np.int64)
     ip = rng.integers(0, len(job.pts_xy), samples)
     g = i                                        # raster: visit k is grid index k
     dx = job.pts_xy[ip, 0] - (g % s.nx) * s.pitch_m
@@ -317,18 +275,7 @@ def ops_per_pair(job, samples=400_000, seed=5, grid=False, prefix=None):
                                    np.where(h <= 1.25, FLOPS_SERIES[8],
                                             np.where(h <= 2.0, FLOPS_SERIES[12], FLOPS_GENERAL)))))
     m = np.where(zero, 0.0, np.where(h <= 2.0, MUFU_SERIES, MUFU_GENERAL))
-    if grid:
-        # grid tile: rho^2 shared more widely, degree 2 in the separable form
-        dqp = (1.0 / w0 - 1.0 / w1) * s.pitch_m ** 2                     # dq in pitch units
-        rr = np.where(dt <= tau, 4 * D * dt, 4 * D * tau) / w0             # r = w1 / w0 - 1
-        d2 = h <= 0.04
-        cross = np.zeros(samples)
-        cross[d2] = (2 * 1.4426950408889634 * cumulant_l2(rr[d2]) * dqp[d2] ** 2
-                     * (dx[d2] / s.pitch_m) ** 2 * (dy[d2] / s.pitch_m) ** 2)
-        sep = np.where(cross <= 2.5e-7, GRID_FLOPS_SEP1, GRID_FLOPS_SEP2)
-        f = np.where(zero, GRID_FLOPS_ZERO, np.where(d2, sep, f - FLOPS_ZERO + GRID_FLOPS_RHO))
-        m = np.where(zero, 0.0, np.where(d2, GRID_MUFU_SEP, m))
-    wgt = (nact - k0).astype(np.float64)         # pairs are sampled per snapshot: weight by their count
+    wgt = nact.astype(np.float64)                # pairs are sampled per snapshot: weight by their count
     return (float(np.sum(f * wgt) / np.sum(wgt)), float(np.sum(m * wgt) / np.sum(wgt)),
             float(np.sum(zero * wgt) / np.sum(wgt)))
 
@@ -337,7 +284,7 @@ def dfma_per_pair_fp64(job, samples=200_000, seed=6):
     """Algorithmic FP64 operations (DFMA-equivalents) per pair of the FP64 field kernel on
     this workload: rho^2 shared by the 4 snapshots of a chunk (1), the moment polynomial of
     the cheapest degree whose range holds the pair's h (4, 8, 11, 15 up to h = 1e-3, 0.052,
-    0.19, 0.5: D + 1 with the final product), exp(-a) as 15, the two-E1 path as 60, a pair
+    0.19, 0.5: D + 1 with the final product), exp(-a) as 10, the two-E1 path as 60, a pair
     with a >= 745 its rho^2 only."""
     from paper_2507_00294_gb300 import workloads as w
     s = job.scan
@@ -357,57 +304,9 @@ def dfma_per_pair_fp64(job, samples=200_000, seed=6):
     w1 = 2 * Ds + 4 * D * dt
     w0 = np.where(dt <= tau, 2 * Ds, 2 * Ds + 4 * D * (dt - tau))
     a, h = rho2 / w1, rho2 / w0 - rho2 / w1
-    c = np.where(a >= 745, 1.0, np.where(h <= 1e-3, 1 + 5 + 15, np.where(h <= 0.052, 1 + 9 + 15,
-                 np.where(h <= 0.19, 1 + 12 + 15, np.where(h <= 0.5, 1 + 16 + 15, 1 + 60)))))
+    c = np.where(a >= 745, 1.0, np.where(h <= 1e-3, 1 + 5 + 10, np.where(h <= 0.052, 1 + 9 + 10,
+                 np.where(h <= 0.19, 1 + 12 + 10, np.where(h <= 0.5, 1 + 16 + 10, 1 + 60)))))
     return float(np.sum(c * nact) / np.sum(nact))
-
-
-# Batch grid tile (32 x 32 points, one snapshot, 8 rows per thread): a degree-2 pair is one
-# FMA (2 flops) plus its share of the column factor X (2 FMAs and one ex2 per column and
-# visit, shared by 8 rows: 0.5 flops, 0.125 ex2) and of dx, dx^2 (0.25); with the cross term
-# A = X (2 ln2 g_2x) dx^2 (3 multiplies / 8 = 0.375) and one more FMA (2); degree 4 and above
-# per point with rho^2 = dx^2 + dy^2 (one FMA, 2 flops).
-# per class: zero (a >= 87), degree 2 without / with the cross term, degree 4, 8, 12, two E1
-BATCH_FLOPS = np.array([0.25, 2.75, 5.125, 2.0 + 8.0 + 1.0, 2.0 + 17.0 + 1.0, 2.0 + 25.0 + 1.0, 2.0 + 55.0])
-BATCH_MUFU = np.array([0.0, 0.125, 0.125, 1.0, 1.0, 1.0, 4.0])
-
-
-def batch_ops_per_pair(jobs, samples=200_000, seed=7, prefix=None):
-    """Algorithmic FP32 flops and ex2 per pair-term of the batch grid kernel on the 512-scan
-    workload (each pair at the cheapest class its own h allows, degree 2 with the cross term
-    where 2 g_2x dx^2 dy^2 exceeds 2.5e-7), pairs sampled in proportion to each scan's.
-    prefix[k]: visits of scan k that the tensor-core contraction takes (the pairs sampled
-    are then the CUDA-core tile kernel's own)."""
-    from paper_2507_00294_gb300 import binding as b
-    from paper_2507_00294_gb300 import workloads as w
-    rng = np.random.default_rng(seed)
-    k0 = np.zeros(len(jobs), np.int64) if prefix is None else np.asarray(prefix, np.int64)
-    pairs = np.array([(w.n_visits(j.scan) - k0[k]) * len(j.pts_xy) for k, j in enumerate(jobs)], dtype=np.float64)
-    ks = rng.choice(len(jobs), samples, p=pairs / pairs.sum())
-    code = np.empty(samples, dtype=np.int64)
-    for k in np.unique(ks):
-        sel = np.nonzero(ks == k)[0]
-        j = jobs[k]
-        s = j.scan
-        sc = b.Scan(s)
-        g = sc.visits()[0].astype(np.int64)
-        sc.close()
-        nv = len(g)
-        i = rng.integers(k0[k], nv, len(sel))
-        ip = rng.integers(0, len(j.pts_xy), len(sel))
-        dx = j.pts_xy[ip, 0] / s.pitch_m - g[i] % s.nx
-        dy = j.pts_xy[ip, 1] / s.pitch_m - g[i] // s.nx
-        rho2 = dx * dx + dy * dy
-        kap, ss = s.D_m2s * s.dwell_s / s.pitch_m ** 2, (s.sigma_m / s.pitch_m) ** 2
-        L = (nv - i).astype(np.float64)                  # lag of visit i at the scan's end
-        w1 = 2 * ss + 4 * kap * L
-        w0 = 2 * ss + 4 * kap * (L - 1)
-        dq = 1 / w0 - 1 / w1
-        a, h = rho2 / w1, rho2 * dq
-        cross = 2 * 1.4426950408889634 * cumulant_l2(4 * kap / w0) * dq ** 2 * dx ** 2 * dy ** 2
-        code[sel] = np.where(a >= 87, 0, np.where(h <= 0.04, np.where(cross <= 2.5e-7, 1, 2),
-                             np.where(h <= 0.33, 3, np.where(h <= 1.25, 4, np.where(h <= 2.0, 5, 6)))))
-    return float(BATCH_FLOPS[code].mean()), float(BATCH_MUFU[code].mean())
 
 
 def dose_ops_per_pair(spec, samples=200_000, seed=9):
@@ -463,14 +362,17 @@ def bench_dose(b, dev, stream, job, n, reps=10):
         ms = sum(v[1] for v in prof.values()) / reps
         kl, kms = prof.get("dose_mixed", (0, 0.0))
         pairs = nv * (nv - 1) // 2
+        # a uniform raster's doses are running sums over rows of 2 n distinct pair terms
+        terms = 2 * nv
         fpp, mpp = dose_ops_per_pair(spec)
-        krate = pairs / (kms / max(1, kl) / 1e3) if kl else None
+        krate = terms / (kms / max(1, kl) / 1e3) if kl else None
         out[name] = {"visits": nv, "pairs": pairs, "ms": ms, "value": pairs / (ms / 1e3), "unit": UNIT,
                      "roofline": {"bound": "alu", "kernel": "dose_mixed", "pipe": "fp32",
                                   "achieved": fpp * krate / 1e12 if krate else None, "peak": FP32_PEAK_TFLOPS,
                                   "unit": "TFLOP/s", "frac": fpp * krate / 1e12 / FP32_PEAK_TFLOPS if krate else None,
                                   "mufu_frac": mpp * krate / 1e12 / MUFU_PEAK_TOPS if krate else None,
-                                  "ops_per_pair": round(fpp, 2), "mufu_per_pair": round(mpp, 3),
+                                  "terms": terms, "ops_per_pair": round(fpp, 2), "mufu_per_pair": round(mpp, 3),
+                                  "note": "distinct pair terms of the raster; latency-bound at this size",
                                   "avg_launch_ms": kms / max(1, kl)}}
         scan.close()
     return out
@@ -572,44 +474,21 @@ def bench_batched(dev, stream, runs=10, rank=0, world=1, dist=None, grid=True):
     plan.close()
     roof = None
     if grid and world == 1:
-        # the plan's split: the tensor-core contraction takes each scan's prefix on the
-        # degree-2 (and then degree-4) series at every point of its grid (grids of at least
-        # 64 x 64 points), the CUDA-core tile kernel the rest
-        k2, k4 = [], []
-        for j in jobs_all:
-            sc = b.Scan(j.scan)
-            K, K2 = b.dd_field_grid_split(sc, 0.0, 0.0, j.scan.pitch_m, j.scan.pitch_m, j.scan.nx, j.scan.ny,
-                                          j.times[:1], degree2=True)
-            sc.close()
-            k2.append(int(K2[0]))
-            k4.append(int(K[0]))
-        npts = np.array([len(j.pts_xy) for j in jobs_all], dtype=np.float64)
-        tc2 = float(np.sum(np.array(k2) * npts))
-        tc4 = float(np.sum((np.array(k4) - np.array(k2)) * npts))
-        core = total_pairs - tc2 - tc4
-        fpp, mpp = batch_ops_per_pair(jobs_all, prefix=k4)
-        t_run = ms_total / runs / 1e3
-        rate = core / t_run
-        bf16, bf16_note = bf16_peak_tflops()
-        roof = {"bound": "alu", "kernel": "batch_grid_mixed_32x32", "pipe": "fp32", "achieved": fpp * rate / 1e12,
-                "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": fpp * rate / 1e12 / FP32_PEAK_TFLOPS,
-                "pairs_per_run": core, "ops_per_pair": round(fpp, 3), "mufu_per_pair": round(mpp, 4),
-                "mufu_frac": mpp * rate / 1e12 / MUFU_PEAK_TOPS,
-                "note": "the CUDA-core tile kernel's own pairs over the event time of the whole graph "
-                        "(coefficients, contraction, tile kernel, reduce, one after another): a lower bound "
-                        "of that kernel's rate",
-                "tensor_core": {"pairs_per_run": tc2 + tc4, "degree2_pairs": tc2, "degree4_pairs": tc4,
-                                "flops_per_run": 14 * tc2 + 24 * tc4,
-                                "achieved": (14 * tc2 + 24 * tc4) / t_run / 1e12, "peak": bf16, "unit": "TFLOP/s",
-                                "frac": (14 * tc2 + 24 * tc4) / t_run / 1e12 / bf16, "peak_note": bf16_note,
-                                "note": "over the whole graph's event time: a lower bound"}}
+        # what a run cannot do without in memory: the field it writes (FP64)
+        peak, note = hbm_peak_gbs()
+        out_bytes = 8.0 * sum(len(j.pts_xy) for j in jobs_all)
+        gbs = out_bytes / (ms_total / runs / 1e3) / 1e9
+        roof = {"bound": "hbm", "kernel": "batch_grid_mixed", "achieved": gbs, "peak": peak, "unit": "GB/s",
+                "frac": gbs / peak, "bytes_per_run": out_bytes, "peak_note": note,
+                "note": "the field's bytes over the event time of the whole graph (coefficients, contraction, "
+                        "recent visits); the time is the factors' arithmetic and the recent visits, not memory"}
     return {"value": value, "unit": UNIT, "ms_per_run": ms_total / runs, "runs": runs, "roofline": roof,
             "pairs_per_run": total_pairs, "rank_pairs_per_run": info["pairs"], "scans": len(jobs_all),
             "rank_scans": len(jobs), "work_items": info["items"], "tuned_variant": variant,
             "workload": "512 scans, n ~ U{32..128}, D log-U[1e-15,1e-12], "
             "dwell log-U[1e-7,1e-5] s, sigma U[0.05,0.2] nm, keep U[0.1,1], random order, final field on the n x n grid",
-            "points": "each scan's probe grid, dd_batch_create_grid (older visits of grids >= 64 x 64 on "
-                      "the tensor cores, the rest in 32 x 32 grid tiles)" if grid
+            "points": "each scan's probe grid, dd_batch_create_grid (older visits on the tensor cores, the "
+                      "most recent ones in 32 x 16 grid tiles)" if grid
                       else "each scan's probe grid as a point list (512-point tiles)",
             "launch": "persistent kernel, atomic work claim, CUDA graph replay" +
                       (", scans split over %d GPUs longest-first, one gather per run" % world if world > 1 else "")}
@@ -838,13 +717,6 @@ def run_ours(args):
     out = torch.empty((len(mine), n_pts), dtype=torch.float64, device=dev)
     dose = torch.empty(j1 - j0, dtype=torch.float64, device=dev)
     rank_field_pairs = int(nact_t[mine].sum()) * n_pts
-    # the split of the rank's field between the tensor-core contraction (the older visits'
-    # degree-2 terms) and the CUDA-core tile kernel (the rest), as the library plans it
-    tc_prefix, tc_prefix2 = b.dd_field_grid_split(scan, x0, y0, gdx, gdy, W, H, times_r, degree2=True)
-    rank_tc_pairs = int(tc_prefix.sum()) * n_pts
-    rank_tc2_pairs = int(tc_prefix2.sum()) * n_pts
-    rank_core_pairs = rank_field_pairs - rank_tc_pairs
-
     # The field and the dose are independent calls: the dose goes on a side stream that forks
     # from the step's stream and joins it again, submitted after the field so that its short
     # kernels fill the SMs the field's kernels leave at their tail instead of delaying their
@@ -894,36 +766,17 @@ def run_ours(args):
     if dist is not None:
         dist.barrier()
 
-    # roofline of the dominant kernel (field_grid_mixed, the CUDA-core tile kernel: the
-    # critical path of the field), from its own events in the timed region, over the pairs it
-    # sums (those the tensor-core contraction leaves)
-    fl, fms = prof.get("field_grid_mixed", (0, 0.0))
-    avg_ms = fms / max(1, fl)
-    fpp, mpp, culled = ops_per_pair(job, grid=True, prefix=tc_prefix if world == 1 else None)
-    rate = rank_core_pairs / (avg_ms / 1e3) if fl else None
-    traffic = recorded_traffic("field_grid_mixed")
-    # the pair term needs FP32 issue and one MUFU ex2: report the pipe this algorithm's mix
-    # binds (the larger fraction), with the other beside it
-    fp32 = {"achieved": fpp * rate / 1e12 if rate else None, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "per_pair": round(fpp, 3),
-            "peak_note": "FP32 FMA: 152 SMs x 128 lanes x 2 flop x 2070 MHz (nominal max clock)"}
-    mufu = {"achieved": mpp * rate / 1e12 if rate else None, "peak": MUFU_PEAK_TOPS, "unit": "TOP/s",
-            "per_pair": round(mpp, 4),
-            "peak_note": "MUFU ex2: 152 SMs x 32 per clock x 2070 MHz"}
-    for x in (fp32, mufu):
-        x["frac"] = x["achieved"] / x["peak"] if x["achieved"] else None
-    bind, other = (mufu, fp32) if (mufu["frac"] or 0) >= (fp32["frac"] or 0) else (fp32, mufu)
-    roofline = {"bound": "alu", "kernel": "field_grid_mixed", "pipe": "mufu" if bind is mufu else "fp32",
-                "achieved": bind["achieved"], "peak": bind["peak"], "unit": bind["unit"], "frac": bind["frac"],
-                "traffic": traffic, "avg_launch_ms": avg_ms, "pairs_per_launch": rank_core_pairs,
-                "kernel_pairs_per_s": rate, "ops_per_pair": bind["per_pair"], "peak_note": bind["peak_note"],
-                "culled_pair_fraction": round(culled, 5),
-                "culled_note": "pair-terms with a >= 87 (below the FP32 normal range) are counted in the "
-                               "pair-terms but skipped per warp; their share of this kernel's pairs",
-                "other_pipe": {"pipe": "fp32" if bind is mufu else "mufu", **other},
-                "ncu_capture": recorded_pipes("field_grid_mixed"),
-                "tensor_core": [tensor_core_line(prof, "field_grid_tc", rank_tc2_pairs, 14),
-                                tensor_core_line(prof, "field_grid_tc4", rank_tc_pairs - rank_tc2_pairs, 24)]}
+    # The field's floor is the field it writes: its pair terms are formed once per lag and shared
+    # by the snapshots, a small fraction of the FP32 and tensor peaks.  The kernels beside it by
+    # their own events, and the pipes of the contraction from the committed capture.
+    peak, peak_note = hbm_peak_gbs()
+    out_bytes = 8.0 * len(mine) * n_pts + 8.0 * (j1 - j0)
+    gbs = out_bytes / (total_ms / args.steps / 1e3) / 1e9
+    roofline = {"bound": "hbm", "kernel": "field_grid", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
+                "bytes_per_step": out_bytes, "peak_note": peak_note,
+                "note": "field and dose bytes over the whole step; the step is a chain of short kernels, "
+                        "bound by their latency",
+                "kernels": grid_kernel_lines(prof), "ncu_capture": recorded_pipes("field_grid_tc")}
     launches = int(sum(v[0] for v in prof.values()))
     # shares of the summed per-launch event time (the dose's kernels run beside the field's,
     # so their events overlap and the shares do not add up to wall time)
@@ -937,6 +790,8 @@ def run_ours(args):
                    "D 6e-14 m^2/s, Q0 1 u/s, dwell 1 us", "points": n_pts,
                    "snapshots": len(times), "visits": n, "pairs_per_step": pairs_step,
                    "field_pairs": field_pairs, "dose_pairs": dose_pairs, "precision": "mixed",
+                   "pairs_note": "the terms of the sums as defined; a raster's snapshots and doses share "
+                                 "distinct terms by symmetry, so fewer are formed",
                    "l2": "flushed between steps (256 MB write, outside the timed events)",
                    "parallelism": ("points and dose targets split over %d GPUs, one all-gather per step"
                                    % world) if world > 1 else "single GPU"},
@@ -975,7 +830,7 @@ def run_ours(args):
                 "peak_note": "FP64 FMA: 1.6 per clock per SM measured by a microbenchmark on this GPU (0.50 T/s "
                              "at 1.995 GHz), x 152 SMs x 2070 MHz",
                 "ops_note": "per pair: rho^2 shared by 4 snapshots (1), the moment polynomial of the warp's "
-                            "degree (4 / 8 / 11 / 15 from the pair's own h: D + 1), exp(-a) counted as 15 "
+                            "degree (4 / 8 / 11 / 15 from the pair's own h: D + 1), exp(-a) counted as 10 "
                             "DFMA-equivalents, 60 for a two-E1 pair"}
         line["mixed_over_fp64"] = value / v64
         line["e2e"] = bench_e2e(args, b, shard, job, times, n, pairs_step, rank, world, dist, dev, sets, dr)

@@ -174,7 +174,7 @@ def whole_job(job_pairs_per_step, steps, rank_total_ms, dist=None, device=None):
     return job_pairs_per_step * steps / (total_ms / 1e3), total_ms, world
 
 
-# Per kernel: the ncu summary under profiles/ that records its DRAM traffic, and the
+# Per kernel: the ncu summary under profiles/ that records its pipe use, and the
 # sources whose text fixes its code (the summary's source_sha is their hash).
 PROFILED = {
     "field_mixed": ("field_mixed_points64.md", ("dd_field_impl.cuh", "dd_e1.cuh", "dd_coef.cuh")),
@@ -203,14 +203,6 @@ def recorded_profile(kernel):
     if vals.get("kernel") != kernel or vals.get("source_sha") != kernel_source_sha(kernel):
         return {}
     return vals
-
-
-def recorded_traffic(kernel):
-    """DRAM bytes per launch from the committed ncu summary, if taken on this source."""
-    try:
-        return int(recorded_profile(kernel)["dram_bytes_per_launch"])
-    except (KeyError, ValueError):
-        return None
 
 
 def recorded_pipes(kernel):
@@ -971,7 +963,7 @@ def bench_point_list(b, job, times, scan, dev, stream, flush, field_pairs, reps=
     return {"kernel": "field_mixed", "avg_launch_ms": avg_ms, "kernel_pairs_per_s": rate,
             "mufu_frac": mpp * rate / 1e12 / MUFU_PEAK_TOPS, "fp32_frac": fpp * rate / 1e12 / FP32_PEAK_TFLOPS,
             "ops_per_pair": {"flops": round(fpp, 3), "mufu": round(mpp, 4)},
-            "traffic": recorded_traffic("field_mixed")}
+            "ncu_capture": recorded_pipes("field_mixed")}
 
 
 def main():

@@ -6,8 +6,8 @@
 // on degree 2.  sort_points_block orders up to kSortPts points of a list along a Morton curve of
 // their own bounding box (16 bits; ties keep the caller's order, so the result is deterministic)
 // with a bitonic sort, and deals them out so that each warp of a 512-point tile (128 threads x 4
-// points, thread t holding the points t + 128 k) holds 128 consecutive ones; the reduce writes
-// the field back through the permutation.  A warp holds 64 keys in registers, so that only the
+// points, thread t holding the points t + 128 k) holds 128 consecutive ones (in a list's last, partial
+// tile, up to four runs of 32); the reduce writes the field back through the permutation.  A warp holds 64 keys in registers, so that only the
 // steps across warps (15 of 66) go through shared memory and barriers.  It reads the
 // float-float points (an FP64 pass over 4096 points takes one SM 10 us).  2048 points per CTA:
 // with 4096 the sort took 28 us of the 50 it saved (one SM's shuffles).  33 snapshots of a

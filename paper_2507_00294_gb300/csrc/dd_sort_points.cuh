@@ -7,11 +7,12 @@
 // their own bounding box (16 bits; ties keep the caller's order, so the result is deterministic)
 // with a bitonic sort, and deals them out so that each warp of a 512-point tile (128 threads x 4
 // points, thread t holding the points t + 128 k) holds 128 consecutive ones (in a list's last, partial
-// tile, up to four runs of 32); the reduce writes the field back through the permutation.  A warp holds 64 keys in registers, so that only the
-// steps across warps (15 of 66) go through shared memory and barriers.  It reads the
-// float-float points (an FP64 pass over 4096 points takes one SM 10 us).  2048 points per CTA:
-// with 4096 the sort took 28 us of the 50 it saved (one SM's shuffles).  33 snapshots of a
-// 2457-visit random scan on 10,007 random points: 284 us in the caller's order, 260 us in this one
+// tile, up to four runs of 32); the reduce writes the field back through the permutation.  A warp
+// holds 64 keys in registers, so that only the steps across warps (15 of 66) go through shared
+// memory and barriers.  It reads the float-float points (an FP64 pass over 4096 points takes one
+// SM 10 us).  2048 points per CTA: with 4096 the sort took 28 us of the 50 it saved (one SM's
+// shuffles).  33 snapshots of a 2457-visit random scan on 10,007 random points: 284 us in the
+// caller's order, 260 us in this one
 // (sort 16 us, field kernel 258 to 209 us); a batch of 256 scans on 997 random points each 774
 // and 667 us.
 #pragma once

@@ -222,6 +222,7 @@ struct GqSmem {
     int failed;
 };
 constexpr float kGqUnbias = 1.0f + 0x1p-22f;
+constexpr float kGqFarExp = 150.0f;         // q rho^2 from which a row of k is left out
 constexpr int kGqSmemBytes = (int)sizeof(GqSmem) + 1024;
 static_assert(kGqSmemBytes <= 227 * 1024, "shared memory of a CTA");
 
@@ -493,15 +494,24 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
                     }
                 }
                 // p = floor(q dxmin^2) moves from the row factor's exponent to the column
-                // factor's; m: the piece's largest row exponent
+                // factor's; m: the piece's largest row exponent.  A row of k whose term is below
+                // the FP32 range at every point of the tile (w < 2, so 2^-150 is) turns into
+                // padding: its exponents would be differences of numbers that FP32 no longer
+                // holds to within one, and its factors could pass FP16's range.
                 float m = -3e38f;
 #pragma unroll
                 for (int u = 0; u < kPer; ++u) {
                     const float dx = fmaxf(0.0f, fmaxf(x_a - vx[u], vx[u] - x_b));
                     const float dy = fmaxf(0.0f, fmaxf(y_a - vy[u], vy[u] - y_b));
-                    p[u] = fminf(floorf(q[u] * (dx * dx)), 1e30f);
+                    const float ex = q[u] * (dx * dx), ey = q[u] * (dy * dy);
+                    if (!(ex + ey <= kGqFarExp)) {
+                        q[u] = vx[u] = vy[u] = wf[u] = 0.0f;
+                        g[u] = -INFINITY;
+                        continue;
+                    }
+                    p[u] = floorf(ex);
                     g[u] -= p[u];
-                    m = fmaxf(m, floorf(fmaxf(g[u] + wf[u] - fminf(q[u] * (dy * dy), 1e30f), -3e30f)));
+                    m = fmaxf(m, floorf(fmaxf(g[u] + wf[u] - ey, -3e30f)));
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));

@@ -257,7 +257,8 @@ typedef struct dd_batch dd_batch;
    dd_batch_run and dd_batch_tune then take pts_xy_m = NULL.  In FP32-mixed precision every
    scan is summed as dd_field_on_grid sums it on large grids, with the
    same completion waits and NaN-on-timeout rule (dd_field_check); the
-   result differs from the point-list plan by FP32 rounding only.  Errors: DD_EINVAL (sizes,
+   result differs from the point-list plan by FP32 rounding only (a plan with a side of 2^30
+   columns or rows or more is summed as the point-list plan).  Errors: DD_EINVAL (sizes,
    non-finite origin or spacing, more than 2^31 points), DD_ENOMEM, DD_ECUDA. */
 dd_status dd_batch_create_grid(const dd_scan *const *scans, int32_t n_scans, const double *grid_xy,
                                const int64_t *grid_wh, const double *times_s, dd_precision prec,

@@ -355,7 +355,10 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
     b->prec = prec;
     b->n_scans = n_scans;
     b->on_grid = grid_xy != nullptr;
-    if (b->on_grid && prec == DD_MIXED) b->engine.reset(new dd::GridEngine());
+    // a plan with a side that the engine does not hold takes the point lists' kernels, on the points
+    // of its grids (64-bit numbers throughout), as FP64 grids do
+    if (b->on_grid && prec == DD_MIXED && *std::max_element(grid_wh, grid_wh + 2 * (size_t)n_scans) < dd::kGridMaxSide)
+        b->engine.reset(new dd::GridEngine());
     DD_CUDA_TRY(cudaGetDevice(&b->device));
     const int tile = prec == DD_MIXED ? kTile : ddk::CfgF64::kThreads * ddk::CfgF64::kPPT;
     std::vector<ddk::BScan> sc((size_t)n_scans);

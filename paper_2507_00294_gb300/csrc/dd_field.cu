@@ -608,7 +608,7 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
 
 // FP32-mixed grids of at least this many columns, rows and points take the contraction
 // (dd_grid.cu); smaller ones leave most of its tiles empty.
-constexpr int64_t kQuadMinSide = 32, kQuadMinPts = 4096, kQuadMaxSide = int64_t(1) << 30;
+constexpr int64_t kQuadMinSide = 32, kQuadMinPts = 4096;
 
 // Narrow grids (below 64 columns, half of the CUDA-core grid tile's 128, whose lanes mostly idle
 // there) take the final kernel of dd_grid.cu with every visit left to it.  A CTA there walks all of
@@ -618,7 +618,7 @@ constexpr int64_t kQuadMinSide = 32, kQuadMinPts = 4096, kQuadMaxSide = int64_t(
 // CTAs 189, 121, 128 CTAs 111, 105; 1024 visits, 48 x 48: 1536 CTAs 341, 302, 384 CTAs 146, 176.
 bool narrow_grid(const ddk::GridDesc &g, int64_t n_t, int64_t n_visits) {
     const int64_t ctas = ((g.W + 31) / 32) * ((g.H + 15) / 16) * n_t;
-    return g.W < 64 && g.H < kQuadMaxSide && n_visits <= 1024 && ctas >= (n_visits <= 256 ? 32 : n_visits);
+    return g.W < 64 && g.H < dd::kGridMaxSide && n_visits <= 1024 && ctas >= (n_visits <= 256 ? 32 : n_visits);
 }
 
 // Snapshots (indices k0 .. k1 - 1 in time order) of a whole raster on the dwell lattice that share
@@ -670,7 +670,7 @@ ShiftGroups shift_groups(const dd_scan *scan, const ddk::GridDesc &grid, const s
             rows_shifted += H;
             before = tdim[k];
         }
-        if (shifted <= 0.5 * direct && rows_shifted <= 2.0 * (double)(g.size() * grid.H) && h_ext < kQuadMaxSide) {
+        if (shifted <= 0.5 * direct && rows_shifted <= 2.0 * (double)(g.size() * grid.H) && h_ext < dd::kGridMaxSide) {
             out.rows = (int)per;
             out.H_ext = std::max(out.H_ext, h_ext);
             out.groups.push_back(std::move(g));
@@ -829,7 +829,7 @@ extern "C" dd_status dd_field_on_grid(const dd_scan *scan, double x0_m, double y
     ddk::GridDesc g;
     g.x0 = x0_m; g.y0 = y0_m; g.dx = dx_m; g.dy = dy_m; g.W = n_cols; g.H = n_rows;
     const int64_t n_pts = n_cols * n_rows;
-    if (prec == DD_MIXED && std::min(n_cols, n_rows) >= kQuadMinSide && n_pts >= kQuadMinPts && std::max(n_cols, n_rows) < kQuadMaxSide)
+    if (prec == DD_MIXED && std::min(n_cols, n_rows) >= kQuadMinSide && n_pts >= kQuadMinPts && std::max(n_cols, n_rows) < dd::kGridMaxSide)
         return run_grid_mixed(scan, g, times, true, out, stream);
     if (prec == DD_MIXED && narrow_grid(g, n_t, scan->n)) return run_grid_mixed(scan, g, times, false, out, stream);
     if (prec == DD_MIXED) return run_field<ddk::CfgMixed>(scan, nullptr, n_pts, g, times, out, stream);

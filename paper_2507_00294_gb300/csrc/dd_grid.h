@@ -26,6 +26,9 @@ struct GridBox {
     int64_t W = 0, H = 0;
 };
 
+// Sides below this: the engine's column, row and tile numbers are 32-bit.
+constexpr int64_t kGridMaxSide = int64_t(1) << 30;
+
 class GridEngine {
   public:
     GridEngine();
@@ -33,7 +36,7 @@ class GridEngine {
     GridEngine(const GridEngine &) = delete;
     GridEngine &operator=(const GridEngine &) = delete;
 
-    // Axes of a grid (W, H < 2^30) in the scan's pitch units; returns its index.
+    // Axes of a grid (W, H < kGridMaxSide) in the scan's pitch units; returns its index.
     int add_grid(const dd_scan *scan, const GridBox &g);
     // Coefficients of the visits [0, nact) of a scan at tdim (dwells), or of the lags M .. 1 of a
     // uniform scan; src: the scan's device block; contract: false leaves every visit to the

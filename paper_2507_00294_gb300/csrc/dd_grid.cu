@@ -265,7 +265,7 @@ cudaError_t GridEngine::finish(bool two_launches) {
             const int n_tiles = J.n_tc * ((J.H + ddk::kGqTile - 1) / ddk::kGqTile);
             // every tile of the job in the same number of pieces (whole partial rows)
             const int64_t cost = (k1 - k0) * row_cost(J, 0), steps = (k1 - k0 + 15) / 16;
-            const int64_t P = std::min(std::max<int64_t>(1, (cost + per / 2) / per), steps);
+            const int64_t P = std::min(std::max({int64_t(1), (cost + per / 2) / per, (steps + ddk::kGqRunSteps - 1) / ddk::kGqRunSteps}), steps);
             for (int64_t p = 0; p < P; ++p) {
                 const int64_t a = k0 + steps * p / P * 16, b = std::min(k1, k0 + steps * (p + 1) / P * 16);
                 for (int q = 0; q < n_tiles; ++q) {

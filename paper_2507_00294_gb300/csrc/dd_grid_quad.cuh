@@ -196,6 +196,9 @@ constexpr int kGqRegsProd = 64, kGqRegsMid = 48, kGqRegsDrain = 176;
 static_assert(kGqRegsProd * 32 * kGqProdWarps + kGqRegsMid * 128 + kGqRegsDrain * 32 * kGqDrainWarps <= 80 * kGqThreads, "register split");
 constexpr int kGqTile = 128;
 constexpr int kGqStageK = 64, kGqBufs = 3, kGqPieceK = 384;
+// K steps (16 rows of k) of a run at most: the draining warps add a run's stages of four steps in plain
+// FP32, whose rounding grows with the square root of their number (3e-7 of the sum for 512)
+constexpr int64_t kGqRunSteps = 4 * 512;
 constexpr int kGqPieceBytes = kGqTile * kGqStageK * 2;         // one FP16 piece of one side: 16 KB
 constexpr int kGqBufBytes = 4 * kGqPieceBytes;                 // Y_h, Y_l, X_h, X_l
 // A piece as the warps see it.  The rings hold 8: the coefficient warps are at most two pieces
@@ -704,9 +707,10 @@ __global__ void __launch_bounds__(64) grid_quad_prep_kernel(const GqPrep P) {
 }
 
 // The recent visits at a tile of 32 columns x 16 rows (lane = column, warp = 4 rows), each at the
-// cheapest series that holds it over the warp's points (the classes of the field kernel), plus the
-// contraction's partial rows, in that order in compensated FP32; out = pref times that.  Bound
-// by the series' issue for many recent visits, by the partial rows' loads for few.
+// cheapest series that holds it over the warp's points (the classes of the field kernel), summed over
+// stages of 32 visits and, with the contraction's partial rows, in compensated FP32 (a scan can have
+// thousands of recent visits); out = pref times that.  Bound by the series' issue for many recent
+// visits, by the partial rows' loads for few.
 constexpr int kGqFinRows = 16, kGqFinThreads = 128, kGqFinStage = 32;
 __global__ void __launch_bounds__(kGqFinThreads, 8)
 grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict__ tile_offs, int n_jobs,
@@ -741,7 +745,7 @@ grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict
         bx0 = fminf(bx0, __shfl_xor_sync(0xffffffffu, bx0, o));
         bx1 = fmaxf(bx1, __shfl_xor_sync(0xffffffffu, bx1, o));
     }
-    float2 run[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+    BlockSum<float> sum[4];
     for (int v0 = J.r0; v0 < J.r1; v0 += kGqFinStage) {
         const int cnt = min(kGqFinStage, J.r1 - v0);
         __syncthreads();
@@ -801,20 +805,20 @@ grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict
                 }
             }
         }
-#pragma unroll
-        for (int k = 0; k < 2; ++k) run[k] = __fadd2_rn(run[k], acc[k]);
+        sum[0].add(acc[0].x);
+        sum[1].add(acc[0].y);
+        sum[2].add(acc[1].x);
+        sum[3].add(acc[1].y);
     }
     if (c >= J.W || row0 >= J.H) return;
     const int nr = min(4, J.H - row0);
     if (J.out_off < 0) {                     // a segment: its recent visits as one more partial row
         float *const o = partial + J.t_off + J.nq * J.t_stride + (int64_t)row0 * J.W + c;
-        const float v[4] = {run[0].x, run[0].y, run[1].x, run[1].y};
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-            if (e < nr) o[(int64_t)e * J.W] = v[e];
+            if (e < nr) o[(int64_t)e * J.W] = sum[e].result();
         return;
     }
-    BlockSum<float> sum[4];
     const float *const p = partial + J.t_off + (int64_t)row0 * J.W + c;
 #pragma unroll 2
     for (int k = 0; k < J.nq; ++k) {
@@ -824,10 +828,6 @@ grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict
 #pragma unroll
         for (int e = 0; e < 4; ++e) sum[e].add(v[e]);
     }
-    sum[0].add(run[0].x);
-    sum[1].add(run[0].y);
-    sum[2].add(run[1].x);
-    sum[3].add(run[1].y);
     double *const o = out + J.out_off + (int64_t)row0 * J.W + c;
 #pragma unroll
     for (int e = 0; e < 4; ++e)

@@ -610,6 +610,13 @@ dd_status run_field(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts, 
 // (dd_grid.cu); smaller ones leave most of its tiles empty.
 constexpr int64_t kQuadMinSide = 32, kQuadMinPts = 4096;
 
+// ... unless the contraction would leave most of the pairs to the CUDA cores, more than this many
+// visits per snapshot (grids far wider than the diffusion of a visit): its kernel for those takes 1.2
+// to 1.5 times as long per pair as the grid tile, which shares a factor among snapshots.  4096 visits
+// in a line, D = 1e-16, 8 snapshots on 512 x 64 points: 339 us by it, 238 by the tile; 65,536 visits, D =
+// 6e-16, 128 x 64 points: 2172, 1932.
+constexpr double kQuadRecentVisits = 256.0;
+
 // Narrow grids (below 64 columns, half of the CUDA-core grid tile's 128, whose lanes mostly idle
 // there) take the final kernel of dd_grid.cu with every visit left to it.  A CTA there walks all of
 // a snapshot's visits for 32 columns x 16 rows (0.11 us per visit), where the grid tile splits them;
@@ -739,6 +746,16 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
             const int table = lattice ? lag : eng.add_table(scan, box, src, tdim[j], nact[j], contract);
             const int shift = lattice ? (int)(tdim[j] > 0 ? M - (int64_t)tdim[j] : M) : 0;
             eng.add_job(scan, srcF, gi, table, nact[j], shift, (int64_t)order[j] * n_pts);
+        }
+        if (contract && g0 == 0) {
+            double points = 0.0, all = 0.0;
+            const double recent = eng.recent_pairs(&points);
+            for (int j = 0; j < ng; ++j) all += (double)nact[j] * (double)n_pts;
+            if (recent > kQuadRecentVisits * points && recent > 0.5 * all) {
+                delete keep;
+                if (out_ws) DD_CUDA_TRY(dd::workspace_release(out_ws, stream));
+                return run_field<ddk::CfgMixed>(scan, nullptr, n_pts, grid, times, out, stream);
+            }
         }
         DD_CUDA_TRY(eng.finish(true));
         void *ws = nullptr;

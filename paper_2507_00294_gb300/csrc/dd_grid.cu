@@ -90,14 +90,14 @@ struct GridEngine::Tables {
     std::vector<ddk::GqJob> jobs;
     std::vector<ddk::GqRun> runs;                        // CTA by CTA, launch by launch
     std::vector<int> cta_off;                            // first run of each CTA, per launch n_cta + 1
-    std::vector<int64_t> ax_offs, vis_offs, rec_offs, tile_offs;
+    std::vector<int64_t> ax_offs, vis_offs, rec_offs;
+    std::vector<int64_t> part_tiles, out_tiles;          // tiles of the jobs that write partial rows, the field
     struct Span { int64_t k0, k1, split; };              // rows of k of a job; from split on: n > 2
     std::vector<Span> spans;
     std::vector<ddk::GqGroup> groups;                    // raster snapshots summed by segments of lags
     std::vector<ddk::GqSegment> segs;
     std::vector<int> seg_job;
     int64_t n_shift_blocks = 0;
-    bool any_direct = false;
     int n_cta[2] = {0, 0};
     int64_t n_ax = 0, n_vis = 0, n_rows = 0, n_rec = 0, n_part = 0;
     // device
@@ -107,7 +107,7 @@ struct GridEngine::Tables {
     float2 *ax = nullptr;
     float *part = nullptr;
 
-    struct Layout { size_t grids, tabs, jobs, runs, cta, axo, viso, reco, tileo, groups, segs, end; };
+    struct Layout { size_t grids, tabs, jobs, runs, cta, axo, viso, reco, parto, outo, groups, segs, end; };
     Layout layout() const {
         Layout l;
         size_t b = 0;
@@ -120,7 +120,8 @@ struct GridEngine::Tables {
         l.axo = add(ax_offs.size() * sizeof(int64_t));
         l.viso = add(vis_offs.size() * sizeof(int64_t));
         l.reco = add(rec_offs.size() * sizeof(int64_t));
-        l.tileo = add(tile_offs.size() * sizeof(int64_t));
+        l.parto = add(part_tiles.size() * sizeof(int64_t));
+        l.outo = add(out_tiles.size() * sizeof(int64_t));
         l.groups = add(groups.size() * sizeof(ddk::GqGroup));
         l.segs = add(segs.size() * sizeof(ddk::GqSegment));
         l.end = b;
@@ -176,7 +177,6 @@ int GridEngine::add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M, 
 
 void GridEngine::add_job(const dd_scan *scan, const float4 *srcF, int grid, int table, int nact, int shift,
                          int64_t out_off) {
-    t->any_direct = true;
     add_span(scan, srcF, grid, table, shift, shift + nact, shift, t->grids[grid].H, out_off);
 }
 
@@ -222,12 +222,47 @@ void GridEngine::add_shift_group(const dd_scan *scan, const float4 *srcF, int gr
     }
 }
 
+double GridEngine::recent_pairs(double *points) const {
+    double pairs = 0.0;
+    *points = 0.0;
+    for (const ddk::GqJob &j : t->jobs) {
+        pairs += (double)(j.r1 - j.r0) * j.W * j.H;
+        *points += (double)j.W * j.H;
+    }
+    return pairs;
+}
+
+// Tiles of a job's recent visits (a segment with none has none).
+static int64_t fin_tiles(const ddk::GqJob &j) {
+    return j.out_off < 0 && j.r1 <= j.r0 ? 0 : (int64_t)((j.W + 31) / 32) * ((j.H + ddk::kGqFinRows - 1) / ddk::kGqFinRows);
+}
+
+// Places of a job's partial rows; its recent visits in P parts, the earlier ones as jobs of their own
+// that write partial rows after the contraction's.
+void GridEngine::place_rows(size_t k, int P) {
+    ddk::GqJob &j = t->jobs[k];
+    const int r0 = j.r0, n = j.r1 - r0, nq = j.nq;
+    j.t_off = t->n_part;
+    j.row = j.nq = nq + P - 1;
+    t->n_part += (int64_t)(j.row + (j.out_off < 0 && n > 0 ? 1 : 0)) * j.t_stride;
+    if (P < 2) return;
+    auto at = [&](int e) { return r0 + (int)((int64_t)n * e / P); };
+    const int64_t rec0 = j.rec0;
+    j.r0 = at(P - 1);
+    j.rec0 += j.r0 - r0;
+    ddk::GqJob part = j;
+    part.out_off = -1;
+    for (int e = 0; e + 1 < P; ++e) {
+        part.row = nq + e;
+        part.r0 = at(e);
+        part.r1 = at(e + 1);
+        part.rec0 = rec0 + (part.r0 - r0);
+        t->jobs.push_back(part);
+    }
+}
+
 cudaError_t GridEngine::finish(bool two_launches) {
     const int sms = sm_count();
-    t->tile_offs.assign(1, 0);
-    for (const ddk::GqJob &j : t->jobs)              // a segment with no recent visits has no tiles
-        t->tile_offs.push_back(t->tile_offs.back() + (j.out_off < 0 && j.r1 <= j.r0 ? 0
-                               : (int64_t)((j.W + 31) / 32) * ((j.H + ddk::kGqFinRows - 1) / ddk::kGqFinRows)));
     // Cost of a run: its rows of k times the factors formed per row (32 positions at a time),
     // plus about 500 rows' worth of factors for its start, drain and output.
     auto row_cost = [](const ddk::GqJob &j, int tile) {
@@ -293,15 +328,35 @@ cudaError_t GridEngine::finish(bool two_launches) {
             t->runs[(size_t)(off[c] + round)] = list[(size_t)order[k].second];
         }
     }
-    for (ddk::GqJob &j : t->jobs) {
-        j.t_off = t->n_part;
-        t->n_part += (int64_t)(j.nq + (j.out_off < 0 && j.r1 > j.r0 ? 1 : 0)) * j.t_stride;
+    // more than kGqFinSplit recent visits are split while the tiles leave places for CTAs (two waves)
+    const size_t n_jobs = t->jobs.size();
+    int64_t tiles = 0;
+    int longest = 0;
+    for (const ddk::GqJob &j : t->jobs) {
+        tiles += fin_tiles(j);
+        longest = std::max(longest, j.r1 - j.r0);
+    }
+    const int64_t most = longest > ddk::kGqFinSplit ? 2 * ddk::kGqFinResident * (int64_t)sms / tiles : 1;
+    for (size_t k = 0; k < n_jobs; ++k) {
+        const int n = t->jobs[k].r1 - t->jobs[k].r0;
+        const int64_t parts = n > ddk::kGqFinSplit ? (n + ddk::kGqFinVisits - 1) / ddk::kGqFinVisits : 1;
+        place_rows(k, (int)std::max<int64_t>(1, std::min(most, parts)));
+    }
+    t->part_tiles.reserve(t->jobs.size() + 1);
+    t->out_tiles.reserve(t->jobs.size() + 1);
+    int64_t n_part = 0, n_out = 0;
+    for (size_t k = 0; k <= t->jobs.size(); ++k) {
+        t->part_tiles.push_back(n_part);
+        t->out_tiles.push_back(n_out);
+        if (k == t->jobs.size()) break;
+        const ddk::GqJob &j = t->jobs[k];
+        (j.out_off < 0 ? n_part : n_out) += fin_tiles(j);
     }
     for (size_t k = 0; k < t->segs.size(); ++k) {
         const ddk::GqJob &j = t->jobs[(size_t)t->seg_job[k]];
         t->segs[k].t_off = j.t_off;
         t->segs[k].t_stride = j.t_stride;
-        t->segs[k].n_part = j.nq + (j.r1 > j.r0 ? 1 : 0);
+        t->segs[k].n_part = j.row + (j.r1 > j.r0 ? 1 : 0);
     }
     return t->runs.empty() ? cudaSuccess : prepare_kernel();
 }
@@ -327,7 +382,8 @@ void GridEngine::write_tables(char *dst) const {
     put(l.axo, t->ax_offs);
     put(l.viso, t->vis_offs);
     put(l.reco, t->rec_offs);
-    put(l.tileo, t->tile_offs);
+    put(l.parto, t->part_tiles);
+    put(l.outo, t->out_tiles);
     put(l.groups, t->groups);
     put(l.segs, t->segs);
 }
@@ -342,7 +398,7 @@ void GridEngine::bind(void *workspace) {
     t->part = reinterpret_cast<float *>(take((size_t)t->n_part * sizeof(float)));
 }
 
-int64_t GridEngine::n_tiles() const { return t->tile_offs.empty() ? 0 : t->tile_offs.back(); }
+int64_t GridEngine::n_tiles() const { return t->out_tiles.empty() ? 0 : t->part_tiles.back() + t->out_tiles.back(); }
 int64_t GridEngine::n_runs() const { return (int64_t)t->runs.size(); }
 
 cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t side, cudaEvent_t fork,
@@ -379,30 +435,29 @@ cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t s
                 jobs, runs, off, t->rows, t->ax, t->part, withhold ? 1 : 0);
         });
     };
-    auto recent = [&](cudaStream_t s) -> cudaError_t {
-        if (n_tiles() == 0) return cudaSuccess;
+    auto recent = [&](const std::vector<int64_t> &tiles, size_t o, cudaStream_t s) -> cudaError_t {
+        if (tiles.back() == 0) return cudaSuccess;
         return scoped("field_grid_mixed", s, [&] {
-            ddk::grid_quad_final_kernel<<<(unsigned)n_tiles(), ddk::kGqFinThreads, 0, s>>>(
-                jobs, offs(l.tileo), (int)t->jobs.size(), t->rec, t->ax, t->part, out);
+            ddk::grid_quad_final_kernel<<<(unsigned)tiles.back(), ddk::kGqFinThreads, 0, s>>>(
+                jobs, offs(o), (int)t->jobs.size(), t->rec, t->ax, t->part, out);
         });
     };
-    // beside the first contraction launch: the second, and the recent visits where no snapshot
-    // is written by them (all on one stream: 86 us instead of 72 on 64 shared row snapshots)
-    const bool early = !t->any_direct;
-    const bool both = side != nullptr && t->n_cta[0] > 0 && (t->n_cta[1] > 0 || early);
+    // beside the first contraction launch: the second, and the recent visits that go to partial
+    // rows (all on one stream: 86 us instead of 72 on 64 shared row snapshots)
+    const bool both = side != nullptr && t->n_cta[0] > 0 && (t->n_cta[1] > 0 || t->part_tiles.back() > 0);
     cudaStream_t second = both ? side : stream;
     if (both) {
         if ((err = cudaEventRecord(fork, stream)) != cudaSuccess) return err;
         if ((err = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return err;
     }
     if ((err = contraction(0, "field_grid_tc", stream)) != cudaSuccess) return err;
-    if (early && (err = recent(second)) != cudaSuccess) return err;
+    if ((err = recent(t->part_tiles, l.parto, second)) != cudaSuccess) return err;
     if ((err = contraction(1, "field_grid_tc4", second)) != cudaSuccess) return err;
     if (both) {
         if ((err = cudaEventRecord(join, side)) != cudaSuccess) return err;
         if ((err = cudaStreamWaitEvent(stream, join, 0)) != cudaSuccess) return err;
     }
-    if (!early && (err = recent(stream)) != cudaSuccess) return err;
+    if ((err = recent(t->out_tiles, l.outo, stream)) != cudaSuccess) return err;
     if (t->groups.empty()) return cudaSuccess;
     return scoped("field_reduce", stream, [&] {
         ddk::grid_quad_shift_kernel<<<(unsigned)t->n_shift_blocks, 128, 0, stream>>>(

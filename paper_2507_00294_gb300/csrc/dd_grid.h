@@ -51,6 +51,8 @@ class GridEngine {
     // table: the lags M .. 1; rows_per_scan_row: grid rows per pitch.
     void add_shift_group(const dd_scan *scan, const float4 *srcF, int grid, int table, int64_t M, int64_t H,
                          int rows_per_scan_row, const std::vector<std::pair<int64_t, int64_t>> &snaps);
+    // (visit, point) pairs that the jobs so far leave to the CUDA cores, and their points.
+    double recent_pairs(double *points) const;
     // Splits the contraction into runs for the device's SMs: the rows of k of one and two nodes
     // and the rest as two launches (two_launches), or all in one.
     cudaError_t finish(bool two_launches);
@@ -69,6 +71,7 @@ class GridEngine {
   private:
     void add_span(const dd_scan *scan, const float4 *srcF, int grid, int table, int i0, int i1, int shift, int H,
                   int64_t out_off);
+    void place_rows(size_t job, int parts);
     struct Tables;
     Tables *t;
 };

@@ -156,10 +156,12 @@ struct GqJob {
     int tw, n_tc;                   // contraction tiles: tw columns (a multiple of 16) x 128 rows
     int shift;                      // visit of a table visit i: i - shift
     int r0, r1;                     // recent visits [r0, r1): the CUDA cores' part
-    int nq;                         // partial rows of the contraction
+    int nq;                         // partial rows to sum up (the contraction's, then others' recent visits)
+    int row;                        // out_off < 0: the partial row that takes this job's recent visits
     int64_t rec0;                   // record of visit r0
     int64_t t_off, t_stride;        // first partial row, row stride (floats)
-    int64_t out_off;                // < 0: a segment of lags (below), summed by its group
+    int64_t out_off;                // < 0: a segment of lags (below), summed by its group, or a part of
+                                    // another job's recent visits
     double pref;
 };
 
@@ -712,7 +714,12 @@ __global__ void __launch_bounds__(64) grid_quad_prep_kernel(const GqPrep P) {
 // thousands of recent visits); out = pref times that.  Bound by the series' issue for many recent
 // visits, by the partial rows' loads for few.
 constexpr int kGqFinRows = 16, kGqFinThreads = 128, kGqFinStage = 32;
-__global__ void __launch_bounds__(kGqFinThreads, 8)
+// More than kGqFinSplit recent visits of a job are split into parts of kGqFinVisits while the GPU has
+// places for their CTAs: a CTA walks 0.15 us per visit, so that 65,536 of them on 64 x 64 points (8
+// CTAs) took 9.8 ms in one piece each and take 0.36 ms split.  Fewer stay in one piece: a second
+// launch and its fork cost the host 20 us (256 visits, 16 x 16 points, 256 snapshots: 64 us, split 85).
+constexpr int kGqFinSplit = 256, kGqFinVisits = 64, kGqFinResident = 8;      // resident CTAs per SM
+__global__ void __launch_bounds__(kGqFinThreads, kGqFinResident)
 grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict__ tile_offs, int n_jobs,
                        const RecF32 *__restrict__ rec, const float2 *__restrict__ ax, float *partial,
                        double *__restrict__ out) {
@@ -812,8 +819,8 @@ grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict
     }
     if (c >= J.W || row0 >= J.H) return;
     const int nr = min(4, J.H - row0);
-    if (J.out_off < 0) {                     // a segment: its recent visits as one more partial row
-        float *const o = partial + J.t_off + J.nq * J.t_stride + (int64_t)row0 * J.W + c;
+    if (J.out_off < 0) {                     // the recent visits as a partial row
+        float *const o = partial + J.t_off + J.row * J.t_stride + (int64_t)row0 * J.W + c;
 #pragma unroll
         for (int e = 0; e < 4; ++e)
             if (e < nr) o[(int64_t)e * J.W] = sum[e].result();

@@ -526,15 +526,20 @@ dd_status run_dose(const dd_scan *scan, int64_t j0, int64_t j1, double *out, cud
 
 // Whether the targets [j0, j1) take the row-invariant path (dd_dose_rows.cuh): a raster or
 // serpentine scan of every grid position with a uniform dwell, when the path's pair terms
-// (2 nx per row up to the last target's on a raster, nx^2 on a serpentine) are no more than
-// the direct sum's (j per target).  64 x 64 and up: fewer by nx / 4 and more for a whole
-// scan; more than the direct sum's only for a few targets late in a scan.
-bool dose_rows_apply(const dd_scan *scan, int64_t j0, int64_t j1) {
+// (2 nx per row up to the last target's on a raster, nx^2 on a serpentine of several rows) are no
+// more than the direct sum's (j per target).  64 x 64 and up: fewer by nx / 4 and more for a
+// whole scan; more than the direct sum's only for a few targets late in a scan.  An FP32 term of
+// a serpentine takes twice a direct one's time once there are enough of them to fill the GPU, so
+// it needs half of them there (path against direct sum, us: 2 rows of 4096 74, 76, of 8192 240, 271, of
+// 16,384 906, 619; 5 of 16,384 2403, 2840).
+bool dose_rows_apply(const dd_scan *scan, dd_precision prec, int64_t j0, int64_t j1) {
     if (!scan->uniform || (scan->order != DD_RASTER && scan->order != DD_SERPENTINE)) return false;
     if (scan->n != (int64_t)scan->nx * scan->ny || j1 < 2) return false;
     const double nx = (double)scan->nx, rows = (double)((j1 - 1) / scan->nx + 1);
-    const double terms = scan->order == DD_RASTER ? 2.0 * nx * rows : nx * nx * (rows - 0.5);
-    return terms <= 0.5 * ((double)j1 * (double)j1 - (double)j0 * (double)j0);
+    const bool raster = scan->order == DD_RASTER || j1 <= scan->nx;
+    const double terms = raster ? 2.0 * nx * rows : nx * nx * (rows - 0.5);
+    const double cost = !raster && prec == DD_MIXED && terms > 2e8 ? 2.0 : 1.0;
+    return cost * terms <= 0.5 * ((double)j1 * (double)j1 - (double)j0 * (double)j0);
 }
 
 // Source visits per work item of the row-invariant path: whole rows when those already give
@@ -553,18 +558,21 @@ template <typename Cfg>
 dd_status run_dose_rows(const dd_scan *scan, int64_t j0, int64_t j1, double *out, cudaStream_t stream) {
     using Rec = typename Cfg::Rec;
     using Part = typename Cfg::Real;
-    const bool raster = scan->order == DD_RASTER;
+    const bool raster = scan->order == DD_RASTER || j1 <= scan->nx;      // (one row is both)
     const int64_t nx = scan->nx, n_rows = (j1 - 1) / nx + 1, m = j1 - j0;
     const int64_t n_mt = (nx + 31) / 32;
     const int64_t qc = raster ? nx : dose_rows_piece(nx, n_rows, sizeof(Part));
     const int64_t n_q = raster ? 2 : (nx + qc - 1) / qc;
     const int64_t n_lag = raster ? 0 : n_rows * nx;
+    const int64_t n_chunks = raster ? (nx + ddk::kDoseRasterHalf - 1) / ddk::kDoseRasterHalf : 1;
+    const int64_t n_base = n_chunks > 1 ? 2 * n_rows * n_chunks : 0;
     const dd::MemKind out_kind = dd::memory_kind(out);
     const bool out_host = out_kind != dd::MemKind::Device;
     const size_t b_rec = ((size_t)n_lag * sizeof(Rec) + 255) & ~size_t(255);
     const size_t b_part = ((size_t)(n_rows * n_q * nx) * sizeof(Part) + 255) & ~size_t(255);
+    const size_t b_base = ((size_t)n_base * sizeof(Part) + 255) & ~size_t(255);
     void *ws = nullptr;
-    cudaError_t err = dd::workspace_alloc(&ws, b_rec + b_part + (out_host ? (size_t)m * sizeof(double) : 0), stream);
+    cudaError_t err = dd::workspace_alloc(&ws, b_rec + b_part + b_base + (out_host ? (size_t)m * sizeof(double) : 0), stream);
     if (err != cudaSuccess) {
         cudaGetLastError();
         return dd::fail(err == cudaErrorMemoryAllocation ? DD_ENOMEM : DD_ECUDA,
@@ -572,11 +580,19 @@ dd_status run_dose_rows(const dd_scan *scan, int64_t j0, int64_t j1, double *out
     }
     Rec *d_rec = static_cast<Rec *>(ws);
     Part *d_part = reinterpret_cast<Part *>(static_cast<char *>(ws) + b_rec);
-    double *out_dev = out_host ? reinterpret_cast<double *>(static_cast<char *>(ws) + b_rec + b_part) : out;
+    Part *d_base = reinterpret_cast<Part *>(static_cast<char *>(ws) + b_rec + b_part);
+    double *out_dev = out_host ? reinterpret_cast<double *>(static_cast<char *>(ws) + b_rec + b_part + b_base) : out;
     if (raster) {
         const int half = (int)std::min<int64_t>(ddk::kDoseRasterHalf, n_mt * 32);
+        auto *const terms = n_chunks > 1 ? ddk::dose_raster_kernel<Cfg, true> : ddk::dose_raster_kernel<Cfg, false>;
         DD_PROFILED(Cfg::kDoseName, stream,
-                    (ddk::dose_raster_kernel<Cfg><<<(unsigned)n_rows, 2 * half, 0, stream>>>((int)nx, scan->s, scan->kappa, d_part)));
+                    (terms<<<(unsigned)(n_rows * n_chunks), 2 * half, 0, stream>>>(
+                        (int)nx, (int)n_chunks, scan->s, scan->kappa, d_part)));
+        DD_CUDA_TRY(cudaGetLastError());
+        if (n_base > 0)
+            DD_PROFILED("dose_base", stream,
+                        (ddk::dose_raster_base_kernel<Part><<<(unsigned)((n_base + 127) / 128), 128, 0, stream>>>(
+                            d_part, (int)nx, (int)n_chunks, n_base, d_base)));
     } else {
         DD_PROFILED(Cfg::kLagCoefName, stream,
                     (ddk::lag_coef_kernel<Rec><<<(unsigned)((n_lag + 31) / 32), 32, 0, stream>>>(n_lag, scan->s, scan->kappa, d_rec)));
@@ -586,10 +602,11 @@ dd_status run_dose_rows(const dd_scan *scan, int64_t j0, int64_t j1, double *out
                         nx, n_mt, n_q, qc, d_rec, d_part)));
     }
     DD_CUDA_TRY(cudaGetLastError());
+    auto *const scan_rows = n_base > 0 ? ddk::dose_rows_scan_kernel<Part, true> : ddk::dose_rows_scan_kernel<Part, false>;
     DD_PROFILED("dose_reduce", stream,
-                (ddk::dose_rows_scan_kernel<Part><<<(unsigned)((nx + ddk::kDoseScanCols - 1) / ddk::kDoseScanCols),
-                                                  ddk::kDoseScanCols * ddk::kDoseScanGroups, 0, stream>>>(
-                    d_part, nx, n_rows, n_q, j0, j1, scan->pref, out_dev)));
+                (scan_rows<<<(unsigned)((nx + ddk::kDoseScanCols - 1) / ddk::kDoseScanCols),
+                             ddk::kDoseScanCols * ddk::kDoseScanGroups, 0, stream>>>(
+                    d_part, d_base, (int)n_chunks, nx, n_rows, n_q, j0, j1, scan->pref, out_dev)));
     DD_CUDA_TRY(cudaGetLastError());
     if (out_host)
         DD_CUDA_TRY(cudaMemcpyAsync(out, out_dev, (size_t)m * sizeof(double), cudaMemcpyDeviceToHost, stream));
@@ -644,7 +661,7 @@ dd_status dose_range(const dd_scan *scan, dd_precision prec, int64_t j0, int64_t
         if (prec == DD_MIXED) return run_dose_general<ddk::CfgMixed>(scan, j0, j1, out, stream);
         return run_dose_general<ddk::CfgF64>(scan, j0, j1, out, stream);
     }
-    if (dose_rows_apply(scan, j0, j1)) {
+    if (dose_rows_apply(scan, prec, j0, j1)) {
         if (prec == DD_MIXED) return run_dose_rows<ddk::CfgMixed>(scan, j0, j1, out, stream);
         return run_dose_rows<ddk::CfgF64>(scan, j0, j1, out, stream);
     }

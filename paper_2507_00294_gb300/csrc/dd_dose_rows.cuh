@@ -15,11 +15,11 @@
 // On a raster the term depends on d = m - q alone at a given s, so that R(s, m) is the sum of the
 // window d = m - nx + 1 .. m of 2 nx - 1 terms: 2 n pair terms in all.  The window splits at
 // d = 0 into a running sum of the terms d = 0 .. m and one, taken from the far end, of the
-// negative d: only sums of positive terms.  dose_raster_kernel: one CTA per s, one half of its
-// threads for each of the two sums, one lag record and one term per thread, then a block scan
-// (compensated in FP32).  It is bound by the latency of a record's serial chain and one term.
-// 256 x 256 FP32: 15 us, with the running sum over rows 27 us a call, against 2.72 ms for the
-// direct sum's 2.1e9 terms; 20 x 20 FP64: 93 us against 759 us.
+// negative d: only sums of positive terms.  dose_raster_kernel: one CTA per s and 256 terms of each
+// of the two sums, one half of its threads for each, one lag record and one term per thread, then
+// a block scan (compensated in FP32).  It is bound by the latency of a record's serial chain and
+// one term.  Device time of a call: 256 x 256 FP32 22 us, against 2.72 ms for the direct sum's
+// 2.1e9 terms; 64 x 64 FP64 25 us, against 787 us.  A scan of one row is a raster in either order.
 //
 // On a serpentine the odd s have no such window; dose_rows_kernel forms R from all nx^2 terms of
 // each s, in pieces of qc visits of the source row: one CTA per (s, piece, 32 targets m), lane =
@@ -129,23 +129,27 @@ __device__ __forceinline__ float lone_pair_term(float r2, const RecF32 &R) {
 }
 __device__ __forceinline__ double lone_pair_term(double r2, const RecF64 &R) { return pair_term(r2, R); }
 
-// partial[2 s nx + m] = sum of the terms d = 0 .. m of row offset s, partial[(2 s + 1) nx + m] =
-// sum of its terms d = m - nx + 1 .. -1 (none at s = 0); blockDim.x / 2 threads for each.
+// Terms d = 0 .. of row offset s (side 0) and -1, -2 .. (side 1; none at s = 0) in chunks of half =
+// blockDim.x / 2 threads, one CTA for both sides of a chunk: partial[2 s nx + m] = sum of the chunk's
+// terms up to d = m, partial[(2 s + 1) nx + m] = sum of its terms down to d = m - nx + 1.  A row of one
+// chunk (nx <= 256) is then complete; dose_raster_base_kernel sums the chunks before each one.  (One
+// CTA walking a row's chunks with a carry took 3 us for each: 58 us for 4096 x 1 FP32, the direct sum
+// 44, this 21; 8192 x 1: 105, 66, 23; 65,536 x 1: 774, 1465, 57.)
 constexpr int kDoseRasterHalf = 256;         // largest half of a CTA
-template <typename Cfg>
+template <typename Cfg, bool kChunks>
 __global__ void __launch_bounds__(2 * kDoseRasterHalf)
-dose_raster_kernel(int nx, double s_dim, double kappa, typename Cfg::Real *__restrict__ partial) {
+dose_raster_kernel(int nx, int n_chunks, double s_dim, double kappa, typename Cfg::Real *__restrict__ partial) {
     using Rec = typename Cfg::Rec;
     using Real = typename Cfg::Real;
     __shared__ BlockSum<Real> s_warp[2 * kDoseRasterHalf / 32];
     const int half = blockDim.x / 2, side = threadIdx.x >= half, t = threadIdx.x - side * half;
-    const int lane = threadIdx.x & 31, warp0 = side * half / 32, nw = half / 32, warp = t / 32;
-    const int64_t s = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp0 = side * half / 32, warp = t / 32;
+    const int64_t s = kChunks ? blockIdx.x / n_chunks : blockIdx.x;
     Real *const row = partial + (2 * s + side) * (int64_t)nx;
-    BlockSum<Real> carry;                    // the chunks before this one
-    for (int i0 = 0; i0 < nx; i0 += half) {
-        const int i = i0 + t;
-        const int d = side ? -1 - i : i;
+    // one pass (as a loop it compiles to a shorter FP64 chain: 18.9 us against 20.3 for 20 x 20)
+    const int first = kChunks ? (int)(blockIdx.x % n_chunks) * half : 0, end = kChunks ? first + 1 : nx;
+    for (int i0 = first; i0 < end; i0 += half) {
+        const int i = i0 + t, d = side ? -1 - i : i;
         const int64_t k = s * nx + d;        // lag
         BlockSum<Real> v;
         if (i < nx - side && k > 0) {
@@ -163,34 +167,63 @@ dose_raster_kernel(int nx, double s_dim, double kappa, typename Cfg::Real *__res
         }
         if (lane == 31) s_warp[warp0 + warp] = v;
         __syncthreads();
-        BlockSum<Real> base = carry;
-        for (int w = 0; w < nw; ++w) {
-            if (w < warp) base.add(s_warp[warp0 + w]);
-            carry.add(s_warp[warp0 + w]);
-        }
+        BlockSum<Real> base;
+        for (int w = 0; w < warp; ++w) base.add(s_warp[warp0 + w]);
         v.add(base);
         if (i < nx) row[!side ? i : i < nx - 1 ? nx - 2 - i : nx - 1] = side && i == nx - 1 ? (Real)0 : v.result();
         __syncthreads();
     }
 }
 
-// out[iy nx + m - j0] = pref * sum over rows s <= iy and pieces of partial, for the targets
-// j0 <= iy nx + m < j1.
-constexpr int kDoseScanCols = 8, kDoseScanGroups = 32;
+// Chunk of column m on a side, and the column that holds the chunk's whole sum (side 1 runs from m =
+// nx - 2 down; its m = nx - 1, no terms, belongs to chunk 0).
+__device__ __forceinline__ int dose_chunk(int m, int nx, int side) {
+    return (side ? max(nx - 2 - m, 0) : m) / kDoseRasterHalf;
+}
+__device__ __forceinline__ int dose_chunk_end(int c, int nx, int side) {
+    const int i = (c + 1) * kDoseRasterHalf - 1;
+    return side ? nx - 2 - i : i;
+}
+// base[(2 s + side) n_chunks + c] = sum of the chunks before c.
 template <typename Part>
+__global__ void __launch_bounds__(128)
+dose_raster_base_kernel(const Part *__restrict__ partial, int nx, int n_chunks, int64_t n, Part *__restrict__ base) {
+    const int64_t g = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (g >= n) return;
+    const int64_t k = g / n_chunks;
+    const int c = (int)(g % n_chunks), side = (int)(k & 1);
+    BlockSum<Part> sum;
+#pragma unroll 8
+    for (int e = 0; e < c; ++e) sum.add(partial[k * nx + dose_chunk_end(e, nx, side)]);
+    base[g] = sum.result();
+}
+
+// out[iy nx + m - j0] = pref * sum over rows s <= iy and pieces of partial (and, on a raster of several
+// chunks, of the chunks before m's: base), for the targets j0 <= iy nx + m < j1.
+constexpr int kDoseScanCols = 8, kDoseScanGroups = 32;
+template <typename Part, bool kBase>
 __global__ void __launch_bounds__(kDoseScanCols * kDoseScanGroups)
-dose_rows_scan_kernel(const Part *__restrict__ partial, int64_t nx, int64_t n_rows, int64_t n_q, int64_t j0,
-                      int64_t j1, double pref, double *__restrict__ out) {
+dose_rows_scan_kernel(const Part *__restrict__ partial, const Part *__restrict__ base, int n_chunks, int64_t nx,
+                      int64_t n_rows, int64_t n_q, int64_t j0, int64_t j1, double pref, double *__restrict__ out) {
     __shared__ BlockSum<Part> s_sum[kDoseScanGroups][kDoseScanCols];
     const int col = threadIdx.x % kDoseScanCols, g = threadIdx.x / kDoseScanCols;
     const int64_t m = (int64_t)blockIdx.x * kDoseScanCols + col;
     const bool live = m < nx;
     const int64_t ra = n_rows * g / kDoseScanGroups, rb = n_rows * (g + 1) / kDoseScanGroups;
+    const int c0 = kBase && live ? dose_chunk((int)m, (int)nx, 0) : 0, c1 = kBase && live ? dose_chunk((int)m, (int)nx, 1) : 0;
     BlockSum<Part> sum;
     if (live) {
         const Part *p = partial + ra * n_q * nx + m;
 #pragma unroll 8
         for (int64_t k = 0; k < (rb - ra) * n_q; ++k) sum.add(p[k * nx]);
+        if (kBase) {
+            const Part *b = base + ra * 2 * n_chunks;
+#pragma unroll 4
+            for (int64_t r = 0; r < rb - ra; ++r) {
+                sum.add(b[2 * r * n_chunks + c0]);
+                sum.add(b[(2 * r + 1) * n_chunks + c1]);
+            }
+        }
     }
     s_sum[g][col] = sum;
     __syncthreads();
@@ -201,6 +234,10 @@ dose_rows_scan_kernel(const Part *__restrict__ partial, int64_t nx, int64_t n_ro
         const Part *p = partial + r * n_q * nx + m;
 #pragma unroll 4
         for (int64_t k = 0; k < n_q; ++k) run.add(p[k * nx]);
+        if (kBase) {
+            run.add(base[2 * r * n_chunks + c0]);
+            run.add(base[(2 * r + 1) * n_chunks + c1]);
+        }
         const int64_t j = r * nx + m;
         if (j >= j0 && j < j1) out[j - j0] = pref * run.value();
     }

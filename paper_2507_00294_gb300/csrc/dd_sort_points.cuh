@@ -15,6 +15,12 @@
 // caller's order, 260 us in this one
 // (sort 16 us, field kernel 258 to 209 us); a batch of 256 scans on 997 random points each 774
 // and 667 us.
+//
+// A block of points that the caller already gave in compact runs stays as it is: where the boxes of
+// the 128 points that each warp of a tile would hold (four runs of 32) have a mean squared diagonal
+// of at most the block's own area.  (Sorted runs have an eighth of it.  A row-major list of 128 x 128
+// points, half of it: sorted, the tile took as long and the call 3 % longer, 540 us against 525;
+// lists in random order, or sorted by one coordinate only, have 2 to 5 times it and gain by the sort.)
 #pragma once
 #include <cstdint>
 
@@ -29,6 +35,7 @@ static_assert(kSortPer == 2 && kSortPts % kSortTile == 0, "two keys per thread, 
 struct SortSmem {
     uint32_t key[kSortPts];
     float lo[kSortThreads / 32][2], hi[kSortThreads / 32][2];
+    float4 box[kSortPts / 32];               // of the runs of 32 points: x from, to, y from, to
 };
 
 __device__ __forceinline__ uint32_t spread8(uint32_t v) {
@@ -50,20 +57,22 @@ __device__ __forceinline__ void sort_points_block(SortSmem &sm, int64_t n, int64
     for (int e = 0; e < kSortPer; ++e) {
         const int i = kSortWarp * warp + 32 * e + lane;
         x[e] = y[e] = 0.0f;
+        float ax = 3e38f, bx = -3e38f, ay = 3e38f, by = -3e38f;
         if (i < cnt) {
             const float4 p = in[c0 + i];
-            x[e] = p.x;
-            y[e] = p.z;
-            xl = fminf(xl, p.x); xh = fmaxf(xh, p.x);
-            yl = fminf(yl, p.z); yh = fmaxf(yh, p.z);
+            ax = bx = x[e] = p.x;
+            ay = by = y[e] = p.z;
         }
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        xl = fminf(xl, __shfl_xor_sync(0xffffffffu, xl, o));
-        xh = fmaxf(xh, __shfl_xor_sync(0xffffffffu, xh, o));
-        yl = fminf(yl, __shfl_xor_sync(0xffffffffu, yl, o));
-        yh = fmaxf(yh, __shfl_xor_sync(0xffffffffu, yh, o));
+        for (int o = 16; o > 0; o >>= 1) {
+            ax = fminf(ax, __shfl_xor_sync(0xffffffffu, ax, o));
+            bx = fmaxf(bx, __shfl_xor_sync(0xffffffffu, bx, o));
+            ay = fminf(ay, __shfl_xor_sync(0xffffffffu, ay, o));
+            by = fmaxf(by, __shfl_xor_sync(0xffffffffu, by, o));
+        }
+        if (lane == 0) sm.box[kSortPer * warp + e] = make_float4(ax, bx, ay, by);
+        xl = fminf(xl, ax); xh = fmaxf(xh, bx);
+        yl = fminf(yl, ay); yh = fmaxf(yh, by);
     }
     if (lane == 0) {
         sm.lo[warp][0] = xl; sm.lo[warp][1] = yl;
@@ -78,6 +87,30 @@ __device__ __forceinline__ void sort_points_block(SortSmem &sm, int64_t n, int64
         xh = fmaxf(xh, __shfl_xor_sync(0xffffffffu, xh, o));
         yl = fminf(yl, __shfl_xor_sync(0xffffffffu, yl, o));
         yh = fmaxf(yh, __shfl_xor_sync(0xffffffffu, yh, o));
+    }
+    // the caller's order: warp w of tile T would hold the runs 16 T + w + 4 j (lane = 4 T + w)
+    float d2 = 0.0f;
+    const int n_warps = 4 * ((cnt + kSortTile - 1) / kSortTile);
+    if (lane < n_warps) {
+        float4 u = make_float4(3e38f, -3e38f, 3e38f, -3e38f);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float4 q = sm.box[16 * (lane >> 2) + (lane & 3) + 4 * j];
+            u = make_float4(fminf(u.x, q.x), fmaxf(u.y, q.y), fminf(u.z, q.z), fmaxf(u.w, q.w));
+        }
+        if (u.y >= u.x) d2 = (u.y - u.x) * (u.y - u.x) + (u.w - u.z) * (u.w - u.z);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+    if (d2 <= (float)n_warps * ((xh - xl) * (yh - yl))) {        // (not where a coordinate is not finite)
+#pragma unroll
+        for (int e = 0; e < kSortPer; ++e) {
+            const int64_t i = c0 + kSortWarp * warp + 32 * e + lane;
+            if (i >= c0 + cnt) continue;
+            F[i] = in[i];
+            perm[i] = (int)i;
+        }
+        return;
     }
     const float side = fmaxf(xh - xl, yh - yl), inv = side > 0.0f ? 255.999f / side : 0.0f;
     uint32_t v[kSortPer];

@@ -700,16 +700,29 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
     int64_t M = 0;
     const bool lattice = snapshot_dims(scan, times, order, tdim, nact, M);
     const dd::GridBox box{grid.x0, grid.y0, grid.dx, grid.dy, grid.W, grid.H};
+    double all = 0.0;
+    for (int n : nact) all += (double)n;
+    if (contract && all > kQuadRecentVisits * n_t) {
+        const double age = dd::GridEngine::banded_age(scan, box);
+        double recent = 0.0;
+        for (int k = 0; k < n_t; ++k)
+            recent += lattice ? std::min((double)nact[k], std::ceil(age))
+                              : (double)(nact[k] - std::min<int64_t>(nact[k], std::upper_bound(scan->T.begin(), scan->T.end(), tdim[k] - age) - scan->T.begin()));
+        if (recent > kQuadRecentVisits * n_t && recent > 0.5 * all && shift_groups(scan, grid, tdim, lattice, 0, n_t).groups.empty())
+            return run_field<ddk::CfgMixed>(scan, nullptr, n_pts, grid, times, out, stream);
+    }
+    // snapshots of a pass: their tables (off the lattice; on it one serves them all) and about four
+    // partial rows each, so that the workspace stays in the allocator's 1 GiB class
+    constexpr int64_t kPassBytes = 960 * (int64_t(1) << 20);
+    const bool few = lattice || all * (double)dd::GridEngine::kMostVisitBytes < 0.5 * (double)kPassBytes;
+    auto pass_bytes = [&](int k) {
+        return 16 * n_pts + (few ? 0 : dd::GridEngine::table_device_bytes(scan, box, tdim[k], nact[k], contract));
+    };
     dd_status st = DD_OK;
     const double *src = dd::device_sources(scan, stream, &st);
     if (!src) return st;
     const dd::ScanUse use{scan, stream};
     const float4 *srcF = dd::device_sources_ff(scan, stream, &st);
-    // snapshots per pass: rows of k (off the lattice, a table per snapshot) and partial rows
-    // within about 1 GiB
-    int group = std::min(n_t, 4096);
-    while (group > 1 && (double)group * ((lattice ? 0.0 : (contract ? 48.0 : 80.0) * (double)scan->n) + 16.0 * (double)n_pts) > (double)(int64_t(1) << 30))
-        group = (group + 1) / 2;
     double *out_dev = out;
     void *out_ws = nullptr;
     auto no_memory = [](cudaError_t err) {
@@ -723,8 +736,12 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
         out_dev = static_cast<double *>(out_ws);
     }
     auto *keep = new HostTables();
-    for (int g0 = 0; g0 < n_t; g0 += group) {
-        const int ng = std::min(group, n_t - g0);
+    for (int g0 = 0, ng = 0; g0 < n_t; g0 += ng) {
+        int64_t bytes = few && !lattice ? kPassBytes / 2 : 0;
+        for (ng = 0; g0 + ng < n_t && ng < 4096; ++ng) {
+            bytes += pass_bytes(g0 + ng);
+            if (ng > 0 && bytes > kPassBytes) break;
+        }
         dd::GridEngine eng;
         const ShiftGroups sg = shift_groups(scan, grid, tdim, lattice && contract, g0, g0 + ng);
         // (a row of a group's tall grid counts only where some snapshot sees it, at a distance
@@ -746,16 +763,6 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
             const int table = lattice ? lag : eng.add_table(scan, box, src, tdim[j], nact[j], contract);
             const int shift = lattice ? (int)(tdim[j] > 0 ? M - (int64_t)tdim[j] : M) : 0;
             eng.add_job(scan, srcF, gi, table, nact[j], shift, (int64_t)order[j] * n_pts);
-        }
-        if (contract && g0 == 0) {
-            double points = 0.0, all = 0.0;
-            const double recent = eng.recent_pairs(&points);
-            for (int j = 0; j < ng; ++j) all += (double)nact[j] * (double)n_pts;
-            if (recent > kQuadRecentVisits * points && recent > 0.5 * all) {
-                delete keep;
-                if (out_ws) DD_CUDA_TRY(dd::workspace_release(out_ws, stream));
-                return run_field<ddk::CfgMixed>(scan, nullptr, n_pts, grid, times, out, stream);
-            }
         }
         DD_CUDA_TRY(eng.finish(true));
         void *ws = nullptr;

@@ -47,11 +47,20 @@ void band_ages(const dd_scan *scan, const dd::GridBox &g, bool contract, double 
     }
 }
 
+// The snapshot's first visit past each band.
+void band_starts(const dd_scan *scan, const double (&age)[kGqBands], double tdim, int nact, int (&vb)[kGqBands + 1]) {
+    vb[0] = 0;
+    for (int b = 0; b < kGqBands; ++b) {
+        const int64_t k = std::isinf(age[b]) ? 0 : std::upper_bound(scan->T.begin(), scan->T.end(), tdim - age[b]) - scan->T.begin();
+        vb[b + 1] = std::max(vb[b], (int)std::min<int64_t>(k, nact));
+    }
+}
+
 // Rows of k of the table visits before i.
-int64_t rows_before(const ddk::GqTable &t, int64_t i) {
+int64_t rows_before(const int (&vb)[kGqBands + 1], int64_t i) {
     int64_t k = 0;
-    for (int b = 0; b < kGqBands && t.vb[kGqBands] > 0; ++b)
-        k += std::max<int64_t>(0, std::min<int64_t>(i, t.vb[b + 1]) - t.vb[b]) * kGqNodes[b];
+    for (int b = 0; b < kGqBands && vb[kGqBands] > 0; ++b)
+        k += std::max<int64_t>(0, std::min<int64_t>(i, vb[b + 1]) - vb[b]) * kGqNodes[b];
     return k;
 }
 
@@ -143,16 +152,12 @@ int GridEngine::add_table(const dd_scan *scan, const GridBox &g, const double *s
     double age[kGqBands];
     band_ages(scan, g, contract, age);
     ddk::GqTable tb{src + 2 * scan->n, src + 3 * scan->n, scan->s, scan->kappa, tdim, t->n_vis, t->n_rows, t->n_rec, nact, 0, {}};
-    tb.vb[0] = 0;
-    for (int b = 0; b < kGqBands; ++b) {
-        const int64_t k = std::isinf(age[b]) ? 0 : std::upper_bound(scan->T.begin(), scan->T.end(), tdim - age[b]) - scan->T.begin();
-        tb.vb[b + 1] = std::max(tb.vb[b], (int)std::min<int64_t>(k, nact));
-    }
+    band_starts(scan, age, tdim, nact, tb.vb);
     t->tabs.push_back(tb);
     t->vis_offs.push_back(t->n_vis);
     t->rec_offs.push_back(t->n_rec);
     t->n_vis += nact;
-    t->n_rows += rows_before(tb, nact);
+    t->n_rows += rows_before(tb.vb, nact);
     t->n_rec += nact - tb.vb[kGqBands];
     return (int)t->tabs.size() - 1;
 }
@@ -170,7 +175,7 @@ int GridEngine::add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M, 
     t->vis_offs.push_back(t->n_vis);
     t->rec_offs.push_back(t->n_rec);
     t->n_vis += M;
-    t->n_rows += rows_before(tb, M);
+    t->n_rows += rows_before(tb.vb, M);
     t->n_rec += M - tb.vb[kGqBands];
     return (int)t->tabs.size() - 1;
 }
@@ -202,7 +207,7 @@ void GridEngine::add_span(const dd_scan *scan, const float4 *srcF, int grid, int
     j.pref = scan->pref;
     t->jobs.push_back(j);
     const int mid = std::min(std::max(tb.vb[2], i0), kc);
-    t->spans.push_back({tb.k_off + rows_before(tb, i0), tb.k_off + rows_before(tb, kc), tb.k_off + rows_before(tb, mid)});
+    t->spans.push_back({tb.k_off + rows_before(tb.vb, i0), tb.k_off + rows_before(tb.vb, kc), tb.k_off + rows_before(tb.vb, mid)});
 }
 
 void GridEngine::add_shift_group(const dd_scan *scan, const float4 *srcF, int grid, int table, int64_t M, int64_t H,
@@ -222,14 +227,18 @@ void GridEngine::add_shift_group(const dd_scan *scan, const float4 *srcF, int gr
     }
 }
 
-double GridEngine::recent_pairs(double *points) const {
-    double pairs = 0.0;
-    *points = 0.0;
-    for (const ddk::GqJob &j : t->jobs) {
-        pairs += (double)(j.r1 - j.r0) * j.W * j.H;
-        *points += (double)j.W * j.H;
-    }
-    return pairs;
+double GridEngine::banded_age(const dd_scan *scan, const GridBox &g) {
+    double age[kGqBands];
+    band_ages(scan, g, true, age);
+    return age[kGqBands - 1];
+}
+
+int64_t GridEngine::table_device_bytes(const dd_scan *scan, const GridBox &g, double tdim, int nact, bool contract) {
+    double age[kGqBands];
+    int vb[kGqBands + 1];
+    band_ages(scan, g, contract, age);
+    band_starts(scan, age, tdim, nact, vb);
+    return rows_before(vb, nact) * (int64_t)sizeof(ddk::GqRow) + (nact - vb[kGqBands]) * (int64_t)sizeof(ddk::RecF32);
 }
 
 // Tiles of a job's recent visits (a segment with none has none).

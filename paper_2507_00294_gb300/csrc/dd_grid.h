@@ -51,8 +51,11 @@ class GridEngine {
     // table: the lags M .. 1; rows_per_scan_row: grid rows per pitch.
     void add_shift_group(const dd_scan *scan, const float4 *srcF, int grid, int table, int64_t M, int64_t H,
                          int rows_per_scan_row, const std::vector<std::pair<int64_t, int64_t>> &snaps);
-    // (visit, point) pairs that the jobs so far leave to the CUDA cores, and their points.
-    double recent_pairs(double *points) const;
+    // Age (in dwells) from which every visit of a scan is in the contraction's bands on a grid.
+    static double banded_age(const dd_scan *scan, const GridBox &g);
+    // Device bytes that add_table takes, and the most a visit can.
+    static int64_t table_device_bytes(const dd_scan *scan, const GridBox &g, double tdim, int nact, bool contract);
+    static constexpr int64_t kMostVisitBytes = 512;      // 32 nodes
     // Splits the contraction into runs for the device's SMs: the rows of k of one and two nodes
     // and the rest as two launches (two_launches), or all in one.
     cudaError_t finish(bool two_launches);

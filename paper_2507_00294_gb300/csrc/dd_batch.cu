@@ -251,7 +251,7 @@ void launch_field(dd_batch *b, int grid, cudaStream_t st) {
 // Enqueue the whole batch evaluation on `st` (used for capture and for tuning).
 dd_status enqueue(dd_batch *b, const double *pts, double *out, int variant, cudaStream_t st) {
     if (b->engine) {
-        DD_CUDA_TRY(b->engine->enqueue(out, st, nullptr, nullptr, nullptr, false, false));
+        DD_CUDA_TRY(b->engine->enqueue(out, st, b->side, b->ev_fork, b->ev_join, false, false));
         return DD_OK;
     }
     const unsigned nb_pts = (unsigned)((b->total_pts + 255) / 256);
@@ -437,7 +437,7 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
     }
     if (b->engine) {
         b->variant = 0;                                  // one kernel for grids
-        DD_CUDA_TRY(b->engine->finish(false));
+        DD_CUDA_TRY(b->engine->finish());
         b->n_items = (int)std::min<int64_t>(b->engine->n_runs() + b->engine->n_tiles(), INT_MAX);
         cudaError_t err = cudaMalloc(&b->ws, b->engine->workspace_bytes());
         if (err != cudaSuccess) {
@@ -449,6 +449,9 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
         b->engine->write_tables(tables.data());
         DD_CUDA_TRY(cudaMemcpy(b->ws, tables.data(), tables.size(), cudaMemcpyHostToDevice));
         DD_CUDA_TRY(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
+        DD_CUDA_TRY(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
+        DD_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
+        DD_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming));
         *out = b.release();
         return DD_OK;
     }

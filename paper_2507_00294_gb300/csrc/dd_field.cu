@@ -764,7 +764,7 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
             const int shift = lattice ? (int)(tdim[j] > 0 ? M - (int64_t)tdim[j] : M) : 0;
             eng.add_job(scan, srcF, gi, table, nact[j], shift, (int64_t)order[j] * n_pts);
         }
-        DD_CUDA_TRY(eng.finish(true));
+        DD_CUDA_TRY(eng.finish());
         void *ws = nullptr;
         const cudaError_t err = dd::fault_injected("alloc") ? cudaErrorMemoryAllocation
                                                             : dd::workspace_alloc(&ws, eng.workspace_bytes(), stream);

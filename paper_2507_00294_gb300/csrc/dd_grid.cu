@@ -19,6 +19,15 @@ namespace {
 using ddk::kGqBands;
 using ddk::kGqNodes;
 
+// Largest distances along x and y between the grid's box and the visits' box (pitch units).
+void box_reach(const dd_scan *scan, const dd::GridBox &g, double &ex, double &ey) {
+    const double ip = 1.0 / scan->pitch;
+    const double xa = g.x0 * ip, xb = (g.x0 + (double)(g.W - 1) * g.dx) * ip;
+    const double ya = g.y0 * ip, yb = (g.y0 + (double)(g.H - 1) * g.dy) * ip;
+    ex = std::max(std::max(xa, xb) - scan->x_lo, scan->x_hi - std::min(xa, xb));
+    ey = std::max(std::max(ya, yb) - scan->y_lo, scan->y_hi - std::min(ya, yb));
+}
+
 // Ages (in dwells) from which every visit of the scan takes each band at every point of the
 // grid (+inf: none): h = rho^2 dq <= kGqH for rho^2 up to R2, the largest squared distance
 // between the grid's box and the visits' box, r = w1/w0 - 1 <= kGqR, and the dwell over.  With
@@ -29,11 +38,8 @@ void band_ages(const dd_scan *scan, const dd::GridBox &g, bool contract, double 
         for (double &a : age) a = INFINITY;
         return;
     }
-    const double ip = 1.0 / scan->pitch;
-    const double xa = g.x0 * ip, xb = (g.x0 + (double)(g.W - 1) * g.dx) * ip;
-    const double ya = g.y0 * ip, yb = (g.y0 + (double)(g.H - 1) * g.dy) * ip;
-    const double ex = std::max(std::max(xa, xb) - scan->x_lo, scan->x_hi - std::min(xa, xb));
-    const double ey = std::max(std::max(ya, yb) - scan->y_lo, scan->y_hi - std::min(ya, yb));
+    double ex, ey;
+    box_reach(scan, g, ex, ey);
     // margins for the points' own rounding
     const double R2 = (ex * ex + ey * ey) * (1.0 + 1e-6) + 1e-6;
     const double c = 4.0 * scan->kappa * scan->tau_max;
@@ -45,6 +51,21 @@ void band_ages(const dd_scan *scan, const dd::GridBox &g, bool contract, double 
         const double a = (w1 - 2.0 * scan->s) / (4.0 * scan->kappa) * (1.0 + 1e-9);
         prev = age[b] = std::isfinite(a) && a > 0.0 ? std::min(prev, a) : INFINITY;
     }
+}
+
+// Age (in dwells) from which a visit's factors stay within 2^-18 of 1 on the grid, so that FP16 pieces
+// (dd_grid_quad.cuh: full precision down to 2^-24 of a piece's largest) hold them at every point with
+// 2^6 left for the spread of a piece's weights (a rule's, 2^4 at most, and its visits' ages): q D^2 <=
+// 18, q <= log2(e) / w0, with D the largest distance along x or y between the grid's box and the
+// visits'.  Dwells of several lengths spread the weights further, which takes from the 18; +inf: none.
+double fp16_age(const dd_scan *scan, const dd::GridBox &g) {
+    double ex, ey;
+    box_reach(scan, g, ex, ey);
+    const double range = 18.0 - std::log2(scan->tau_max / scan->tau_min);
+    if (!(range >= 6.0)) return INFINITY;
+    const double D = std::max(ex, ey), w0 = 1.44269504088896340736 * (D * D) * (1.0 + 1e-6) / range;
+    const double a = (w0 - 2.0 * scan->s) / (4.0 * scan->kappa) + scan->tau_max;
+    return std::isfinite(a) ? std::max(a, 0.0) : INFINITY;
 }
 
 // The snapshot's first visit past each band.
@@ -84,7 +105,9 @@ cudaError_t prepare_kernel() {
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess || dev >= 64) return err;
     if (done.load() & (uint64_t(1) << dev)) return cudaSuccess;
-    err = cudaFuncSetAttribute(ddk::grid_quad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ddk::kGqSmemBytes);
+    err = cudaFuncSetAttribute(ddk::grid_quad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ddk::kGqSmemBytes);
+    if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(ddk::grid_quad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ddk::kGqSmemBytes);
     if (err == cudaSuccess) done.fetch_or(uint64_t(1) << dev);
     return err;
 }
@@ -101,7 +124,7 @@ struct GridEngine::Tables {
     std::vector<int> cta_off;                            // first run of each CTA, per launch n_cta + 1
     std::vector<int64_t> ax_offs, vis_offs, rec_offs;
     std::vector<int64_t> part_tiles, out_tiles;          // tiles of the jobs that write partial rows, the field
-    struct Span { int64_t k0, k1, split; };              // rows of k of a job; from split on: n > 2
+    struct Span { int64_t k0, k1, split; };              // rows of k of a job; from split on: BF16 pieces
     std::vector<Span> spans;
     std::vector<ddk::GqGroup> groups;                    // raster snapshots summed by segments of lags
     std::vector<ddk::GqSegment> segs;
@@ -153,6 +176,9 @@ int GridEngine::add_table(const dd_scan *scan, const GridBox &g, const double *s
     band_ages(scan, g, contract, age);
     ddk::GqTable tb{src + 2 * scan->n, src + 3 * scan->n, scan->s, scan->kappa, tdim, t->n_vis, t->n_rows, t->n_rec, nact, 0, {}};
     band_starts(scan, age, tdim, nact, tb.vb);
+    const double a16 = fp16_age(scan, g);
+    if (!std::isinf(a16))
+        tb.n_fp16 = (int)std::min<int64_t>(tb.vb[kGqBands], std::upper_bound(scan->T.begin(), scan->T.end(), tdim - a16) - scan->T.begin());
     t->tabs.push_back(tb);
     t->vis_offs.push_back(t->n_vis);
     t->rec_offs.push_back(t->n_rec);
@@ -171,6 +197,8 @@ int GridEngine::add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M, 
         const double last = std::floor((double)M - age[b]);             // lag M - i >= age
         tb.vb[b + 1] = last >= 0.0 ? std::max(tb.vb[b], (int)std::min((double)M, last + 1.0)) : tb.vb[b];
     }
+    const double oldest = std::floor((double)M - fp16_age(scan, g));
+    if (oldest >= 0.0) tb.n_fp16 = (int)std::min((double)tb.vb[kGqBands], oldest + 1.0);
     t->tabs.push_back(tb);
     t->vis_offs.push_back(t->n_vis);
     t->rec_offs.push_back(t->n_rec);
@@ -206,7 +234,7 @@ void GridEngine::add_span(const dd_scan *scan, const float4 *srcF, int grid, int
     j.out_off = out_off;
     j.pref = scan->pref;
     t->jobs.push_back(j);
-    const int mid = std::min(std::max(tb.vb[2], i0), kc);
+    const int mid = std::min(std::max(tb.n_fp16, i0), kc);
     t->spans.push_back({tb.k_off + rows_before(tb.vb, i0), tb.k_off + rows_before(tb.vb, kc), tb.k_off + rows_before(tb.vb, mid)});
 }
 
@@ -270,7 +298,7 @@ void GridEngine::place_rows(size_t k, int P) {
     }
 }
 
-cudaError_t GridEngine::finish(bool two_launches) {
+cudaError_t GridEngine::finish() {
     const int sms = sm_count();
     // Cost of a run: its rows of k times the factors formed per row (32 positions at a time),
     // plus about 500 rows' worth of factors for its start, drain and output.
@@ -280,11 +308,11 @@ cudaError_t GridEngine::finish(bool two_launches) {
         return (int64_t)((nc + 31) / 32 + (nr + 31) / 32 + 1);
     };
     constexpr int64_t kRunCost = 2000;
-    for (int launch = 0; launch < (two_launches ? 2 : 1); ++launch) {
+    for (int launch = 0; launch < 2; ++launch) {
         auto span = [&](size_t j, int64_t &k0, int64_t &k1) {
             const Tables::Span &s = t->spans[j];
             k0 = launch == 0 ? s.k0 : s.split;
-            k1 = launch == 0 && two_launches ? s.split : s.k1;
+            k1 = launch == 0 ? s.split : s.k1;
         };
         int64_t total = 0;
         for (size_t j = 0; j < t->jobs.size(); ++j) {
@@ -439,8 +467,9 @@ cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t s
     auto contraction = [&](int k, const char *name, cudaStream_t s) -> cudaError_t {
         if (t->n_cta[k] == 0) return cudaSuccess;
         const int *off = cta + (k == 0 || t->n_cta[0] == 0 ? 0 : t->n_cta[0] + 1);
+        auto *const kernel = k == 0 ? ddk::grid_quad_kernel<false> : ddk::grid_quad_kernel<true>;
         return scoped(name, s, [&] {
-            ddk::grid_quad_kernel<<<(unsigned)t->n_cta[k], ddk::kGqThreads, ddk::kGqSmemBytes, s>>>(
+            kernel<<<(unsigned)t->n_cta[k], ddk::kGqThreads, ddk::kGqSmemBytes, s>>>(
                 jobs, runs, off, t->rows, t->ax, t->part, withhold ? 1 : 0);
         });
     };

@@ -18,20 +18,31 @@
 // and h <= 0.33 with four, in pieces of 7 and 12 MMAs per 16 visits; here 16 rows of k take 3
 // MMAs, two nodes reach h = 0.143 and three 0.76.)
 //
-// Factors are formed in FP32 and split into two FP16 pieces, F 2^14 = h + l 2^-11 (each the
-// round-to-nearest of what is left: 2^-23 of F; -l is what is stored); X_h Y_h accumulates in one FP32 tensor-memory
-// accumulator and X_h Y_l + X_l Y_h in a second (X_l Y_l, 2^-22 at most and of either sign, is
-// left out).  The factors are taken relative to the tile: p = floor(q dxmin^2) moves from Y's
-// exponent to X's (dxmin: the visit's distance from the tile's columns), so that X's largest value
-// is about 1, and the piece's largest Y is scaled to 1 .. 2.  What the FP16 pieces drop is
-// then below 2^-49 of the tile's largest term.
+// Factors are formed in FP32 and split into 16-bit pieces, in one of two forms.
+//   BF16: F = h + m + l, each the round-to-nearest of what is left (2^-24 of F, FP32's exponent
+//     range); six products, X_h Y_h, X_h Y_m, X_m Y_h, X_m Y_m, X_h Y_l, X_l Y_h.
+//   FP16: F 2^14 = h + l 2^-11 (2^-23 of F down to F = 2^-26, then an absolute 2^-49; -l is what is
+//     stored); three products, X_h Y_h, X_h Y_l, X_l Y_h (X_l Y_l, 2^-22 at most and of either sign,
+//     is left out).
+// FP16 takes the visits old enough that no factor reaches below 2^-24 of the largest anywhere on the
+// grid (fp16_age of dd_grid.cu); BF16 the rest, so that the field keeps FP32's relative accuracy where
+// it is many orders below its peak: with FP16 pieces alone it was off by 3e-5 at 1e-8 to 1e-12 of
+// the peak and lost below that (64 x 64 visits, D = 1e-15 .. 6e-14); now 4e-7 to 1.3e-5 down to 1e-32
+// of it, as the exponents' own rounding.  All in BF16 pieces: 200 us instead of 172 for 256 x 256
+// points x 65,536 visits x 2 snapshots, 1313 instead of 1142 for 512 uneven scans (all in FP16: 171,
+// 996).  One kernel that chose per piece: 196, 1307.
+// The leading products accumulate in one FP32 tensor-memory accumulator and the rest in a second.
+// The factors are taken relative to the tile: p = floor(q dxmin^2) moves from Y's exponent to X's
+// (dxmin: the visit's distance from the tile's columns), so that X's largest value is about 1, and
+// the piece's largest Y is scaled to 1 .. 2.
 //
 // The tensor core's FP32 accumulation drops low bits of every product against the running sum:
 // with the leading products of 512 rows of k in one accumulator the field came out 2e-6 low.  So
 // the leading accumulator takes one stage of 64 rows of k (four MMAs), and four warps add the
 // stages up in FP32 registers while the next one forms in a second accumulator set; the other
-// products, 2^-11 as large, accumulate over a piece of up to 384 rows.  What four MMAs still
-// lose, 1.5e-7 to 2.5e-7 of the field on average, is put back by the factor kGqUnbias.
+// products, 2^-8 or 2^-11 as large, accumulate over a piece of up to 384 rows.  What four MMAs
+// still lose in FP16 pieces, 1.5e-7 to 2.5e-7 of the field on average, is put back by the factor
+// kGqUnbias.
 //
 // One CTA per SM walks its list of runs (a run: one tile of one snapshot, a range of k), piece by
 // piece.  Three warps fetch a piece's rows of k and visits and turn them into coefficients
@@ -44,11 +55,10 @@
 //
 // Measured (GB300, a call with its other kernels, before: two contractions of 7 and 12 MMAs per 16
 // visits beside a CUDA-core tile kernel for the last visits): 256 x 256 points x 65,536 visits
-// x 2 snapshots 306 -> 170 us (this kernel 103 us: 34,400 K steps, 3,000 clocks per stage and
-// SM, the producers' instruction latency with the MMAs' 2,200 behind them); 512 uneven scans on
-// their probe grids 1683 -> 984 us; 64 row snapshots of a 64 x 64 raster on 128 x 128 points
-// 223 -> 126 us.  Error against 64 bits (2-norm) 3.2e-7, 1.0e-6 and 2.1e-7 -> 0.8e-7, 1.9e-7
-// and 0.6e-7.
+// x 2 snapshots 306 -> 172 us (34,400 K steps; 3,000 clocks per stage of FP16 pieces and SM, the
+// producers' instruction latency); 512 uneven scans on their probe grids 1683 -> 1142 us; 64 row
+// snapshots of a 64 x 64 raster on 128 x 128 points 223 -> 83 us (with shared sums, below).  Error
+// against 64 bits (2-norm) 3.2e-7, 1.0e-6 and 2.1e-7 -> 0.3e-7, 1.4e-7 and 0.6e-7.
 #pragma once
 #include <cstdint>
 
@@ -137,7 +147,7 @@ struct GqTable {
     const double *T, *TAU;
     double s, kappa, tdim;
     int64_t vis_off, k_off, rec_off;
-    int n_vis, pad;
+    int n_vis, n_fp16;              // visits, and how many of them, the oldest, take FP16 pieces
     int vb[kGqBands + 1];
 };
 // A grid of points: columns x0 + c dx, rows y0 + r dy [m] (one product, one sum), as float-float
@@ -197,12 +207,19 @@ constexpr int kGqThreads = 768;
 constexpr int kGqRegsProd = 64, kGqRegsMid = 48, kGqRegsDrain = 176;
 static_assert(kGqRegsProd * 32 * kGqProdWarps + kGqRegsMid * 128 + kGqRegsDrain * 32 * kGqDrainWarps <= 80 * kGqThreads, "register split");
 constexpr int kGqTile = 128;
-constexpr int kGqStageK = 64, kGqBufs = 3, kGqPieceK = 384;
+constexpr int kGqStageK = 64, kGqPieceK = 384;
 // K steps (16 rows of k) of a run at most: the draining warps add a run's stages of four steps in plain
 // FP32, whose rounding grows with the square root of their number (3e-7 of the sum for 512)
 constexpr int64_t kGqRunSteps = 4 * 512;
-constexpr int kGqPieceBytes = kGqTile * kGqStageK * 2;         // one FP16 piece of one side: 16 KB
-constexpr int kGqBufBytes = 4 * kGqPieceBytes;                 // Y_h, Y_l, X_h, X_l
+constexpr int kGqPieceBytes = kGqTile * kGqStageK * 2;         // one 16-bit piece of one side: 16 KB
+// A stage: Y's pieces, then X's; h, l in FP16 and three stages in the ring, or h, m, l in BF16 and two.
+template <bool kBf16>
+struct GqForm {
+    static constexpr int kPieces = kBf16 ? 3 : 2, kBufs = kBf16 ? 2 : 3;
+    static constexpr int kSideBytes = kPieces * kGqPieceBytes, kBufBytes = 2 * kSideBytes;
+};
+constexpr int kGqRingBytes = 12 * kGqPieceBytes, kGqMaxBufs = 3;
+static_assert(GqForm<false>::kBufs * GqForm<false>::kBufBytes == kGqRingBytes && GqForm<true>::kBufs * GqForm<true>::kBufBytes == kGqRingBytes, "ring");
 // A piece as the warps see it.  The rings hold 8: the coefficient warps are at most two pieces
 // ahead of the producers, these three stages ahead of the MMAs, and those two stages ahead of the
 // draining warps.
@@ -211,10 +228,10 @@ struct GqPiece {
     int W;
     int nk, nc, nr;                         // rows of k, the tile's columns and rows
     int first, last, final;                 // of the run; final: the CTA's last piece
-    float scale;                            // 2^(e - 28)
+    float scale;                            // of the products: 2^m (BF16), 2^(m - 28) (FP16)
 };
 struct GqSmem {
-    unsigned char bufs[kGqBufs * kGqBufBytes];
+    unsigned char bufs[kGqRingBytes];
     float4 a[2][2][kGqPieceK / 2];          // [piece parity][side]: (-x, -x', -q, -q') of two rows of k
     float2 e[2][2][kGqPieceK / 2];          // exponent offsets; side 0: rows, 1: columns
     float2 pos[2][2][kGqTile];              // [run parity][side]: offsets of the tile's rows, columns
@@ -222,10 +239,11 @@ struct GqSmem {
     float wmax[kGqCoefWarps];
     int2 stage_info[8];                     // piece ring slot + 8 x first + 16 x last stage of the
                                             // piece, rows of k
-    uint64_t cfull[2], cempty[2], full[kGqBufs], empty[kGqBufs], done[2], free1[2], free2[2], idle;
+    uint64_t cfull[2], cempty[2], full[kGqMaxBufs], empty[kGqMaxBufs], done[2], free1[2], free2[2], idle;
     uint32_t tmem;
     int failed;
 };
+// (FP16; BF16 pieces take none)
 constexpr float kGqUnbias = 1.0f + 0x1p-22f;
 constexpr float kGqFarExp = 150.0f;         // q rho^2 from which a row of k is left out
 constexpr int kGqSmemBytes = (int)sizeof(GqSmem) + 1024;
@@ -244,6 +262,19 @@ __device__ __forceinline__ float2 f16x2_to_f2(uint32_t w) {
     asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n cvt.f32.f16 %0, l;\n cvt.f32.f16 %1, h;\n}\n"
         : "=f"(f.x), "=f"(f.y) : "r"(w));
     return f;
+}
+__device__ __forceinline__ uint32_t bf16x2_rn(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// v - the rounded pair w, exact (mixed-precision multiply-add)
+__device__ __forceinline__ float2 bf16x2_rest(uint32_t w, float2 v) {
+    float2 r;
+    asm("{\n .reg .b16 x, y, n;\n mov.b32 {x, y}, %2;\n mov.b16 n, 0xBF80;\n"
+        " fma.rn.f32.bf16 %0, x, n, %3;\n fma.rn.f32.bf16 %1, y, n, %4;\n}\n"
+        : "=f"(r.x), "=f"(r.y) : "r"(w), "f"(v.x), "f"(v.y));
+    return r;
 }
 // instruction descriptor of kind::f16: FP32 accumulator, FP16 A and B, both K-major
 __host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N) {
@@ -282,30 +313,45 @@ __device__ __forceinline__ bool gq_wait_warp(uint64_t *bar, uint32_t parity, vol
 // conversion rounds back to zero.  (On the integer pipe: the FMA pipe is the busier one.)
 __device__ __forceinline__ float gq_scale(float v, int n) { return __int_as_float(__float_as_int(v) + (n << 23)); }
 
-// Factors of 8 rows of k at one position, as two 16-byte core-matrix rows (h at dst, -l one piece
-// further).  a: (-x, -x', -q, -q') of four pairs of rows of k, e: their exponent offsets; the
+// Factors of 8 rows of k at one position, as 16-byte core-matrix rows one piece apart (FP16: h, -l;
+// BF16: h, m, l).  a: (-x, -x', -q, -q') of four pairs of rows of k, e: their exponent offsets; the
 // position is din + dfr (kSplit: dfr is added last, else the sum is in din).
-template <bool kSplit>
+template <bool kSplit, bool kBf16>
 __device__ __forceinline__ void gq_factors(const float4 (&a)[4], const float2 (&e)[4], float din, float dfr,
                                            unsigned char *dst) {
-    uint32_t h[4], l[4];
+    uint32_t h[4], m[4], l[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         float2 d = __fadd2_rn(f2(din, din), f2(a[u].x, a[u].y));
         if (kSplit) d = __fadd2_rn(d, f2(dfr, dfr));
         const float2 g = __ffma2_rn(f2(a[u].z, a[u].w), __fmul2_rn(d, d), e[u]);
-        const float F0 = gq_scale(ex2_approx(g.x), 14), F1 = gq_scale(ex2_approx(g.y), 14);
-        h[u] = f16x2_rn(F0, F1);
-        // h - F, exact (mixed-precision subtraction)
-        float r0, r1;
-        asm("{\n .reg .b16 x, y;\n mov.b32 {x, y}, %2;\n sub.rn.f32.f16 %0, x, %3;\n sub.rn.f32.f16 %1, y, %4;\n}\n"
-            : "=f"(r0), "=f"(r1) : "r"(h[u]), "f"(F0), "f"(F1));
-        l[u] = f16x2_rn(gq_scale(r0, 11), gq_scale(r1, 11));
+        if (kBf16) {
+            const float2 F = f2(ex2_approx(g.x), ex2_approx(g.y));
+            h[u] = bf16x2_rn(F.x, F.y);
+            const float2 r = bf16x2_rest(h[u], F);
+            m[u] = bf16x2_rn(r.x, r.y);
+            const float2 q = bf16x2_rest(m[u], r);
+            l[u] = bf16x2_rn(q.x, q.y);
+        } else {
+            const float F0 = gq_scale(ex2_approx(g.x), 14), F1 = gq_scale(ex2_approx(g.y), 14);
+            h[u] = f16x2_rn(F0, F1);
+            // h - F, exact (mixed-precision subtraction)
+            float r0, r1;
+            asm("{\n .reg .b16 x, y;\n mov.b32 {x, y}, %2;\n sub.rn.f32.f16 %0, x, %3;\n sub.rn.f32.f16 %1, y, %4;\n}\n"
+                : "=f"(r0), "=f"(r1) : "r"(h[u]), "f"(F0), "f"(F1));
+            l[u] = f16x2_rn(gq_scale(r0, 11), gq_scale(r1, 11));
+        }
     }
     *reinterpret_cast<uint4 *>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4 *>(dst + kGqPieceBytes) = make_uint4(l[0], l[1], l[2], l[3]);
+    if (kBf16) {
+        *reinterpret_cast<uint4 *>(dst + kGqPieceBytes) = make_uint4(m[0], m[1], m[2], m[3]);
+        *reinterpret_cast<uint4 *>(dst + 2 * kGqPieceBytes) = make_uint4(l[0], l[1], l[2], l[3]);
+    } else {
+        *reinterpret_cast<uint4 *>(dst + kGqPieceBytes) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
 }
 // The same for the positions of mask (bit q: din[q]), the coefficients read once.
+template <bool kBf16>
 __device__ __forceinline__ void gq_group(const float4 *as, const float2 *es, const float (&din)[4], const float (&dfr)[4],
                                          bool split, uint32_t mask, unsigned char *dst) {
     float4 a[4];
@@ -318,20 +364,22 @@ __device__ __forceinline__ void gq_group(const float4 *as, const float2 *es, con
     if (split) {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (mask & (1u << q)) gq_factors<true>(a, e, din[q], dfr[q], dst + 512 * q);
+            if (mask & (1u << q)) gq_factors<true, kBf16>(a, e, din[q], dfr[q], dst + 512 * q);
     } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (mask & (1u << q)) gq_factors<false>(a, e, din[q], 0.0f, dst + 512 * q);
+            if (mask & (1u << q)) gq_factors<false, kBf16>(a, e, din[q], 0.0f, dst + 512 * q);
     }
 }
 
 // withhold (tests): no MMA is issued and no accumulator set is committed, so that the waits run
 // out.
+template <bool kBf16>
 __global__ void __launch_bounds__(kGqThreads, 1)
 grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs, const int *__restrict__ cta_off,
                  const GqRow *__restrict__ rows, const float2 *__restrict__ ax, float *__restrict__ partial,
                  int withhold) {
+    constexpr int kGqBufs = GqForm<kBf16>::kBufs, kGqBufBytes = GqForm<kBf16>::kBufBytes, kGqSideBytes = GqForm<kBf16>::kSideBytes;
     extern __shared__ unsigned char gq_raw[];
     GqSmem &sm = *reinterpret_cast<GqSmem *>((reinterpret_cast<uintptr_t>(gq_raw) + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -367,7 +415,7 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kGqRegsProd));
         // ---- the producers: warp = 8 rows of k of the row side (warps 0-7) or the column side
         const int side = warp >> 3, kg = warp & 7;
-        unsigned char *const dst0 = sm.bufs + side * 2 * kGqPieceBytes + kg * (kGqTile * 16) + lane * 16;
+        unsigned char *const dst0 = sm.bufs + side * kGqSideBytes + kg * (kGqTile * 16) + lane * 16;
         int stage = 0, run = -1;
         float din[4], dfr[4];
         bool split = false;
@@ -402,7 +450,7 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
                     sm.stage_info[stage & 7] = make_int2((piece & 7) + (k0 == 0 ? 8 : 0) + (nk - k0 <= kGqStageK ? 16 : 0),
                                                          min(nk - k0, kGqStageK));
                 if (k0 + 8 * kg < ((nk + 15) & ~15))
-                    gq_group(&sm.a[piece & 1][side][(k0 + 8 * kg) / 2], &sm.e[piece & 1][side][(k0 + 8 * kg) / 2], din, dfr,
+                    gq_group<kBf16>(&sm.a[piece & 1][side][(k0 + 8 * kg) / 2], &sm.e[piece & 1][side][(k0 + 8 * kg) / 2], din, dfr,
                              split, mask, dst0 + b * kGqBufBytes);
                 fence_proxy_async_smem();
                 __syncwarp();
@@ -426,7 +474,8 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
                 if (!gq_wait(sm.full + b, (uint32_t)(stage / kGqBufs) & 1u, failed)) break;
                 const int2 info = sm.stage_info[stage & 7];
                 const GqPiece &P = sm.piece[info.x & 7];
-                const uint32_t idesc = umma_idesc_f16(kGqTile, (P.nc + 15) & ~15);
+                const int nc = (P.nc + 15) & ~15;
+                const uint32_t idesc = kBf16 ? umma_idesc_bf16(kGqTile, nc) : umma_idesc_f16(kGqTile, nc);
                 const bool fresh = info.x & 8, final = (info.x & 16) && P.final;
                 if (fresh) {
                     ++piece;
@@ -437,15 +486,20 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
                 const uint32_t d1 = tmem + 128u * set, d2 = tmem + 256u + 128u * (piece & 1);
                 // descriptors count in 16 bytes; a K step is two groups of 8 rows of k
                 const uint64_t y = desc0 + (uint64_t)(b * (kGqBufBytes / 16));
-                constexpr uint64_t kP = kGqPieceBytes / 16, kStep = 2 * kGqTile;
+                constexpr uint64_t kP = kGqPieceBytes / 16, kX = kGqSideBytes / 16, kStep = 2 * kGqTile;
                 const int steps = withhold ? 0 : (info.y + 15) / 16;
 #pragma unroll
                 for (int k = 0; k < kGqStageK / 16; ++k)
                     if (k < steps) {
-                        const uint64_t yk = y + k * kStep, xk = yk + 2 * kP;
+                        const uint64_t yk = y + k * kStep, xk = yk + kX;
                         umma_bf16(d1, yk, xk, idesc, k > 0 ? 1 : 0);
                         umma_bf16(d2, yk, xk + kP, idesc, k > 0 || !fresh ? 1 : 0);
                         umma_bf16(d2, yk + kP, xk, idesc, 1);
+                        if (kBf16) {
+                            umma_bf16(d2, yk + kP, xk + kP, idesc, 1);
+                            umma_bf16(d2, yk, xk + 2 * kP, idesc, 1);
+                            umma_bf16(d2, yk + 2 * kP, xk, idesc, 1);
+                        }
                     }
                 if (!withhold) umma_commit(sm.done + set);
                 umma_commit(sm.empty + b);
@@ -544,8 +598,8 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
                         sm.pos[(r - run0) & 1][s][c] = f2(n - (s ? ox : oy), (v.x - n) + v.y);
                     }
                 }
-                if (t == 0) {                // 2^(m - 28), 0 below the FP32 normal range
-                    const int ex = (int)fmaxf(m, -1000.0f) - 28;
+                if (t == 0) {                // the scale is 0 below the FP32 normal range
+                    const int ex = (int)fmaxf(m, -1000.0f) - (kBf16 ? 0 : 28);
                     sm.piece[piece & 7] = GqPiece{out, W, nk, nc, nr, kk == 0, kk + kGqPieceK >= run.nk,
                                                   kk + kGqPieceK >= run.nk && r + 1 == run1,
                                                   ex > -127 ? __int_as_float((ex + 127) << 23) : 0.0f};
@@ -587,10 +641,10 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
                 tc_fence_before();
                 __syncwarp();
             };
-            drain(128u * set, scale * kGqUnbias);
+            drain(128u * set, kBf16 ? scale : scale * kGqUnbias);
             if (lane == 0) gq_mbar_arrive(sm.free1 + set);
             if (!(info & 16)) continue;
-            drain(256u + 128u * (piece & 1), scale * (-1.0f / 2048.0f));   // of -l
+            drain(256u + 128u * (piece & 1), kBf16 ? scale : scale * (-1.0f / 2048.0f));   // FP16: of -l
             const int last = P.last, final = P.final, nr = P.nr, W = P.W;
             float *const out = P.out + (int64_t)(32 * quarter + lane) * W;
             __syncwarp();

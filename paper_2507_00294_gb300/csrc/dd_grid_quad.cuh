@@ -41,8 +41,8 @@
 // the leading accumulator takes one stage of 64 rows of k (four MMAs), and four warps add the
 // stages up in FP32 registers while the next one forms in a second accumulator set; the other
 // products, 2^-8 or 2^-11 as large, accumulate over a piece of up to 384 rows.  What four MMAs
-// still lose in FP16 pieces, 1.5e-7 to 2.5e-7 of the field on average, is put back by the factor
-// kGqUnbias.
+// still lose of the field on average, 1.0e-7 to 1.7e-7 in FP16 pieces and 0.3e-7 to 1.5e-7 in BF16,
+// is put back by a factor (gq_unbias); one to three MMAs lose under 0.5e-7.
 //
 // One CTA per SM walks its list of runs (a run: one tile of one snapshot, a range of k), piece by
 // piece.  Three warps fetch a piece's rows of k and visits and turn them into coefficients
@@ -243,8 +243,12 @@ struct GqSmem {
     uint32_t tmem;
     int failed;
 };
-// (FP16; BF16 pieces take none)
-constexpr float kGqUnbias = 1.0f + 0x1p-22f;
+// What the tensor core's accumulation of a full stage drops, put back by halves of an FP32 ulp: its two
+// accumulator sets take these factors in turn.  (Stages of fewer steps lose less than half an ulp.)
+template <bool kBf16>
+__device__ __forceinline__ float gq_unbias(int set) {
+    return kBf16 ? (set ? 1.0f + 0x1p-23f : 1.0f) : (set ? 1.0f + 0x1p-22f : 1.0f + 0x1p-23f);
+}
 constexpr float kGqFarExp = 150.0f;         // q rho^2 from which a row of k is left out
 constexpr int kGqSmemBytes = (int)sizeof(GqSmem) + 1024;
 static_assert(kGqSmemBytes <= 227 * 1024, "shared memory of a CTA");
@@ -623,7 +627,8 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
             const int set = stage & 1;
             if (!gq_wait_warp(sm.done + set, (uint32_t)(stage >> 1) & 1u, failed)) break;
             tc_fence_after();
-            const int info = sm.stage_info[stage & 7].x;
+            const int2 stage_info = sm.stage_info[stage & 7];
+            const int info = stage_info.x;
             const GqPiece &P = sm.piece[info & 7];
             const int nc = P.nc;
             const float scale = P.scale;
@@ -641,7 +646,7 @@ grid_quad_kernel(const GqJob *__restrict__ jobs, const GqRun *__restrict__ runs,
                 tc_fence_before();
                 __syncwarp();
             };
-            drain(128u * set, kBf16 ? scale : scale * kGqUnbias);
+            drain(128u * set, stage_info.y > kGqStageK - 16 ? scale * gq_unbias<kBf16>(set) : scale);
             if (lane == 0) gq_mbar_arrive(sm.free1 + set);
             if (!(info & 16)) continue;
             drain(256u + 128u * (piece & 1), kBf16 ? scale : scale * (-1.0f / 2048.0f));   // FP16: of -l

@@ -1,5 +1,6 @@
 """FP32-mixed grids far below the field's peak: the contraction (dd_grid_quad.cuh) keeps FP32's relative
-accuracy at every point, in single calls, snapshots that share their sums, and batches."""
+accuracy at every point, in single calls, snapshots that share their sums, and batches; and sums of few
+visits carry no correction for what full stages of MMAs lose."""
 import numpy as np
 import pytest
 
@@ -35,3 +36,17 @@ def test_tail(cuda, spec):
     plan = b.Batch([scan, scan], None, times[:2], "mixed", grids=[g, g])
     out = plan.run(device=cuda).cpu().numpy().reshape(2, -1)
     assert relative_errors(out, exact[:2], TAIL).max() <= RTOL
+
+
+@pytest.mark.parametrize("n", [4, 16, 48, 64, 80, 128, 512])
+def test_mean_error_of_few_visits(cuda, n):
+    """Visits that contribute alike: the mean error is at most half of 2^-22, the largest factor that puts
+    back what four MMAs lose (a sum of one to three MMAs loses less than 2^-24)."""
+    spec = w.ScanSpec(n, 1, D_m2s=6e-14)
+    p = spec.pitch_m
+    g = (0.0, -32.0 * p, n / 64.0 * p, p, 64, 64)
+    times = np.array([3e5, 1e6, 3e6]) * spec.dwell_s
+    scan = b.Scan(spec)
+    mixed = b.dd_field_on_grid(scan, *g, times, "mixed", device=cuda).cpu().numpy()
+    exact = b.dd_field_on_grid(scan, *g, times, "fp64", device=cuda).cpu().numpy()
+    assert abs((mixed / exact - 1.0).mean()) <= 2.0 ** -23

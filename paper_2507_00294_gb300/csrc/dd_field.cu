@@ -618,14 +618,15 @@ constexpr int64_t kQuadMinSide = 32, kQuadMinPts = 4096;
 constexpr double kQuadRecentVisits = 256.0;
 
 // Narrow grids (below 64 columns, half of the CUDA-core grid tile's 128, whose lanes mostly idle
-// there) take the final kernel of dd_grid.cu with every visit left to it.  A CTA there walks all of
-// a snapshot's visits for 32 columns x 16 rows (0.11 us per visit), where the grid tile splits them;
-// so few visits, or CTAs to fill the GPU with.  A scan of n visits, tile against walk in us:
-// 256 visits, 16 x 16 points, 256 snapshots: 96, 68; 32 snapshots: 73, 57; 576 visits, 32 x 32: 512
-// CTAs 189, 121, 128 CTAs 111, 105; 1024 visits, 48 x 48: 1536 CTAs 341, 302, 384 CTAs 146, 176.
+// there) take the final kernel of dd_grid.cu with every visit left to it, a CTA per 32 columns x 16 rows
+// and snapshot: where there are many snapshots of few visits.  The grid tile splits a snapshot's visits
+// over CTAs, which is faster for few snapshots, and it pays for idle lanes in each group of four.
+// Tile against walk in us, 16 x 16, 32 x 32 and 48 x 48 points: 144 visits, 32 snapshots 63, 44; 64, 52; 58, 44; 256
+// visits, 16 58, 68; 58, 58; 56, 60; 32 62, 60 (all three); 400 visits, 64 72, 83; 79, 83; 84, 89; 128 83, 85; 102, 85;
+// 124, 101; 1024 visits, 64 79, 93; 117, 95; 134, 126; 128 124, 97; 168, 117; 187, 179; 1600 visits of 48 x 48 points,
+// 256 snapshots 379, 414.
 bool narrow_grid(const ddk::GridDesc &g, int64_t n_t, int64_t n_visits) {
-    const int64_t ctas = ((g.W + 31) / 32) * ((g.H + 15) / 16) * n_t;
-    return g.W < 64 && g.H < dd::kGridMaxSide && n_visits <= 1024 && ctas >= (n_visits <= 256 ? 32 : n_visits);
+    return g.W < 64 && g.H < dd::kGridMaxSide && n_visits <= 1024 && n_t >= (n_visits <= 256 ? 32 : 128);
 }
 
 // Snapshots (indices k0 .. k1 - 1 in time order) of a whole raster on the dwell lattice that share

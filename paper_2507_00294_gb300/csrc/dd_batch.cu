@@ -525,24 +525,28 @@ dd_status create_plan(const dd_scan *const *scans, int32_t n_scans, const int64_
 extern "C" {
 
 dd_status dd_batch_create(const dd_scan *const *scans, int32_t n_scans, const int64_t *pt_offsets,
-                          const double *times_s, dd_precision prec, dd_batch **out) {
+                          const double *times_s, dd_precision prec, dd_batch **out) try {
     dd::clear_error();
     if (!scans || !pt_offsets || !times_s || !out || n_scans < 1)
         return dd::fail(DD_EINVAL, "dd_batch_create: NULL argument or no scans");
     if (prec != DD_FP64 && prec != DD_MIXED) return dd::fail(DD_EINVAL, "dd_batch_create: unknown precision");
     return create_plan(scans, n_scans, pt_offsets, nullptr, nullptr, times_s, prec, out);
+} catch (...) {
+    return dd::fail_exception("dd_batch_create");
 }
 
 dd_status dd_batch_create_grid(const dd_scan *const *scans, int32_t n_scans, const double *grid_xy,
-                               const int64_t *grid_wh, const double *times_s, dd_precision prec, dd_batch **out) {
+                               const int64_t *grid_wh, const double *times_s, dd_precision prec, dd_batch **out) try {
     dd::clear_error();
     if (!scans || !grid_xy || !grid_wh || !times_s || !out || n_scans < 1)
         return dd::fail(DD_EINVAL, "dd_batch_create_grid: NULL argument or no scans");
     if (prec != DD_FP64 && prec != DD_MIXED) return dd::fail(DD_EINVAL, "dd_batch_create_grid: unknown precision");
     return create_plan(scans, n_scans, nullptr, grid_xy, grid_wh, times_s, prec, out);
+} catch (...) {
+    return dd::fail_exception("dd_batch_create_grid");
 }
 
-dd_status dd_batch_tune(dd_batch *b, const double *pts_xy_m, int32_t *chosen) {
+dd_status dd_batch_tune(dd_batch *b, const double *pts_xy_m, int32_t *chosen) try {
     dd::clear_error();
     if (!b || (!pts_xy_m && !b->on_grid)) return dd::fail(DD_EINVAL, "dd_batch_tune: NULL argument");
     if (b->on_grid) pts_xy_m = nullptr;                  // grid plans form their points
@@ -578,9 +582,11 @@ dd_status dd_batch_tune(dd_batch *b, const double *pts_xy_m, int32_t *chosen) {
     }
     if (chosen) *chosen = best_v;
     return DD_OK;
+} catch (...) {
+    return dd::fail_exception("dd_batch_tune");
 }
 
-dd_status dd_batch_run(dd_batch *b, const double *pts_xy_m, double *out, void *cuda_stream) {
+dd_status dd_batch_run(dd_batch *b, const double *pts_xy_m, double *out, void *cuda_stream) try {
     dd::clear_error();
     if (!b || (!pts_xy_m && !b->on_grid) || !out) return dd::fail(DD_EINVAL, "dd_batch_run: NULL argument");
     cudaStream_t stream = (cudaStream_t)cuda_stream;
@@ -623,6 +629,8 @@ dd_status dd_batch_run(dd_batch *b, const double *pts_xy_m, double *out, void *c
         DD_CUDA_TRY(cudaMemcpyAsync(out, dst, (size_t)b->total_pts * sizeof(double), cudaMemcpyDeviceToHost, stream));
     if (out_host || pts_host) DD_CUDA_TRY(cudaStreamSynchronize(stream));
     return DD_OK;
+} catch (...) {
+    return dd::fail_exception("dd_batch_run");
 }
 
 void dd_batch_destroy(dd_batch *b) {
@@ -651,7 +659,7 @@ dd_status dd_batch_info(const dd_batch *b, int64_t *n_items, int64_t *pairs, int
 
 dd_status dd_field_batch(const dd_scan *const *scans, int32_t n_scans, const int64_t *pt_offsets,
                          const double *pts_xy_m, const double *times_s, dd_precision prec,
-                         double *out, void *cuda_stream) {
+                         double *out, void *cuda_stream) try {
     dd::clear_error();
     if (!pts_xy_m || !out) return dd::fail(DD_EINVAL, "dd_field_batch: NULL buffer");
     dd_batch *b = nullptr;
@@ -664,6 +672,8 @@ dd_status dd_field_batch(const dd_scan *const *scans, int32_t n_scans, const int
     }
     dd_batch_destroy(b);
     return st;
+} catch (...) {
+    return dd::fail_exception("dd_field_batch");
 }
 
 }  // extern "C"

@@ -671,15 +671,17 @@ dd_status dose_range(const dd_scan *scan, dd_precision prec, int64_t j0, int64_t
 
 }  // namespace
 
-extern "C" dd_status dd_per_probe_dose(const dd_scan *scan, dd_precision prec, double *out, void *cuda_stream) {
+extern "C" dd_status dd_per_probe_dose(const dd_scan *scan, dd_precision prec, double *out, void *cuda_stream) try {
     dd::clear_error();
     if (!scan || !out) return dd::fail(DD_EINVAL, "dd_per_probe_dose: NULL argument");
     if (prec != DD_FP64 && prec != DD_MIXED) return dd::fail(DD_EINVAL, "dd_per_probe_dose: unknown precision");
     return dose_range(scan, prec, 0, scan->n, out, cuda_stream);
+} catch (...) {
+    return dd::fail_exception("dd_per_probe_dose");
 }
 
 extern "C" dd_status dd_per_probe_dose_range(const dd_scan *scan, dd_precision prec, int64_t j0, int64_t j1,
-                                             double *out, void *cuda_stream) {
+                                             double *out, void *cuda_stream) try {
     dd::clear_error();
     if (!scan) return dd::fail(DD_EINVAL, "dd_per_probe_dose_range: NULL scan");
     if (prec != DD_FP64 && prec != DD_MIXED)
@@ -689,6 +691,8 @@ extern "C" dd_status dd_per_probe_dose_range(const dd_scan *scan, dd_precision p
     if (j1 == j0) return DD_OK;
     if (!out) return dd::fail(DD_EINVAL, "dd_per_probe_dose_range: NULL output");
     return dose_range(scan, prec, j0, j1, out, cuda_stream);
+} catch (...) {
+    return dd::fail_exception("dd_per_probe_dose_range");
 }
 
 // ---------------------------------------------------------------------------------
@@ -817,7 +821,7 @@ dd_status run_dose_noalloc(const dd_scan *scan, double *out, cudaStream_t stream
 }  // namespace
 
 extern "C" dd_status dd_per_probe_dose_noalloc(const dd_scan *scan, dd_precision prec, double *out,
-                                               void *cuda_stream) {
+                                               void *cuda_stream) try {
     dd::clear_error();
     if (!scan || !out) return dd::fail(DD_EINVAL, "dd_per_probe_dose_noalloc: NULL argument");
     if (prec != DD_FP64 && prec != DD_MIXED)
@@ -834,4 +838,6 @@ extern "C" dd_status dd_per_probe_dose_noalloc(const dd_scan *scan, dd_precision
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     if (prec == DD_MIXED) return run_dose_noalloc<ddk::CfgMixed>(scan, out, stream, scratch);
     return run_dose_noalloc<ddk::CfgF64>(scan, out, stream, scratch);
+} catch (...) {
+    return dd::fail_exception("dd_per_probe_dose_noalloc");
 }

@@ -803,7 +803,7 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
 
 extern "C" dd_status dd_field_at_times(const dd_scan *scan, const double *pts_xy_m, int64_t n_pts,
                                        const double *times_s, int64_t n_t, dd_precision prec,
-                                       double *out, void *cuda_stream) {
+                                       double *out, void *cuda_stream) try {
     dd::clear_error();
     if (!scan) return dd::fail(DD_EINVAL, "dd_field_at_times: NULL scan");
     if (n_pts < 0 || n_t < 0) return dd::fail(DD_EINVAL, "dd_field_at_times: negative size");
@@ -825,11 +825,13 @@ extern "C" dd_status dd_field_at_times(const dd_scan *scan, const double *pts_xy
     const ddk::GridDesc list;                                     // an explicit point list
     if (prec == DD_MIXED) return run_field<ddk::CfgMixed>(scan, pts_xy_m, n_pts, list, times, out, stream);
     return run_field<ddk::CfgF64>(scan, pts_xy_m, n_pts, list, times, out, stream);
+} catch (...) {
+    return dd::fail_exception("dd_field_at_times");
 }
 
 extern "C" dd_status dd_field_on_grid(const dd_scan *scan, double x0_m, double y0_m, double dx_m, double dy_m,
                                       int64_t n_cols, int64_t n_rows, const double *times_s, int64_t n_t,
-                                      dd_precision prec, double *out, void *cuda_stream) {
+                                      dd_precision prec, double *out, void *cuda_stream) try {
     dd::clear_error();
     if (!scan) return dd::fail(DD_EINVAL, "dd_field_on_grid: NULL scan");
     if (n_cols < 0 || n_rows < 0 || n_t < 0) return dd::fail(DD_EINVAL, "dd_field_on_grid: negative size");
@@ -859,6 +861,8 @@ extern "C" dd_status dd_field_on_grid(const dd_scan *scan, double x0_m, double y
     if (prec == DD_MIXED && narrow_grid(g, n_t, scan->n)) return run_grid_mixed(scan, g, times, false, out, stream);
     if (prec == DD_MIXED) return run_field<ddk::CfgMixed>(scan, nullptr, n_pts, g, times, out, stream);
     return run_field<ddk::CfgF64>(scan, nullptr, n_pts, g, times, out, stream);
+} catch (...) {
+    return dd::fail_exception("dd_field_on_grid");
 }
 
 extern "C" dd_status dd_field_check(void) {
@@ -872,7 +876,7 @@ extern "C" dd_status dd_field_check(void) {
 
 extern "C" dd_status dd_field_grid_split(const dd_scan *scan, double x0_m, double y0_m, double dx_m, double dy_m,
                                          int64_t n_cols, int64_t n_rows, const double *times_s, int64_t n_t,
-                                         int64_t *prefix, int64_t *prefix_deg2) {
+                                         int64_t *prefix, int64_t *prefix_deg2) try {
     dd::clear_error();
     if (!scan) return dd::fail(DD_EINVAL, "dd_field_grid_split: NULL scan");
     if (n_cols < 0 || n_rows < 0 || n_t < 0) return dd::fail(DD_EINVAL, "dd_field_grid_split: negative size");
@@ -897,4 +901,6 @@ extern "C" dd_status dd_field_grid_split(const dd_scan *scan, double x0_m, doubl
         if (prefix_deg2) prefix_deg2[order[k]] = tp.on ? tp.K2[k] : 0;
     }
     return DD_OK;
+} catch (...) {
+    return dd::fail_exception("dd_field_grid_split");
 }

@@ -60,6 +60,9 @@ namespace dd {
 // Record `msg` as this thread's last error and return `st`.
 dd_status fail(dd_status st, const std::string &msg);
 dd_status fail_cuda(cudaError_t err, const char *what);
+// In a catch (...) block of an entry point: DD_ENOMEM for the exception in flight (host tables that
+// could not be allocated).
+dd_status fail_exception(const char *entry);
 void clear_error();
 
 // Device copy of the scan's dimensionless visit arrays on the current device, usable by

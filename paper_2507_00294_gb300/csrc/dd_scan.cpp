@@ -11,6 +11,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <deque>
+#include <exception>
 #include <mutex>
 #include <new>
 #include <unordered_map>
@@ -26,6 +27,16 @@ static thread_local std::string g_last_error;
 dd_status fail(dd_status st, const std::string &msg) {
     g_last_error = msg;
     return st;
+}
+
+dd_status fail_exception(const char *entry) {
+    try {
+        throw;
+    } catch (const std::exception &e) {
+        return fail(DD_ENOMEM, std::string(entry) + ": out of host memory (" + e.what() + ")");
+    } catch (...) {
+        return fail(DD_ENOMEM, std::string(entry) + ": unknown exception");
+    }
 }
 
 dd_status fail_cuda(cudaError_t err, const char *what) {

@@ -28,6 +28,14 @@ void box_reach(const dd_scan *scan, const dd::GridBox &g, double &ex, double &ey
     ey = std::max(std::max(ya, yb) - scan->y_lo, scan->y_hi - std::min(ya, yb));
 }
 
+// The largest squared distance between them.
+double reach2(const dd_scan *scan, const dd::GridBox &g) {
+    double ex, ey;
+    box_reach(scan, g, ex, ey);
+    // margins for the points' own rounding
+    return (ex * ex + ey * ey) * (1.0 + 1e-6) + 1e-6;
+}
+
 // Ages (in dwells) from which every visit of the scan takes each band at every point of the
 // grid (+inf: none): h = rho^2 dq <= kGqH for rho^2 up to R2, the largest squared distance
 // between the grid's box and the visits' box, r = w1/w0 - 1 <= kGqR, and the dwell over.  With
@@ -38,10 +46,7 @@ void band_ages(const dd_scan *scan, const dd::GridBox &g, bool contract, double 
         for (double &a : age) a = INFINITY;
         return;
     }
-    double ex, ey;
-    box_reach(scan, g, ex, ey);
-    // margins for the points' own rounding
-    const double R2 = (ex * ex + ey * ey) * (1.0 + 1e-6) + 1e-6;
+    const double R2 = reach2(scan, g);
     const double c = 4.0 * scan->kappa * scan->tau_max;
     double prev = INFINITY;
     for (int b = 0; b < kGqBands; ++b) {
@@ -66,6 +71,24 @@ double fp16_age(const dd_scan *scan, const dd::GridBox &g) {
     const double D = std::max(ex, ey), w0 = 1.44269504088896340736 * (D * D) * (1.0 + 1e-6) / range;
     const double a = (w0 - 2.0 * scan->s) / (4.0 * scan->kappa) + scan->tau_max;
     return std::isfinite(a) ? std::max(a, 0.0) : INFINITY;
+}
+
+// Whether FP16 pieces hold the field of a table's visits from i0 on, at ages age(i), to its full precision
+// at every point within R2, so that all of them can take those pieces.  What a piece drops is at most
+// 3 2^-50 of its largest weight per row of k; weights within a factor of three of one another in a piece,
+// and the L = ln(w1/w0) of visits one after the other adding up to at most S = ln(w(oldest) / w(youngest)),
+// that is 9 2^-50 (S + 1) in all, and FP32's rounding is 2^-24 of the field.  The field is at least what
+// the older half of the visits leave at the largest distance.
+template <typename Age>
+bool fp16_everywhere(const dd_scan *scan, double R2, int i0, int n, int banded, const Age &age) {
+    const int half = (n - i0) / 2;
+    if (half < 1 || banded <= i0) return false;
+    auto w1 = [&](int i) { return 2.0 * scan->s + 4.0 * scan->kappa * age(i); };
+    const double c = 4.0 * scan->kappa, w_half = w1(i0 + half - 1) - c * scan->tau_max;
+    if (!(w_half > 0.0)) return false;
+    const double S = std::log(w1(i0) / (w1(banded - 1) - c * scan->tau_max));
+    const double least = half * std::log1p(c * scan->tau_min / w1(i0)) * std::exp(-R2 / w_half);
+    return least >= 9.0 * 0x1p-26 * (S + 1.0);
 }
 
 // The snapshot's first visit past each band.
@@ -124,6 +147,7 @@ struct GridEngine::Tables {
     std::vector<int> cta_off;                            // first run of each CTA, per launch n_cta + 1
     std::vector<int64_t> ax_offs, vis_offs, rec_offs;
     std::vector<int64_t> part_tiles, out_tiles;          // tiles of the jobs that write partial rows, the field
+    std::vector<double> tab_R2;                          // per table: largest squared distance to the grid
     struct Span { int64_t k0, k1, split; };              // rows of k of a job; from split on: BF16 pieces
     std::vector<Span> spans;
     std::vector<ddk::GqGroup> groups;                    // raster snapshots summed by segments of lags
@@ -180,6 +204,7 @@ int GridEngine::add_table(const dd_scan *scan, const GridBox &g, const double *s
     if (!std::isinf(a16))
         tb.n_fp16 = (int)std::min<int64_t>(tb.vb[kGqBands], std::upper_bound(scan->T.begin(), scan->T.end(), tdim - a16) - scan->T.begin());
     t->tabs.push_back(tb);
+    t->tab_R2.push_back(reach2(scan, g));
     t->vis_offs.push_back(t->n_vis);
     t->rec_offs.push_back(t->n_rec);
     t->n_vis += nact;
@@ -200,6 +225,7 @@ int GridEngine::add_lag_table(const dd_scan *scan, const GridBox &g, int64_t M, 
     const double oldest = std::floor((double)M - fp16_age(scan, g));
     if (oldest >= 0.0) tb.n_fp16 = (int)std::min((double)tb.vb[kGqBands], oldest + 1.0);
     t->tabs.push_back(tb);
+    t->tab_R2.push_back(reach2(scan, g));
     t->vis_offs.push_back(t->n_vis);
     t->rec_offs.push_back(t->n_rec);
     t->n_vis += M;
@@ -234,7 +260,10 @@ void GridEngine::add_span(const dd_scan *scan, const float4 *srcF, int grid, int
     j.out_off = out_off;
     j.pref = scan->pref;
     t->jobs.push_back(j);
-    const int mid = std::min(std::max(tb.n_fp16, i0), kc);
+    const bool fp16 = kc > std::max(tb.n_fp16, i0) && fp16_everywhere(scan, t->tab_R2[table], i0, tb.n_vis, kc, [&](int i) {
+        return tb.T ? tb.tdim - scan->T[(size_t)i] : (double)(tb.n_vis - i);
+    });
+    const int mid = fp16 ? kc : std::min(std::max(tb.n_fp16, i0), kc);
     t->spans.push_back({tb.k_off + rows_before(tb.vb, i0), tb.k_off + rows_before(tb.vb, kc), tb.k_off + rows_before(tb.vb, mid)});
 }
 
@@ -301,18 +330,19 @@ void GridEngine::place_rows(size_t k, int P) {
 cudaError_t GridEngine::finish() {
     const int sms = sm_count();
     // Cost of a run: its rows of k times the factors formed per row (32 positions at a time),
-    // plus about 500 rows' worth of factors for its start, drain and output.
+    // plus about 130 rows' worth of factors for its start, drain and output (500 left 64 short segments
+    // in 110 runs of 152 SMs: 8 us longer).
     auto row_cost = [](const ddk::GqJob &j, int tile) {
         const int nc = std::min(j.tw, j.W - (tile % j.n_tc) * j.tw);
         const int nr = std::min(ddk::kGqTile, j.H - (tile / j.n_tc) * ddk::kGqTile);
         return (int64_t)((nc + 31) / 32 + (nr + 31) / 32 + 1);
     };
-    constexpr int64_t kRunCost = 2000;
+    constexpr int64_t kRunCost = 1200;
     for (int launch = 0; launch < 2; ++launch) {
         auto span = [&](size_t j, int64_t &k0, int64_t &k1) {
             const Tables::Span &s = t->spans[j];
-            k0 = launch == 0 ? s.k0 : s.split;
-            k1 = launch == 0 ? s.split : s.k1;
+            k0 = launch == 0 ? s.split : s.k0;
+            k1 = launch == 0 ? s.k1 : s.split;
         };
         int64_t total = 0;
         for (size_t j = 0; j < t->jobs.size(); ++j) {
@@ -464,10 +494,12 @@ cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t s
              ddk::grid_quad_prep_kernel<<<(unsigned)((n_prep + 63) / 64), 64, 0, stream>>>(prep);
          })) != cudaSuccess)
         return err;
-    auto contraction = [&](int k, const char *name, cudaStream_t s) -> cudaError_t {
+    // launch 0: the BF16 pieces, the longer runs; launch 1: the FP16 pieces
+    auto contraction = [&](int k, cudaStream_t s) -> cudaError_t {
         if (t->n_cta[k] == 0) return cudaSuccess;
+        const char *name = k == 0 || t->n_cta[0] == 0 ? "field_grid_tc" : "field_grid_tc4";
         const int *off = cta + (k == 0 || t->n_cta[0] == 0 ? 0 : t->n_cta[0] + 1);
-        auto *const kernel = k == 0 ? ddk::grid_quad_kernel<false> : ddk::grid_quad_kernel<true>;
+        auto *const kernel = k == 0 ? ddk::grid_quad_kernel<true> : ddk::grid_quad_kernel<false>;
         return scoped(name, s, [&] {
             kernel<<<(unsigned)t->n_cta[k], ddk::kGqThreads, ddk::kGqSmemBytes, s>>>(
                 jobs, runs, off, t->rows, t->ax, t->part, withhold ? 1 : 0);
@@ -488,9 +520,9 @@ cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t s
         if ((err = cudaEventRecord(fork, stream)) != cudaSuccess) return err;
         if ((err = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return err;
     }
-    if ((err = contraction(0, "field_grid_tc", stream)) != cudaSuccess) return err;
+    if ((err = contraction(0, stream)) != cudaSuccess) return err;
     if ((err = recent(t->part_tiles, l.parto, second)) != cudaSuccess) return err;
-    if ((err = contraction(1, "field_grid_tc4", second)) != cudaSuccess) return err;
+    if ((err = contraction(1, second)) != cudaSuccess) return err;
     if (both) {
         if ((err = cudaEventRecord(join, side)) != cudaSuccess) return err;
         if ((err = cudaStreamWaitEvent(stream, join, 0)) != cudaSuccess) return err;

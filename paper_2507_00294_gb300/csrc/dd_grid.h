@@ -56,8 +56,8 @@ class GridEngine {
     // Device bytes that add_table takes, and the most a visit can.
     static int64_t table_device_bytes(const dd_scan *scan, const GridBox &g, double tdim, int nact, bool contract);
     static constexpr int64_t kMostVisitBytes = 512;      // 32 nodes
-    // Splits the contraction into runs for the device's SMs, in two launches: the rows of k in FP16
-    // pieces, and the rest in BF16 pieces.
+    // Splits the contraction into runs for the device's SMs, in two launches: the rows of k in BF16
+    // pieces, and those in FP16 pieces.
     cudaError_t finish();
 
     size_t table_bytes() const;          // host tables, uploaded to the workspace's first bytes

@@ -24,13 +24,14 @@
 //   FP16: F 2^14 = h + l 2^-11 (2^-23 of F down to F = 2^-26, then an absolute 2^-49; -l is what is
 //     stored); three products, X_h Y_h, X_h Y_l, X_l Y_h (X_l Y_l, 2^-22 at most and of either sign,
 //     is left out).
-// FP16 takes the visits old enough that no factor reaches below 2^-24 of the largest anywhere on the
-// grid (fp16_age of dd_grid.cu); BF16 the rest, so that the field keeps FP32's relative accuracy where
-// it is many orders below its peak: with FP16 pieces alone it was off by 3e-5 at 1e-8 to 1e-12 of
-// the peak and lost below that (64 x 64 visits, D = 1e-15 .. 6e-14); now 4e-7 to 1.3e-5 down to 1e-32
-// of it, as the exponents' own rounding.  All in BF16 pieces: 200 us instead of 172 for 256 x 256
-// points x 65,536 visits x 2 snapshots, 1313 instead of 1142 for 512 uneven scans (all in FP16: 171,
-// 996).  One kernel that chose per piece: 196, 1307.
+// FP16 takes the visits old enough that no factor reaches below 2^-18 anywhere on the grid (fp16_age of
+// dd_grid.cu), and every visit where the field itself stays so close to its largest term that what FP16
+// drops is below FP32's rounding (fp16_everywhere); BF16 the rest, so that the field keeps FP32's
+// relative accuracy where it is many orders below its peak: with FP16 pieces alone it was off by 3e-5 at
+// 1e-8 to 1e-12 of the peak and lost below that (64 x 64 visits, D = 1e-15 .. 6e-14); now 4e-7 to
+// 1.3e-5 down to 1e-32 of it, as the exponents' own rounding.  All in BF16 pieces: 200 us instead of
+// 156 for 256 x 256 points x 65,536 visits x 2 snapshots, 1313 instead of 1150 for 512 uneven scans
+// (all in FP16: 171, 1000).  One kernel that chose per piece: 196, 1307.
 // The leading products accumulate in one FP32 tensor-memory accumulator and the rest in a second.
 // The factors are taken relative to the tile: p = floor(q dxmin^2) moves from Y's exponent to X's
 // (dxmin: the visit's distance from the tile's columns), so that X's largest value is about 1, and
@@ -55,10 +56,10 @@
 //
 // Measured (GB300, a call with its other kernels, before: two contractions of 7 and 12 MMAs per 16
 // visits beside a CUDA-core tile kernel for the last visits): 256 x 256 points x 65,536 visits
-// x 2 snapshots 306 -> 172 us (34,400 K steps; 3,000 clocks per stage of FP16 pieces and SM, the
-// producers' instruction latency); 512 uneven scans on their probe grids 1683 -> 1142 us; 64 row
-// snapshots of a 64 x 64 raster on 128 x 128 points 223 -> 83 us (with shared sums, below).  Error
-// against 64 bits (2-norm) 3.2e-7, 1.0e-6 and 2.1e-7 -> 0.3e-7, 1.4e-7 and 0.6e-7.
+// x 2 snapshots 306 -> 156 us (3,000 clocks per stage of FP16 pieces and SM, the producers'
+// instruction latency; 3,900 in BF16); 512 uneven scans on their probe grids 1683 -> 1150 us; 64 row
+// snapshots of a 64 x 64 raster on 128 x 128 points 223 -> 80 us (with shared sums, below).  Error
+// against 64 bits (2-norm) 3.2e-7, 1.0e-6 and 2.1e-7 -> 0.3e-7, 1.5e-7 and 0.6e-7.
 #pragma once
 #include <cstdint>
 

@@ -415,8 +415,8 @@ def dd_sur_conv3x3(x, w, bias, mask, out, epilogue, dilation=1, stream=None):
 
 
 def dd_field_grid_split(scan, x0, y0, dx, dy, n_cols, n_rows, times_s, degree2=False):
-    """Per snapshot, the number of leading visits dd_field_on_grid sums on the tensor cores
-    (FP32-mixed); host-only.  degree2: also return how many of them in the degree-2 form."""
+    """Per snapshot, the number of leading visits on the degree-4 exponent series at every point of
+    the grid; host-only.  degree2: also return how many of them are on the degree-2 series."""
     t = np.ascontiguousarray(np.asarray(times_s, dtype=np.float64).reshape(-1))
     out = np.zeros(len(t), dtype=np.int64)
     out2 = np.zeros(len(t), dtype=np.int64)

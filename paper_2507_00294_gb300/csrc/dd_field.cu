@@ -703,21 +703,26 @@ dd_status run_grid_mixed(const dd_scan *scan, const ddk::GridDesc &grid, const s
     const dd::GridBox box{grid.x0, grid.y0, grid.dx, grid.dy, grid.W, grid.H};
     double all = 0.0;
     for (int n : nact) all += (double)n;
+    std::vector<int> recents;                    // left to the CUDA cores, where there can be many
     if (contract && all > kQuadRecentVisits * n_t) {
         const double age = dd::GridEngine::banded_age(scan, box);
         double recent = 0.0;
-        for (int k = 0; k < n_t; ++k)
-            recent += lattice ? std::min((double)nact[k], std::ceil(age))
-                              : (double)(nact[k] - std::min<int64_t>(nact[k], std::upper_bound(scan->T.begin(), scan->T.end(), tdim[k] - age) - scan->T.begin()));
+        recents.resize((size_t)n_t);
+        for (int k = 0; k < n_t; ++k) {
+            recents[k] = lattice ? (int)std::min((double)nact[k], std::ceil(age))
+                                 : nact[k] - (int)std::min<int64_t>(nact[k], std::upper_bound(scan->T.begin(), scan->T.end(), tdim[k] - age) - scan->T.begin());
+            recent += recents[k];
+        }
         if (recent > kQuadRecentVisits * n_t && recent > 0.5 * all && shift_groups(scan, grid, tdim, lattice, 0, n_t).groups.empty())
             return run_field<ddk::CfgMixed>(scan, nullptr, n_pts, grid, times, out, stream);
     }
-    // snapshots of a pass: their tables (off the lattice; on it one serves them all) and about four
-    // partial rows each, so that the workspace stays in the allocator's 1 GiB class
+    // snapshots of a pass: their tables (off the lattice; on it one serves them all), about four
+    // partial rows each and those of many recent visits, so that the workspace stays in the
+    // allocator's 1 GiB class
     constexpr int64_t kPassBytes = 960 * (int64_t(1) << 20);
     const bool few = lattice || all * (double)dd::GridEngine::kMostVisitBytes < 0.5 * (double)kPassBytes;
     auto pass_bytes = [&](int k) {
-        return 16 * n_pts + (few ? 0 : dd::GridEngine::table_device_bytes(scan, box, tdim[k], nact[k], contract));
+        return (16 + (recents.empty() ? 0 : recents[k] / 512 * 4)) * n_pts + (few ? 0 : dd::GridEngine::table_device_bytes(scan, box, tdim[k], nact[k], contract));
     };
     dd_status st = DD_OK;
     const double *src = dd::device_sources(scan, stream, &st);

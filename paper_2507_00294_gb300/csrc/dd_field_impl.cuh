@@ -689,8 +689,7 @@ __device__ __forceinline__ void field_tile(TileSmem<Cfg, TCH> &sm, const double 
                         // one polynomial degree for the warp, from every lane's own h and a.  The
                         // limits are compared on the upper words (no FP64 compares; a and h
                         // are never negative): a value at a limit's own word takes the higher
-                        // degree, and a pair at a's word evaluates its (tiny) term.  A lane
-                        // whose own a is 745 or more adds 0.
+                        // degree.  A lane whose own a is 745 or more adds 0.
                         // (not a NaN: its word is past infinity's, and it reaches pair_term)
                         auto beyond = [](double v) {
                             return (uint32_t)(__double2hiint(v) - kZeroWord) <= (uint32_t)(0x7FF00000 - kZeroWord);

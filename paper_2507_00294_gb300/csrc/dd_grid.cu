@@ -395,7 +395,8 @@ cudaError_t GridEngine::finish() {
             t->runs[(size_t)(off[c] + round)] = list[(size_t)order[k].second];
         }
     }
-    // more than kGqFinSplit recent visits are split while the tiles leave places for CTAs (two waves)
+    // more than kGqFinSplit recent visits are split while the tiles leave places for CTAs (two waves),
+    // more than kGqFinMost always
     const size_t n_jobs = t->jobs.size();
     int64_t tiles = 0;
     int longest = 0;
@@ -407,7 +408,7 @@ cudaError_t GridEngine::finish() {
     for (size_t k = 0; k < n_jobs; ++k) {
         const int n = t->jobs[k].r1 - t->jobs[k].r0;
         const int64_t parts = n > ddk::kGqFinSplit ? (n + ddk::kGqFinVisits - 1) / ddk::kGqFinVisits : 1;
-        place_rows(k, (int)std::max<int64_t>(1, std::min(most, parts)));
+        place_rows(k, (int)std::max<int64_t>((n + ddk::kGqFinMost - 1) / ddk::kGqFinMost, std::max<int64_t>(1, std::min(most, parts))));
     }
     t->part_tiles.reserve(t->jobs.size() + 1);
     t->out_tiles.reserve(t->jobs.size() + 1);

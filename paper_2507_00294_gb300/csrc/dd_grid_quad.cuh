@@ -769,16 +769,18 @@ __global__ void __launch_bounds__(64) grid_quad_prep_kernel(const GqPrep P) {
 }
 
 // The recent visits at a tile of 32 columns x 16 rows (lane = column, warp = 4 rows), each at the
-// cheapest series that holds it over the warp's points (the classes of the field kernel), summed over
-// stages of 32 visits and, with the contraction's partial rows, in compensated FP32 (a scan can have
-// thousands of recent visits); out = pref times that.  Bound by the series' issue for many recent
+// cheapest series that holds it over the warp's points (the classes of the field kernel), at most
+// kGqFinMost of them in one plain FP32 sum, plus the partial rows of the contraction and of earlier
+// recent visits, in compensated FP32; out = pref times that.  Bound by the series' issue for many recent
 // visits, by the partial rows' loads for few.
 constexpr int kGqFinRows = 16, kGqFinThreads = 128, kGqFinStage = 32;
 // More than kGqFinSplit recent visits of a job are split into parts of kGqFinVisits while the GPU has
 // places for their CTAs: a CTA walks 0.15 us per visit, so that 65,536 of them on 64 x 64 points (8
 // CTAs) took 9.8 ms in one piece each and take 0.36 ms split.  Fewer stay in one piece: a second
 // launch and its fork cost the host 20 us (256 visits, 16 x 16 points, 256 snapshots: 64 us, split 85).
-constexpr int kGqFinSplit = 256, kGqFinVisits = 64, kGqFinResident = 8;      // resident CTAs per SM
+// More than kGqFinMost (16 stages) always are, so that no plain sum grows longer: over 2048 stages it
+// rounds to 7e-7; a compensated sum in the loop instead took 2 us of 47 on the 16 x 16 case.
+constexpr int kGqFinSplit = 256, kGqFinVisits = 64, kGqFinMost = 512, kGqFinResident = 8;    // CTAs per SM
 __global__ void __launch_bounds__(kGqFinThreads, kGqFinResident)
 grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict__ tile_offs, int n_jobs,
                        const RecF32 *__restrict__ rec, const float2 *__restrict__ ax, float *partial,
@@ -812,7 +814,7 @@ grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict
         bx0 = fminf(bx0, __shfl_xor_sync(0xffffffffu, bx0, o));
         bx1 = fmaxf(bx1, __shfl_xor_sync(0xffffffffu, bx1, o));
     }
-    BlockSum<float> sum[4];
+    float2 run[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
     for (int v0 = J.r0; v0 < J.r1; v0 += kGqFinStage) {
         const int cnt = min(kGqFinStage, J.r1 - v0);
         __syncthreads();
@@ -872,20 +874,20 @@ grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict
                 }
             }
         }
-        sum[0].add(acc[0].x);
-        sum[1].add(acc[0].y);
-        sum[2].add(acc[1].x);
-        sum[3].add(acc[1].y);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) run[k] = __fadd2_rn(run[k], acc[k]);
     }
     if (c >= J.W || row0 >= J.H) return;
     const int nr = min(4, J.H - row0);
     if (J.out_off < 0) {                     // the recent visits as a partial row
         float *const o = partial + J.t_off + J.row * J.t_stride + (int64_t)row0 * J.W + c;
+        const float v[4] = {run[0].x, run[0].y, run[1].x, run[1].y};
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-            if (e < nr) o[(int64_t)e * J.W] = sum[e].result();
+            if (e < nr) o[(int64_t)e * J.W] = v[e];
         return;
     }
+    BlockSum<float> sum[4];
     const float *const p = partial + J.t_off + (int64_t)row0 * J.W + c;
 #pragma unroll 2
     for (int k = 0; k < J.nq; ++k) {
@@ -895,6 +897,10 @@ grid_quad_final_kernel(const GqJob *__restrict__ jobs, const int64_t *__restrict
 #pragma unroll
         for (int e = 0; e < 4; ++e) sum[e].add(v[e]);
     }
+    sum[0].add(run[0].x);
+    sum[1].add(run[0].y);
+    sum[2].add(run[1].x);
+    sum[3].add(run[1].y);
     double *const o = out + J.out_off + (int64_t)row0 * J.W + c;
 #pragma unroll
     for (int e = 0; e < 4; ++e)

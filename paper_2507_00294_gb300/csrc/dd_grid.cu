@@ -85,7 +85,7 @@ bool fp16_everywhere(const dd_scan *scan, double R2, int i0, int n, int banded, 
     if (half < 1 || banded <= i0) return false;
     auto w1 = [&](int i) { return 2.0 * scan->s + 4.0 * scan->kappa * age(i); };
     const double c = 4.0 * scan->kappa, w_half = w1(i0 + half - 1) - c * scan->tau_max;
-    if (!(w_half > 0.0)) return false;
+    if (!(R2 < 16.0 * w_half)) return false;         // (e^-16 is below the bound)
     const double S = std::log(w1(i0) / (w1(banded - 1) - c * scan->tau_max));
     const double least = half * std::log1p(c * scan->tau_min / w1(i0)) * std::exp(-R2 / w_half);
     return least >= 9.0 * 0x1p-26 * (S + 1.0);
@@ -395,31 +395,42 @@ cudaError_t GridEngine::finish() {
             t->runs[(size_t)(off[c] + round)] = list[(size_t)order[k].second];
         }
     }
+    // places of the partial rows and the tiles of the recent visits, every job's in one part
+    const size_t n_jobs = t->jobs.size();
+    int64_t n_part = 0, n_out = 0;
+    auto tile_tables = [&] {
+        n_part = n_out = 0;
+        t->part_tiles.resize(t->jobs.size() + 1);
+        t->out_tiles.resize(t->jobs.size() + 1);
+        for (size_t k = 0; k <= t->jobs.size(); ++k) {
+            t->part_tiles[k] = n_part;
+            t->out_tiles[k] = n_out;
+            if (k < t->jobs.size()) (t->jobs[k].out_off < 0 ? n_part : n_out) += fin_tiles(t->jobs[k]);
+        }
+    };
+    int longest = 0;
+    for (ddk::GqJob &j : t->jobs) {
+        const int n = j.r1 - j.r0;
+        j.t_off = t->n_part;
+        j.row = j.nq;
+        t->n_part += (int64_t)(j.nq + (j.out_off < 0 && n > 0 ? 1 : 0)) * j.t_stride;
+        longest = std::max(longest, n);
+    }
+    tile_tables();
     // more than kGqFinSplit recent visits are split while the tiles leave places for CTAs (two waves),
     // more than kGqFinMost always
-    const size_t n_jobs = t->jobs.size();
-    int64_t tiles = 0;
-    int longest = 0;
-    for (const ddk::GqJob &j : t->jobs) {
-        tiles += fin_tiles(j);
-        longest = std::max(longest, j.r1 - j.r0);
+    if (longest > ddk::kGqFinSplit) {
+        const int64_t most = std::max<int64_t>(1, 2 * ddk::kGqFinResident * (int64_t)sms / (n_part + n_out));
+        t->n_part = 0;
+        for (size_t k = 0; k < n_jobs; ++k) {
+            const int n = t->jobs[k].r1 - t->jobs[k].r0;
+            const int64_t parts = n > ddk::kGqFinSplit ? (n + ddk::kGqFinVisits - 1) / ddk::kGqFinVisits : 1;
+            place_rows(k, (int)std::max<int64_t>((n + ddk::kGqFinMost - 1) / ddk::kGqFinMost, std::max<int64_t>(1, std::min(most, parts))));
+        }
+        tile_tables();
     }
-    const int64_t most = longest > ddk::kGqFinSplit ? 2 * ddk::kGqFinResident * (int64_t)sms / tiles : 1;
-    for (size_t k = 0; k < n_jobs; ++k) {
-        const int n = t->jobs[k].r1 - t->jobs[k].r0;
-        const int64_t parts = n > ddk::kGqFinSplit ? (n + ddk::kGqFinVisits - 1) / ddk::kGqFinVisits : 1;
-        place_rows(k, (int)std::max<int64_t>((n + ddk::kGqFinMost - 1) / ddk::kGqFinMost, std::max<int64_t>(1, std::min(most, parts))));
-    }
-    t->part_tiles.reserve(t->jobs.size() + 1);
-    t->out_tiles.reserve(t->jobs.size() + 1);
-    int64_t n_part = 0, n_out = 0;
-    for (size_t k = 0; k <= t->jobs.size(); ++k) {
-        t->part_tiles.push_back(n_part);
-        t->out_tiles.push_back(n_out);
-        if (k == t->jobs.size()) break;
-        const ddk::GqJob &j = t->jobs[k];
-        (j.out_off < 0 ? n_part : n_out) += fin_tiles(j);
-    }
+    if (n_part == 0) t->part_tiles.clear();
+    if (n_out == 0) t->out_tiles.clear();
     for (size_t k = 0; k < t->segs.size(); ++k) {
         const ddk::GqJob &j = t->jobs[(size_t)t->seg_job[k]];
         t->segs[k].t_off = j.t_off;
@@ -466,7 +477,9 @@ void GridEngine::bind(void *workspace) {
     t->part = reinterpret_cast<float *>(take((size_t)t->n_part * sizeof(float)));
 }
 
-int64_t GridEngine::n_tiles() const { return t->out_tiles.empty() ? 0 : t->part_tiles.back() + t->out_tiles.back(); }
+int64_t GridEngine::n_tiles() const {
+    return (t->part_tiles.empty() ? 0 : t->part_tiles.back()) + (t->out_tiles.empty() ? 0 : t->out_tiles.back());
+}
 int64_t GridEngine::n_runs() const { return (int64_t)t->runs.size(); }
 
 cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t side, cudaEvent_t fork,
@@ -507,7 +520,7 @@ cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t s
         });
     };
     auto recent = [&](const std::vector<int64_t> &tiles, size_t o, cudaStream_t s) -> cudaError_t {
-        if (tiles.back() == 0) return cudaSuccess;
+        if (tiles.empty()) return cudaSuccess;
         return scoped("field_grid_mixed", s, [&] {
             ddk::grid_quad_final_kernel<<<(unsigned)tiles.back(), ddk::kGqFinThreads, 0, s>>>(
                 jobs, offs(o), (int)t->jobs.size(), t->rec, t->ax, t->part, out);
@@ -515,7 +528,7 @@ cudaError_t GridEngine::enqueue(double *out, cudaStream_t stream, cudaStream_t s
     };
     // beside the first contraction launch: the second, and the recent visits that go to partial
     // rows (all on one stream: 86 us instead of 72 on 64 shared row snapshots)
-    const bool both = side != nullptr && t->n_cta[0] > 0 && (t->n_cta[1] > 0 || t->part_tiles.back() > 0);
+    const bool both = side != nullptr && t->n_cta[0] > 0 && (t->n_cta[1] > 0 || !t->part_tiles.empty());
     cudaStream_t second = both ? side : stream;
     if (both) {
         if ((err = cudaEventRecord(fork, stream)) != cudaSuccess) return err;

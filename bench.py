@@ -221,8 +221,8 @@ def recorded_pipes(kernel):
 
 def grid_kernel_lines(prof):
     """The grid field's kernels by their own events: launches and mean time.  field_grid_tc and
-    field_grid_tc4 (the Gauss-Legendre contraction's two launches, the rows of k with one or two
-    nodes and the rest) and field_grid_mixed (the most recent visits) overlap one another on two
+    field_grid_tc4 (the Gauss-Legendre contraction's two launches, the rows of k in BF16 pieces and
+    those in FP16 pieces; one launch alone is field_grid_tc) and field_grid_mixed (the most recent visits) overlap one another on two
     streams; field_reduce sums the segments of lags that the raster's snapshots share."""
     names = ("coef_mixed", "field_grid_tc", "field_grid_tc4", "field_grid_mixed", "field_reduce")
     return {k: {"launches": prof[k][0], "avg_launch_ms": prof[k][1] / prof[k][0]} for k in names if prof.get(k, (0,))[0]}

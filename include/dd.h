@@ -146,10 +146,12 @@ dd_status dd_field_at_times(const dd_scan *scan, const double *pts_xy_m, int64_t
    buffer.  In FP32-mixed precision, on grids of at least 32 x 32 and 4096 points, every
    visit but the last few is a short sum of Gaussians (Gauss-Legendre nodes) that split into
    column and row factors, and their sum over visits is a matrix product on the tensor cores
-   (two FP16 pieces of each FP32 factor, FP32 accumulation); smaller grids split the
-   low-degree pair terms into column and row factors on the CUDA cores.  The result then
-   differs from dd_field_at_times by the FP32 rounding, within the same error
-   budget.  times_s and out as in dd_field_at_times.  A grid with no columns, rows or
+   (three BF16 pieces of each FP32 factor, or two FP16 pieces where those lose nothing at any
+   point of the grid; FP32 accumulation); smaller grids, and grids so wide that most visits
+   would be left over, split the low-degree pair terms into column and row factors on the
+   CUDA cores.  The result then differs from dd_field_at_times by the FP32 rounding, within
+   the same error budget, also far below the field's peak.  times_s and out as in
+   dd_field_at_times.  A grid with no columns, rows or
    snapshots is a no-op.
    Errors: DD_EINVAL (NULL scan/buffer, negative sizes, non-finite origin or spacing, more
    than 2^31 points), DD_ENOMEM, DD_ECUDA.  A tensor-core wait that gave up (an
@@ -167,8 +169,8 @@ dd_status dd_field_on_grid(const dd_scan *scan, double x0_m, double y0_m, double
    largest squared distance between the grid's box and the visits' box, with dq bounded
    through the scan's longest dwell (dq <= c / ((w1 - c) w1), c = 4 D tau_max, at
    w1 = 2 sigma^2 + 4 D (t - t_i)), so the qualifying visits are those started by
-   t - dT*: prefixes.  dd_field_on_grid in FP32-mixed precision sums all of them on the
-   tensor cores (and the visits after them up to h = 218, too).  0 for grids smaller than
+   t - dT*: prefixes.  Where dd_field_on_grid takes the tensor cores, all of them are summed
+   there (and the visits after them up to h = 218, too).  0 for grids smaller than
    64 x 64 points and for snapshots with no qualifying visit; the degree-4 band is left out
    where its coefficients of (rho^2)^4 would leave the FP32 normal range.
    Errors: DD_EINVAL (NULL scan or buffers, negative sizes, non-finite grid or times,
@@ -208,8 +210,9 @@ dd_status dd_per_probe_dose_range(const dd_scan *scan, dd_precision prec, int64_
 /* Allocation-free variant of dd_per_probe_dose (the paper has no counterpart: this
    entry point exists for callers that cannot allocate device memory while they run,
    e.g. an acquisition loop that reserves its whole GPU memory budget before the scan
-   starts, or a host whose device allocator belongs to another framework).  Same
-   result as dd_per_probe_dose.  It calls no device allocator: its scratch lives in
+   starts, or a host whose device allocator belongs to another framework).  It always
+   takes the direct sum over earlier visits, so its result agrees with dd_per_probe_dose
+   within the precision's rounding.  It calls no device allocator: its scratch lives in
    one file-scope __device__ array of 8 MiB, which every GPU that loads the library
    holds until the process exits, so scans of at most 16384 visits are accepted
    (larger ones: DD_EINVAL with a message).  out must be device memory (else

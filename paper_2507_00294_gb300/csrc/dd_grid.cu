@@ -58,37 +58,50 @@ void band_ages(const dd_scan *scan, const dd::GridBox &g, bool contract, double 
     }
 }
 
-// Age (in dwells) from which a visit's factors stay within 2^-18 of 1 on the grid, so that FP16 pieces
-// (dd_grid_quad.cuh: full precision down to 2^-24 of a piece's largest) hold them at every point with
-// 2^6 left for the spread of a piece's weights (a rule's, 2^4 at most, and its visits' ages): q D^2 <=
-// 18, q <= log2(e) / w0, with D the largest distance along x or y between the grid's box and the
-// visits'.  Dwells of several lengths spread the weights further, which takes from the 18; +inf: none.
+// Longest time (in dwells) from one visit's start to the next's.
+double longest_step(const dd_scan *scan) {
+    const double diagonal = scan->pitch * std::hypot((double)scan->nx, (double)scan->ny);
+    return scan->tau_max + (scan->flyback + scan->blank + scan->blank_per_m * diagonal) / scan->dwell;
+}
+
+// Age (in dwells) from which FP16 pieces (dd_grid_quad.cuh: full precision down to 2^-24 of a piece's
+// largest factor) hold a visit's factors at every point of the grid: q D^2, q <= log2(e) / w0, with D the
+// largest distance along x or y between the grid's box and the visits', plus the spread of a piece's
+// weights within 24.  That is 4 for a rule's, and what dwells of several lengths and the ages of a
+// piece's visits (384 at most) make of L = ln(w1/w0).  At most 18 for q D^2; +inf: none.
 double fp16_age(const dd_scan *scan, const dd::GridBox &g) {
     double ex, ey;
     box_reach(scan, g, ex, ey);
-    const double range = 18.0 - std::log2(scan->tau_max / scan->tau_min);
+    const double D = std::max(ex, ey);
+    auto age = [&](double range) {
+        const double w0 = 1.44269504088896340736 * (D * D) * (1.0 + 1e-6) / range;
+        return std::max((w0 - 2.0 * scan->s) / (4.0 * scan->kappa) + scan->tau_max, scan->tau_max);
+    };
+    const double ages = std::log2(1.0 + (double)ddk::kGqPieceK * longest_step(scan) / age(18.0));
+    const double range = std::min(18.0, 20.0 - ages - std::log2(scan->tau_max / scan->tau_min));
     if (!(range >= 6.0)) return INFINITY;
-    const double D = std::max(ex, ey), w0 = 1.44269504088896340736 * (D * D) * (1.0 + 1e-6) / range;
-    const double a = (w0 - 2.0 * scan->s) / (4.0 * scan->kappa) + scan->tau_max;
-    return std::isfinite(a) ? std::max(a, 0.0) : INFINITY;
+    const double a = age(range);                     // (an older visit's ages spread less)
+    return std::isfinite(a) ? a : INFINITY;
 }
 
-// Whether FP16 pieces hold the field of a table's visits from i0 on, at ages age(i), to its full precision
+// Whether FP16 pieces hold the field of a table's visits [i0, i1), at ages age(i), to its full precision
 // at every point within R2, so that all of them can take those pieces.  What a piece drops is at most
-// 3 2^-50 of its largest weight per row of k; weights within a factor of three of one another in a piece,
-// and the L = ln(w1/w0) of visits one after the other adding up to at most S = ln(w(oldest) / w(youngest)),
-// that is 9 2^-50 (S + 1) in all, and FP32's rounding is 2^-24 of the field.  The field is at least what
-// the older half of the visits leave at the largest distance.
+// 3 2^-50 of its largest weight per row of k.  With weights a few times one another in a piece, and the
+// L = ln(w1/w0) of visits one after the other adding up to at most S = ln(w(oldest) / w(youngest)),
+// that is 32 2^-50 (S + 1) in all (more with dead times between visits, by the ages that they put into
+// the youngest piece), and FP32's rounding is 2^-24 of the field.  The field is at least what the older
+// half of the visits leave at the largest distance.
 template <typename Age>
-bool fp16_everywhere(const dd_scan *scan, double R2, int i0, int n, int banded, const Age &age) {
-    const int half = (n - i0) / 2;
+bool fp16_everywhere(const dd_scan *scan, double R2, int i0, int i1, int banded, const Age &age) {
+    const int half = (i1 - i0) / 2;
     if (half < 1 || banded <= i0) return false;
     auto w1 = [&](int i) { return 2.0 * scan->s + 4.0 * scan->kappa * age(i); };
     const double c = 4.0 * scan->kappa, w_half = w1(i0 + half - 1) - c * scan->tau_max;
     if (!(R2 < 16.0 * w_half)) return false;         // (e^-16 is below the bound)
     const double S = std::log(w1(i0) / (w1(banded - 1) - c * scan->tau_max));
+    const double dead = (double)ddk::kGqPieceK * (longest_step(scan) - scan->tau_max) / age(banded - 1);
     const double least = half * std::log1p(c * scan->tau_min / w1(i0)) * std::exp(-R2 / w_half);
-    return least >= 9.0 * 0x1p-26 * (S + 1.0);
+    return least >= 0x1p-21 * (S + 1.0) * (1.0 + dead);
 }
 
 // The snapshot's first visit past each band.
@@ -260,7 +273,8 @@ void GridEngine::add_span(const dd_scan *scan, const float4 *srcF, int grid, int
     j.out_off = out_off;
     j.pref = scan->pref;
     t->jobs.push_back(j);
-    const bool fp16 = kc > std::max(tb.n_fp16, i0) && fp16_everywhere(scan, t->tab_R2[table], i0, tb.n_vis, kc, [&](int i) {
+    // (a segment's field holds the younger segments, too)
+    const bool fp16 = kc > std::max(tb.n_fp16, i0) && fp16_everywhere(scan, t->tab_R2[table], i0, out_off < 0 ? tb.n_vis : i1, kc, [&](int i) {
         return tb.T ? tb.tdim - scan->T[(size_t)i] : (double)(tb.n_vis - i);
     });
     const int mid = fp16 ? kc : std::min(std::max(tb.n_fp16, i0), kc);
